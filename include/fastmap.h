@@ -230,7 +230,7 @@ int fm_map_noise_expected(const void *g1, const void *g2, void *var_out, int n, 
  * results as fm_ks_invert, FM_F32 only (cfg NULL or a valid config with
  * precision FM_F32), n a power of two in [32, 2048], batch * n^2 <= 4194304
  * (so a batch of one 2048^2 map, four of 1024^2, ...).  The FFT work buffer
- * and twiddle tables are file-scope device arrays (32 MiB + 32 KiB per
+ * and twiddle tables are file-scope device arrays (32 MiB + 63 KiB per
  * device); this entry point calls no cudaMalloc, cudaFree or other
  * allocating routine.  The driver allocates the arrays when it loads their
  * module on a device: with CUDA's default lazy module loading that is the

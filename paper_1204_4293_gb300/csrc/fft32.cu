@@ -1,15 +1,29 @@
 // fft32.cu -- fp32 Kaiser-Squires FFT (Sec. 4.5) with register-resident
-// radix-32 sub-transforms, for n = 32 .. 8192.
+// radix-16 or radix-32 sub-transforms, for n = 32 .. 8192.
 //
-// A length-n transform (n = 2^LOGN) is split into Stockham passes: radix 32,
-// then radix 32 again while needed, then one last radix RL = n / 32^k.  Each
-// thread owns 32 elements.  The first pass reads its inputs straight from
-// global memory (x[j + r n/32], coalesced over j), the last pass writes its
-// outputs straight back (X[b + r n/RL], coalesced over b), and the passes in
-// between exchange through shared memory (one slot of padding per 32
-// elements keeps the stride-32 stores conflict free).  Small DFTs run in
-// registers with constant twiddles; inter-pass twiddles come from the FP64
-// table.
+// A length-n transform (n = 2^LOGN) is split into Stockham passes: radix E
+// while more than E points remain, then one last radix RL = n / E^k.  Each of
+// the TV = n / E threads of a vector owns E elements: thread j holds x[j + q
+// TV], q = 0 .. E - 1, before and X[j + q TV] after the transform, so a
+// forward transform's output is in the inverse's input order without a
+// further exchange.  The passes exchange through shared memory (one slot of
+// padding per 16 elements keeps the stride-E stores conflict free; padded
+// addresses are one base a thread plus compile-time offsets).  Small DFTs run
+// in registers with constant twiddles; inter-pass twiddles come from
+// FP64-computed tables laid out in the order in which a warp reads them
+// (fft32_tables.cuh), one or two cache lines per load.
+//
+// What bounds these kernels is latency and instruction issue, not bytes
+// (ncu, 4 maps of 1024^2 from L2: issue slots 36-42 % busy, L2 under 25 %).
+// Against natural-order twiddle tables (gathered from up to 32 lines a load)
+// and per-access padding arithmetic, one 8192^2 map: row pass 361 -> 213 us,
+// real-output column pass 866 -> 622, complex-to-real rows 152 -> 108; 8 maps
+// of 2048^2 with kappa_B 401 -> 357 us; 32 maps of 1024^2 through the
+// pipeline 575 -> 562 us.  E = 32 needs 128 registers (16 warps an SM) but
+// fewer passes than E = 16 (64 registers, 32 warps) from n = 512 up; there
+// the passes decide: E = 16 / 32, KS alone, 32 x 1024^2 294 / 259 us, 4 x
+// 4096^2 805 / 737, 1 x 8192^2 1070 / 930.  At n <= 256 both take two passes
+// and the warps decide: 128 x 256^2 64 / 79 us.
 //
 //   rows_fwd32 : (gamma1 + i gamma2) [rotated for noise maps] -> row FFT
 //   cols_ks32  : column FFT -> x conj(D) (or D, or a given spectrum) ->
@@ -41,44 +55,35 @@
 //                       inverse FFT (even samples real part, odd imaginary).
 #include "common.cuh"
 #include "dft.cuh"
+#include "fft32_tables.cuh"
 #include "rng.cuh"
 #include "tma.cuh"
 
 namespace fm {
 
-__device__ __forceinline__ int pad32(int a) { return a + (a >> 5); }
+__device__ __forceinline__ int pad16(int a) { return a + (a >> 4); }
 
 // threads of a row-pass CTA (RPC rows of TV threads; one row when TV is
-// larger): 128-thread CTAs overlap better with the other chunk stream's
-// kernels than 256-thread ones (KS + starlet, 256 -> 128: 32 x 1024^2
-// 0.813 -> 0.805 ms, 16 x 2048^2 2.025 -> 1.988, 16 x 4096^2 10.95 -> 10.83,
-// noise R = 1000 at 1024^2 31.1 -> 30.7)
+// larger)
 constexpr int kRowThreads = 128;
 
-template <int LOGN> struct Plan32 {
-    static constexpr int N = 1 << LOGN;
-    static constexpr int TV = N / 32;                     // threads per vector
-    static constexpr int NPASS = (LOGN + 4) / 5;          // passes (all radix 32 but the last)
-    static constexpr int LOGRL = LOGN - 5 * (NPASS - 1);  // log2 of the last radix
-    static constexpr int RL = 1 << LOGRL;
-    static constexpr int ML = 32 / RL;                    // butterflies per thread in the last pass
-    static constexpr int NSL = N / RL;                    // stride of the last pass outputs
+template <int LOGN> struct Plan32 : FftPlan<LOGN> {
+    using B = FftPlan<LOGN>;
+    static constexpr int N = B::N, TV = B::TV;
+    // rows of a row-pass CTA, its threads, and the CTAs per SM that its
+    // registers allow
+    static constexpr int RPC = TV >= kRowThreads ? 1 : kRowThreads / TV;
+    static constexpr int ROW_T = RPC * TV;
+    static constexpr int THREADS = 16384 / B::E;  // threads of an SM: 1024 (64 registers) with 16 elements each, 512 (128) with 32
+    static constexpr int ROW_MINB = THREADS / ROW_T < 1 ? 1 : (THREADS / ROW_T > 24 ? 24 : THREADS / ROW_T);
+    static constexpr int VS = N + N / 16;  // exchange buffer of one vector (elements)
     // column strip width: 64 B row segments at n = 1024, 32 B at 2048 and
-    // 4096 (one full sector; 512 threads, 136 KB of shared memory at 4096:
-    // 13 % faster than 16 B strips), 16 B at 8192
+    // 4096 (one full sector), 16 B at 8192
     static constexpr int W = N <= 512 ? 16 : (N >= 8192 ? 2 : (N == 4096 ? 4 : 8192 / N));
+    static constexpr int COL_T = W * TV;
+    static constexpr int COL_MINB = THREADS / COL_T < 1 ? 1 : (THREADS / COL_T > 24 ? 24 : THREADS / COL_T);
 };
 
-template <bool INV> __device__ __forceinline__ float2 twid(const float2 *__restrict__ tw, int t)
-{
-    float2 w = __ldg(tw + t);
-    if (INV) w.y = -w.y;
-    return w;
-}
-
-// In: v[r] = x[j + r TV].  Out: v[m RL + r] = X[j + m TV + r NSL].
-// Element i of the vector lives at sm[pad32(i W + c)] between passes.
-// Every thread of the CTA must call this (it holds barriers).
 // barrier of the threads taking part: the whole CTA (NB = 0) or the first NB
 // threads (named barrier 1; NB a multiple of 32)
 template <int NB> __device__ __forceinline__ void part_sync()
@@ -89,45 +94,81 @@ template <int NB> __device__ __forceinline__ void part_sync()
         asm volatile("bar.sync 1, %0;" ::"n"(NB) : "memory");
 }
 
-template <int LOGN, int W, bool INV, int NB = 0>
-__device__ __forceinline__ void fft_vec(float2 (&v)[32], float2 *sm, int c, int j, const float2 *__restrict__ tw)
+// times the table's twiddle (its conjugate for the inverse)
+template <bool INV> __device__ __forceinline__ float2 mul_tw(float2 a, const float2 *__restrict__ tw)
 {
-    using P = Plan32<LOGN>;
-    Dft<32, INV, float2>::run(v);  // pass 1: Ns = 1, no twiddles; outputs at 32 j + r
-    if constexpr (P::NPASS > 1) {
-        part_sync<NB>();  // the buffer may still be read by an earlier pass
+    float2 w = __ldg(tw);
+    if (INV) w.y = -w.y;
+    return cmul(a, w);
+}
+
+// In: v[q] = x[j + q TV].  Out: v[q] = X[j + q TV].
+// Element i of vector c (of W) lives at sm[pad16(i W + c)] between passes.
+// tw: the pass tables of length N (FftPlan's layout, after the natural table).
+// Every thread taking part must call this (it holds barriers).
+template <int LOGN, int W, bool INV, int NB = 0>
+__device__ __forceinline__ void fft_vec(float2 (&v)[FftPlan<LOGN>::E], float2 *sm, int c, int j,
+                                        const float2 *__restrict__ tw)
+{
+    using P = FftPlan<LOGN>;
+    constexpr int E = P::E;
+    // Padded addresses split into one base a thread and compile-time offsets
+    // (immediates of the loads and stores): exact as long as 16 divides the
+    // strides, i.e. TV W >= 16; smaller vectors take the formula itself.
+    constexpr bool LIN = P::TV * W >= 16;
+    constexpr int TVS = P::TV * W + P::TV * W / 16;  // padded stride of TV elements
+    float2 *rd = sm + pad16(j * W + c);              // x[j], then + q TVS
+    auto load = [&](int q) { return LIN ? rd[q * TVS] : sm[pad16((j + q * P::TV) * W + c)]; };
+    Dft<E, INV, float2>::run(v);  // pass 0: Ns = 1, no twiddles; outputs at E j + r
+    part_sync<NB>();              // the buffer may still be read by an earlier pass
+    {
+        static_assert(W <= 16 && (E * W) % 16 == 0, "padding");
+        float2 *wr = sm + j * (E * W + E * W / 16) + c;
 #pragma unroll
-        for (int r = 0; r < 32; ++r) sm[pad32((j * 32 + r) * W + c)] = v[r];
-        part_sync<NB>();
-        if constexpr (P::NPASS > 2) {
-            // pass 2: radix 32, Ns = 32
-            constexpr int NS = 32;
-#pragma unroll
-            for (int r = 0; r < 32; ++r) v[r] = sm[pad32((j + r * P::TV) * W + c)];
-            const int k = j & (NS - 1);
-            const int step = k * (P::N / (NS * 32));
-#pragma unroll
-            for (int r = 1; r < 32; ++r) v[r] = cmul(v[r], twid<INV>(tw, r * step));
-            Dft<32, INV, float2>::run(v);
-            part_sync<NB>();
-            const int o = (j - k) * 32 + k;
-#pragma unroll
-            for (int r = 0; r < 32; ++r) sm[pad32((o + r * NS) * W + c)] = v[r];
-            part_sync<NB>();
-        }
-        // last pass: radix RL, Ns = NSL, butterfly b = j + m TV (< NSL), twiddle W_n^(r b)
-#pragma unroll
-        for (int m = 0; m < P::ML; ++m) {
-            const int b = j + m * P::TV;
-#pragma unroll
-            for (int r = 0; r < P::RL; ++r) {
-                float2 x = sm[pad32((b + r * P::NSL) * W + c)];
-                if (r > 0) x = cmul(x, twid<INV>(tw, r * b));
-                v[m * P::RL + r] = x;
-            }
-            Dft<P::RL, INV, float2>::run(v + m * P::RL);
-        }
+        for (int r = 0; r < E; ++r) wr[r * W + ((r * W) >> 4)] = v[r];
     }
+    part_sync<NB>();
+    // middle passes: radix E, Ns = E, E^2
+#pragma unroll
+    for (int p = 1; p + 1 < P::NPASS; ++p) {
+        const int NS = 1 << (P::LOGE * p);
+#pragma unroll
+        for (int r = 0; r < E; ++r) v[r] = load(r);
+        const int k = j & (NS - 1);
+        const float2 *t = tw + P::N + P::pass_off(p) + k;
+#pragma unroll
+        for (int r = 1; r < E; ++r) v[r] = mul_tw<INV>(v[r], t + (r - 1) * NS);
+        Dft<E, INV, float2>::run(v);
+        part_sync<NB>();
+        float2 *wr = sm + pad16(((j - k) * E + k) * W + c);
+#pragma unroll
+        for (int r = 0; r < E; ++r) wr[r * (NS * W + NS * W / 16)] = v[r];
+        part_sync<NB>();
+    }
+    // last pass: radix RL, Ns = NSL, butterfly b = j + m TV (< NSL), twiddle W_n^(r b)
+    const float2 *t = tw + P::N + P::pass_off(P::NPASS - 1) + j;
+#pragma unroll
+    for (int m = 0; m < P::ML; ++m) {
+        float2 x[P::RL];
+#pragma unroll
+        for (int r = 0; r < P::RL; ++r) {
+            x[r] = load(m + r * P::ML);
+            if (r > 0) x[r] = mul_tw<INV>(x[r], t + (r - 1) * P::NSL + m * P::TV);
+        }
+        Dft<P::RL, INV, float2>::run(x);
+        // output r of butterfly m is X[j + TV (m + r ML)]
+#pragma unroll
+        for (int r = 0; r < P::RL; ++r) v[m + r * P::ML] = x[r];
+    }
+}
+
+// signed integer frequency of index j + q TV as a float (q a compile-time
+// constant: no select); exact, and so are the squares and products below
+// 2^24 that the KS multiplier takes of it
+template <int LOGN> __device__ __forceinline__ float freq_of(float jf, int q)
+{
+    using P = FftPlan<LOGN>;
+    return jf + (float)(q * P::TV - (q >= P::E / 2 ? P::N : 0));
 }
 
 // With use_tma (n >= 64; in_bs = n^2, or in_bs = 0 with RPC <= n), the CTA's
@@ -137,7 +178,8 @@ __device__ __forceinline__ void fft_vec(float2 (&v)[32], float2 *sm, int c, int 
 // ROT: the noise maps' rotated shear (a separate instantiation, so that the
 // plain transform carries none of the generator's code)
 template <int LOGN, bool SPLIT, bool ROT>
-__global__ void __launch_bounds__(256, 2) k_rows_fwd32(const float *__restrict__ in1, const float *__restrict__ in2,
+__global__ void __launch_bounds__(Plan32<LOGN>::ROW_T, Plan32<LOGN>::ROW_MINB)
+    k_rows_fwd32(const float *__restrict__ in1, const float *__restrict__ in2,
                                                        long in_bs, float2 *__restrict__ work, long total_rows,
                                                        const float2 *__restrict__ tw, uint64_t seed, int r0,
                                                        const __grid_constant__ CUtensorMap m1,
@@ -145,17 +187,17 @@ __global__ void __launch_bounds__(256, 2) k_rows_fwd32(const float *__restrict__
 {
     pdl_entry();
     using P = Plan32<LOGN>;
-    constexpr int RPC = P::TV >= kRowThreads ? 1 : kRowThreads / P::TV;
+    constexpr int RPC = P::RPC;
     extern __shared__ __align__(16) float2 sm32[];
     __shared__ uint64_t bar;
     float2 *smb = align128<float2>(sm32);
     const int vr = threadIdx.x / P::TV, j = threadIdx.x % P::TV;
     const long row = (long)blockIdx.x * RPC + vr;
-    float2 *sm = smb + vr * (P::N + P::N / 32);
+    float2 *sm = smb + vr * P::VS;
     const bool live = row < total_rows;
-    float2 v[32];
+    float2 v[P::E];
     bool staged = false;
-    if constexpr (P::NPASS > 1) {
+    if constexpr (P::N >= 64) {
         if (use_tma) {
             float *st1 = reinterpret_cast<float *>(smb), *st2 = st1 + RPC * P::N;
             if (threadIdx.x == 0) mbar_init(&bar, 1);
@@ -171,7 +213,7 @@ __global__ void __launch_bounds__(256, 2) k_rows_fwd32(const float *__restrict__
             const long b = row >> LOGN;
             const int y = (int)(row & (P::N - 1));
 #pragma unroll
-            for (int r = 0; r < 32; ++r) {
+            for (int r = 0; r < P::E; ++r) {
                 const int x = j + r * P::TV;
                 float a = st1[vr * P::N + x];
                 float cc = in2 ? st2[vr * P::N + x] : 0.f;
@@ -187,7 +229,7 @@ __global__ void __launch_bounds__(256, 2) k_rows_fwd32(const float *__restrict__
         const float *p1 = in1 + b * in_bs + (long)y * P::N;
         const float *p2 = in2 ? in2 + b * in_bs + (long)y * P::N : nullptr;
 #pragma unroll
-        for (int r = 0; r < 32; ++r) {
+        for (int r = 0; r < P::E; ++r) {
             const int x = j + r * P::TV;
             float a = __ldcs(p1 + x);  // the shear is read once
             float cc = p2 ? __ldcs(p2 + x) : 0.f;
@@ -196,29 +238,27 @@ __global__ void __launch_bounds__(256, 2) k_rows_fwd32(const float *__restrict__
         }
     } else if (!staged) {
 #pragma unroll
-        for (int r = 0; r < 32; ++r) v[r] = make_float2(0.f, 0.f);
+        for (int r = 0; r < P::E; ++r) v[r] = make_float2(0.f, 0.f);
     }
     fft_vec<LOGN, 1, false>(v, sm, 0, j, tw);
-    if constexpr (SPLIT && P::NPASS > 1) {
+    if constexpr (SPLIT) {
         // Z through the exchange buffer so that Z(kx) and Z(n - kx) meet
         __syncthreads();  // the last pass's reads of the buffer
 #pragma unroll
-        for (int m = 0; m < P::ML; ++m)
-#pragma unroll
-            for (int r = 0; r < P::RL; ++r) sm[pad32(j + m * P::TV + r * P::NSL)] = v[m * P::RL + r];
+        for (int q = 0; q < P::E; ++q) sm[pad16(j + q * P::TV)] = v[q];
         __syncthreads();
         if (live) {
             // slot kx of the row: (Gamma1(kx), Gamma2(kx)) as one 16-byte element
             float4 *d = reinterpret_cast<float4 *>(work + row * P::N);
 #pragma unroll
-            for (int t = 0; t < 16; ++t) {
+            for (int t = 0; t < P::E / 2; ++t) {
                 const int kx = j + t * P::TV;
-                const float2 a = sm[pad32(kx)];
+                const float2 a = sm[pad16(kx)];
                 if (kx == 0) {
-                    const float2 h = sm[pad32(P::N / 2)];
+                    const float2 h = sm[pad16(P::N / 2)];
                     d[0] = make_float4(a.x, h.x, a.y, h.y);
                 } else {
-                    const float2 bm = sm[pad32(P::N - kx)];  // Z(n - kx); B = conj of it
+                    const float2 bm = sm[pad16(P::N - kx)];  // Z(n - kx); B = conj of it
                     d[kx] = make_float4(0.5f * (a.x + bm.x), 0.5f * (a.y - bm.y), 0.5f * (a.y + bm.y),
                                         -0.5f * (a.x - bm.x));
                 }
@@ -229,9 +269,7 @@ __global__ void __launch_bounds__(256, 2) k_rows_fwd32(const float *__restrict__
     if (live) {
         float2 *dst = work + row * P::N;
 #pragma unroll
-        for (int m = 0; m < P::ML; ++m)
-#pragma unroll
-            for (int r = 0; r < P::RL; ++r) dst[j + m * P::TV + r * P::NSL] = v[m * P::RL + r];
+        for (int q = 0; q < P::E; ++q) dst[j + q * P::TV] = v[q];
     }
 }
 
@@ -241,24 +279,25 @@ __global__ void __launch_bounds__(256, 2) k_rows_fwd32(const float *__restrict__
 // WITH_B: kappa_B (the imaginary part) written too, a separate instantiation
 // so that the kappa_E-only store loop has no per-element branch
 template <int LOGN, bool WITH_B>
-__global__ void __launch_bounds__(256, 2) k_rows_inv32(const float2 *__restrict__ work, float *__restrict__ out1,
+__global__ void __launch_bounds__(Plan32<LOGN>::ROW_T, Plan32<LOGN>::ROW_MINB)
+    k_rows_inv32(const float2 *__restrict__ work, float *__restrict__ out1,
                                                        float *__restrict__ out2, long total_rows,
                                                        const float2 *__restrict__ tw, float scale,
                                                        const __grid_constant__ CUtensorMap mw, int use_tma)
 {
     pdl_entry();
     using P = Plan32<LOGN>;
-    constexpr int RPC = P::TV >= kRowThreads ? 1 : kRowThreads / P::TV;
+    constexpr int RPC = P::RPC;
     extern __shared__ __align__(16) float2 sm32[];
     __shared__ uint64_t bar;
     float2 *smb = align128<float2>(sm32);
     const int vr = threadIdx.x / P::TV, j = threadIdx.x % P::TV;
     const long row = (long)blockIdx.x * RPC + vr;
-    float2 *sm = smb + vr * (P::N + P::N / 32);
+    float2 *sm = smb + vr * P::VS;
     const bool live = row < total_rows;
-    float2 v[32];
+    float2 v[P::E];
     bool staged = false;
-    if constexpr (P::NPASS > 1) {
+    if constexpr (P::N >= 64) {
         if (use_tma) {
             if (threadIdx.x == 0) mbar_init(&bar, 1);
             __syncthreads();
@@ -268,23 +307,21 @@ __global__ void __launch_bounds__(256, 2) k_rows_inv32(const float2 *__restrict_
             }
             if (!tma_wait_all(&bar, 0)) return;  // the copy never completed (flagged)
 #pragma unroll
-            for (int r = 0; r < 32; ++r) v[r] = smb[vr * P::N + j + r * P::TV];
+            for (int r = 0; r < P::E; ++r) v[r] = smb[vr * P::N + j + r * P::TV];
             staged = true;  // fft_vec's first barrier orders these reads before the exchange writes
         }
     }
     if (!staged) {
         const float2 *src = work + row * P::N;
 #pragma unroll
-        for (int r = 0; r < 32; ++r) v[r] = live ? src[j + r * P::TV] : make_float2(0.f, 0.f);
+        for (int r = 0; r < P::E; ++r) v[r] = live ? src[j + r * P::TV] : make_float2(0.f, 0.f);
     }
     fft_vec<LOGN, 1, true>(v, sm, 0, j, tw);
     if (live) {
 #pragma unroll
-        for (int m = 0; m < P::ML; ++m)
-#pragma unroll
-            for (int r = 0; r < P::RL; ++r) {
-                const long pos = row * P::N + j + m * P::TV + r * P::NSL;
-                const float2 x = v[m * P::RL + r];
+        for (int q = 0; q < P::E; ++q) {
+                const long pos = row * P::N + j + q * P::TV;
+                const float2 x = v[q];
                 out1[pos] = x.x * scale;
                 if constexpr (WITH_B) out2[pos] = x.y * scale;
             }
@@ -294,12 +331,13 @@ __global__ void __launch_bounds__(256, 2) k_rows_inv32(const float2 *__restrict_
 // With use_tma bit 0 (mw: the work buffer as floats {2n, n, batch}, box
 // {2W, min(n, 256), 1}), the CTA's strip of W columns arrives by
 // n / min(n, 256) bulk tensor copies into the exchange buffer, densely as
-// [n][W] float2, instead of 32 strided loads per thread; with bit 1 the
+// [n][W] float2, instead of E strided loads per thread; with bit 1 the
 // result leaves the same way (the spectrum-only mode stores per thread).
 // KSINV: the inverse KS multiply fixed at compile time (the pipeline's
 // instantiation, no per-element branch on op); else op chooses at run time.
 template <int LOGN, bool KSINV>
-__global__ void __launch_bounds__(512) k_cols_ks32(float2 *__restrict__ work, const float2 *__restrict__ tw,
+__global__ void __launch_bounds__(Plan32<LOGN>::COL_T, Plan32<LOGN>::COL_MINB)
+    k_cols_ks32(float2 *__restrict__ work, const float2 *__restrict__ tw,
                                                    int op_arg, const float2 *__restrict__ filt,
                                                    const __grid_constant__ CUtensorMap mw, int use_tma)
 {
@@ -314,7 +352,7 @@ __global__ void __launch_bounds__(512) k_cols_ks32(float2 *__restrict__ work, co
     const int x0 = (blockIdx.x % STRIPS) * W;
     const int c = threadIdx.x % W, j = threadIdx.x / W;
     float2 *base = work + b * (long)N * N + x0 + c;
-    float2 v[32];
+    float2 v[P::E];
     if (use_tma & 1) {
         __shared__ uint64_t bar;
         constexpr int BR = N < 256 ? N : 256;  // rows per copy
@@ -326,57 +364,41 @@ __global__ void __launch_bounds__(512) k_cols_ks32(float2 *__restrict__ work, co
         }
         if (!tma_wait_all(&bar, 0)) return;  // the copies never completed (flagged)
 #pragma unroll
-        for (int r = 0; r < 32; ++r) v[r] = sm32[(j + r * P::TV) * W + c];
+        for (int r = 0; r < P::E; ++r) v[r] = sm32[(j + r * P::TV) * W + c];
     } else {
 #pragma unroll
-        for (int r = 0; r < 32; ++r) v[r] = base[(long)(j + r * P::TV) * N];
+        for (int r = 0; r < P::E; ++r) v[r] = base[(long)(j + r * P::TV) * N];
     }
     fft_vec<LOGN, W, false>(v, sm32, c, j, tw);
     if (op == FFT_OP_SPECTRUM) {  // the 2-D spectrum [ky][kx] is the result
 #pragma unroll
-        for (int m = 0; m < P::ML; ++m)
-#pragma unroll
-            for (int r = 0; r < P::RL; ++r) base[(long)(j + m * P::TV + r * P::NSL) * N] = v[m * P::RL + r];
+        for (int q = 0; q < P::E; ++q) base[(long)(j + q * P::TV) * N] = v[q];
         return;
     }
     // kappa_hat = conj(D) gamma_hat (inverse KS) or D kappa_hat (forward KS),
     // D = (k1^2 - k2^2 + 2 i k1 k2) / (k1^2 + k2^2), D(0) = 0; or the given
     // spectrum filt[b][ky][kx]
     const int xi = x0 + c;
-    const int k1 = xi < N / 2 ? xi : xi - N;
+    const float k1 = (float)(xi < N / 2 ? xi : xi - N), jf = (float)j;
     const float2 *fb = filt ? filt + b * (long)N * N + xi : nullptr;
 #pragma unroll
-    for (int m = 0; m < P::ML; ++m)
-#pragma unroll
-        for (int r = 0; r < P::RL; ++r) {
-            const int yi = j + m * P::TV + r * P::NSL;
-            float2 d;
-            if (op == FFT_OP_FILTER) {
-                d = fb[(long)yi * N];
-            } else {
-                const int k2 = yi < N / 2 ? yi : yi - N;
-                const int den = k1 * k1 + k2 * k2;
-                d = make_float2(0.f, 0.f);
-                if (den != 0) {
-                    // the pipeline's instantiation: the fast reciprocal (2 ulp, no
-                    // division subroutine in the unrolled loop)
-                    const float inv = KSINV ? __fdividef(1.f, (float)den) : 1.f / (float)den;
-                    const float im = (float)(2 * k1 * k2) * inv;
-                    d = make_float2((float)(k1 * k1 - k2 * k2) * inv, op == FFT_OP_KS_FWD ? im : -im);
-                }
+    for (int q = 0; q < P::E; ++q) {
+        float2 d;
+        if (op == FFT_OP_FILTER) {
+            d = fb[(long)(j + q * P::TV) * N];
+        } else {
+            const float k2 = freq_of<LOGN>(jf, q);
+            const float den = k1 * k1 + k2 * k2;
+            d = make_float2(0.f, 0.f);
+            if (den != 0.f) {
+                // the pipeline's instantiation: the fast reciprocal (2 ulp, no
+                // division subroutine in the unrolled loop)
+                const float inv = KSINV ? __fdividef(1.f, den) : 1.f / den;
+                const float im = 2.f * k1 * k2 * inv;
+                d = make_float2((k1 * k1 - k2 * k2) * inv, op == FFT_OP_KS_FWD ? im : -im);
             }
-            v[m * P::RL + r] = cmul(v[m * P::RL + r], d);
         }
-    if constexpr (!(P::RL == 32 || P::NPASS == 1)) {
-        // bring the spectrum back to the inverse's input order x[j + r TV]
-        __syncthreads();
-#pragma unroll
-        for (int m = 0; m < P::ML; ++m)
-#pragma unroll
-            for (int r = 0; r < P::RL; ++r) sm32[pad32((j + m * P::TV + r * P::NSL) * W + c)] = v[m * P::RL + r];
-        __syncthreads();
-#pragma unroll
-        for (int r = 0; r < 32; ++r) v[r] = sm32[pad32((j + r * P::TV) * W + c)];
+        v[q] = cmul(v[q], d);
     }
     fft_vec<LOGN, W, true>(v, sm32, c, j, tw);
     if (use_tma & 2) {
@@ -385,9 +407,7 @@ __global__ void __launch_bounds__(512) k_cols_ks32(float2 *__restrict__ work, co
         constexpr int BR = N < 256 ? N : 256;
         __syncthreads();  // the last pass may still read the exchange buffer
 #pragma unroll
-        for (int m = 0; m < P::ML; ++m)
-#pragma unroll
-            for (int r = 0; r < P::RL; ++r) sm32[(j + m * P::TV + r * P::NSL) * W + c] = v[m * P::RL + r];
+        for (int q = 0; q < P::E; ++q) sm32[(j + q * P::TV) * W + c] = v[q];
         fence_async_smem();
         __syncthreads();
         if (threadIdx.x == 0) {
@@ -398,14 +418,12 @@ __global__ void __launch_bounds__(512) k_cols_ks32(float2 *__restrict__ work, co
         return;
     }
 #pragma unroll
-    for (int m = 0; m < P::ML; ++m)
-#pragma unroll
-        for (int r = 0; r < P::RL; ++r) base[(long)(j + m * P::TV + r * P::NSL) * N] = v[m * P::RL + r];
+    for (int q = 0; q < P::E; ++q) base[(long)(j + q * P::TV) * N] = v[q];
 }
 
 // ---- real-output inverse: column and row kernels ------------------------------
 // Slots per column strip (WS; a strip is WS 16-byte (Gamma1, Gamma2) pairs
-// per row, one bulk tensor copy box wide).  A CTA of 2 WS n/32 threads: its
+// per row, one bulk tensor copy box wide).  A CTA of 2 WS n/E threads: its
 // first half transforms the strip's Gamma1 columns, the second half the
 // Gamma2 columns, at the same time; the second half hands its spectra over
 // through shared memory and leaves, and the first half forms kappa_E_hat and
@@ -416,17 +434,17 @@ __global__ void __launch_bounds__(512) k_cols_ks32(float2 *__restrict__ work, co
 template <int LOGN> struct PlanE {
     static constexpr int N = 1 << LOGN;
     static constexpr int WS = N <= 256 ? 16 : (N == 512 ? 8 : (N == 1024 ? 4 : (N <= 4096 ? 2 : 1)));
-    static constexpr int RSZ = (N * WS + N * WS / 32 + 1 + 15) & ~15;  // float2 per region, 128-byte multiple
+    static constexpr int RSZ = (N * WS + N * WS / 16 + 1 + 15) & ~15;  // float2 per region, 128-byte multiple
     // the corner strip's dense exchange (2n elements): with WS >= 2 both
     // halves go to the Gamma1 region after its transform (the Gamma2 region
     // carries the other slots' hand-over); with WS = 1 the strip is the
     // corner slot alone and the second half writes its half in row order to
     // its own region
     static_assert(WS == 1 || RSZ >= 2 * N, "corner exchange");
-    static constexpr int NH = WS * N / 32;  // threads of one half
+    static constexpr int NH = WS * FftPlan<LOGN>::TV;  // threads of one half
     static constexpr int NT = 2 * NH;
-    // CTAs per SM the register budget must allow: at most 128 registers a thread
-    static constexpr int MINB = 65536 / (NT * 128) < 1 ? 1 : (65536 / (NT * 128) > 8 ? 8 : 65536 / (NT * 128));
+    // CTAs per SM the register budget must allow
+    static constexpr int MINB = Plan32<LOGN>::THREADS / NT < 1 ? 1 : Plan32<LOGN>::THREADS / NT;
 };
 
 // With use_tma (mw: the work buffer as floats {2n, n, batch}, box {4 WS,
@@ -450,7 +468,7 @@ __global__ void __launch_bounds__(PlanE<LOGN>::NT, PlanE<LOGN>::MINB)
     const int s0 = (blockIdx.x % STRIPS) * WS;
     const int tid = threadIdx.x, hf = tid / NH, t = tid % NH, c = t % WS, j = t / WS;
     float2 *R = hf ? R2 : R1;  // this half's strip and exchange region
-    float2 v[32];
+    float2 v[P::E];
     if (use_tma) {
         __shared__ uint64_t bar;
         constexpr int BR = N < 256 ? N : 256;  // rows per copy
@@ -465,98 +483,76 @@ __global__ void __launch_bounds__(PlanE<LOGN>::NT, PlanE<LOGN>::MINB)
         // fft_vec's first barrier orders every thread's reads of the strip
         // before the exchange writes that overlay it
 #pragma unroll
-        for (int r = 0; r < 32; ++r) v[r] = R1[((j + r * P::TV) * WS + c) * 2 + hf];
+        for (int r = 0; r < P::E; ++r) v[r] = R1[((j + r * P::TV) * WS + c) * 2 + hf];
     } else {
         // rows of n/2 slots (Gamma1, Gamma2)
         const float2 *src = work + b * (long)N * N + 2 * (s0 + c) + hf;
 #pragma unroll
-        for (int r = 0; r < 32; ++r) v[r] = src[(long)(j + r * P::TV) * N];
+        for (int r = 0; r < P::E; ++r) v[r] = src[(long)(j + r * P::TV) * N];
     }
     fft_vec<LOGN, WS, false>(v, R, c, j, tw);  // Gamma1_hat (first half), Gamma2_hat (second)
     __syncthreads();                           // the last passes' reads of R1 and R2 are done
     if (hf) {
         if (WS == 1 && s0 == 0) {  // the corner slot: in row order
 #pragma unroll
-            for (int m = 0; m < P::ML; ++m)
-#pragma unroll
-                for (int r = 0; r < P::RL; ++r) U2[j + m * P::TV + r * P::NSL] = v[m * P::RL + r];
+            for (int q = 0; q < P::E; ++q) U2[j + q * P::TV] = v[q];
         } else {
 #pragma unroll
-            for (int e = 0; e < 32; ++e) R2[e * NH + t] = v[e];  // for the thread t of the first half
+            for (int e = 0; e < P::E; ++e) R2[e * NH + t] = v[e];  // for the thread t of the first half
         }
     }
     __syncthreads();
     if (hf) return;  // the rest runs on named barrier 1 of the first NH threads
+    const float jf = (float)j;
     const bool corner = s0 == 0 && c == 0;  // slot 0: kx = 0 and kx = n/2 packed
     if (!corner) {
-        const int k1 = s0 + c;  // 1 .. n/2 - 1
+        const float k1 = (float)(s0 + c);  // 1 .. n/2 - 1
 #pragma unroll
-        for (int m = 0; m < P::ML; ++m)
-#pragma unroll
-            for (int r = 0; r < P::RL; ++r) {
-                const int e = m * P::RL + r, yi = j + m * P::TV + r * P::NSL;
-                const int k2 = yi < N / 2 ? yi : yi - N;
-                const float inv = __fdividef(1.f, (float)(k1 * k1 + k2 * k2));  // 2 ulp
-                const float dr = (float)(k1 * k1 - k2 * k2) * inv, di = (float)(2 * k1 * k2) * inv;
-                const float2 a = v[e], g = R2[e * NH + t];
-                v[e] = yi == N / 2 ? make_float2(dr * a.x + di * a.y, dr * a.y - di * a.x)  // conj(D) Gamma1
-                                   : make_float2(dr * a.x + di * g.x, dr * a.y + di * g.y);
-            }
+        for (int q = 0; q < P::E; ++q) {
+            const float k2 = freq_of<LOGN>(jf, q);
+            const float inv = __fdividef(1.f, k1 * k1 + k2 * k2);  // 2 ulp
+            const float dr = (k1 * k1 - k2 * k2) * inv, di = 2.f * k1 * k2 * inv;
+            const float2 a = v[q], g = R2[q * NH + t];
+            v[q] = q == P::E / 2 && j == 0 ? make_float2(dr * a.x + di * a.y, dr * a.y - di * a.x)  // ky = n/2: conj(D) Gamma1
+                                    : make_float2(dr * a.x + di * g.x, dr * a.y + di * g.y);
+        }
     }
     if (s0 == 0) {  // CTA-uniform: the corner column pair needs ky and -ky together
         if (c == 0) {
 #pragma unroll
-            for (int m = 0; m < P::ML; ++m)
-#pragma unroll
-                for (int r = 0; r < P::RL; ++r) {
-                    const int e = m * P::RL + r, yi = j + m * P::TV + r * P::NSL;
-                    U1[yi] = v[e];
-                    if (WS > 1) U2[yi] = R2[e * NH + t];
-                }
+            for (int q = 0; q < P::E; ++q) {
+                const int yi = j + q * P::TV;
+                U1[yi] = v[q];
+                if (WS > 1) U2[yi] = R2[q * NH + t];
+            }
         }
         part_sync<NH>();
         if (c == 0) {
 #pragma unroll
-            for (int m = 0; m < P::ML; ++m)
-#pragma unroll
-                for (int r = 0; r < P::RL; ++r) {
-                    const int e = m * P::RL + r, yi = j + m * P::TV + r * P::NSL;
-                    const int yp = (N - yi) & (N - 1);
-                    const float2 p1 = U1[yi], q1 = U1[yp], p2 = U2[yi], q2 = U2[yp];
-                    // A = Gamma(ky, 0) = (P + conj P(-ky)) / 2, B = Gamma(ky, n/2) = (P - conj P(-ky)) / 2i
-                    const float2 a1 = make_float2(0.5f * (p1.x + q1.x), 0.5f * (p1.y - q1.y));
-                    const float2 b1 = make_float2(0.5f * (p1.y + q1.y), -0.5f * (p1.x - q1.x));
-                    const float2 b2 = make_float2(0.5f * (p2.y + q2.y), -0.5f * (p2.x - q2.x));
-                    const int k2 = yi < N / 2 ? yi : yi - N;
-                    // kx = 0: D = -1 (0 at k = 0)
-                    const float2 kz = yi == 0 ? make_float2(0.f, 0.f) : make_float2(-a1.x, -a1.y);
-                    // kx = n/2 (k1 = -n/2)
-                    const float inv = __fdividef(1.f, (float)(N / 2 * (N / 2) + k2 * k2));
-                    const float dr = (float)(N / 2 * (N / 2) - k2 * k2) * inv, di = (float)(-N * k2) * inv;
-                    const float2 kh = (yi == 0 || yi == N / 2)
-                                          ? make_float2(dr * b1.x + di * b2.x, dr * b1.y + di * b2.y)
-                                          : make_float2(dr * b1.x + di * b1.y, dr * b1.y - di * b1.x);
-                    v[e] = make_float2(kz.x - kh.y, kz.y + kh.x);  // packed kz + i kh
-                }
+            for (int q = 0; q < P::E; ++q) {
+                const int yi = j + q * P::TV;
+                const int yp = (N - yi) & (N - 1);
+                const float2 p1 = U1[yi], q1 = U1[yp], p2 = U2[yi], q2 = U2[yp];
+                // A = Gamma(ky, 0) = (P + conj P(-ky)) / 2, B = Gamma(ky, n/2) = (P - conj P(-ky)) / 2i
+                const float2 a1 = make_float2(0.5f * (p1.x + q1.x), 0.5f * (p1.y - q1.y));
+                const float2 b1 = make_float2(0.5f * (p1.y + q1.y), -0.5f * (p1.x - q1.x));
+                const float2 b2 = make_float2(0.5f * (p2.y + q2.y), -0.5f * (p2.x - q2.x));
+                const float k2 = freq_of<LOGN>(jf, q), h = (float)(N / 2);
+                // kx = 0: D = -1 (0 at k = 0)
+                const float2 kz = yi == 0 ? make_float2(0.f, 0.f) : make_float2(-a1.x, -a1.y);
+                // kx = n/2 (k1 = -n/2)
+                const float inv = __fdividef(1.f, h * h + k2 * k2);
+                const float dr = (h * h - k2 * k2) * inv, di = -2.f * h * k2 * inv;
+                const float2 kh = (yi == 0 || yi == N / 2) ? make_float2(dr * b1.x + di * b2.x, dr * b1.y + di * b2.y)
+                                                           : make_float2(dr * b1.x + di * b1.y, dr * b1.y - di * b1.x);
+                v[q] = make_float2(kz.x - kh.y, kz.y + kh.x);  // packed kz + i kh
+            }
         }
-    }
-    if constexpr (!(P::RL == 32 || P::NPASS == 1)) {
-        // bring the spectrum back to the inverse's input order x[j + r TV]
-        part_sync<NH>();
-#pragma unroll
-        for (int m = 0; m < P::ML; ++m)
-#pragma unroll
-            for (int r = 0; r < P::RL; ++r) R1[pad32((j + m * P::TV + r * P::NSL) * WS + c)] = v[m * P::RL + r];
-        part_sync<NH>();
-#pragma unroll
-        for (int r = 0; r < 32; ++r) v[r] = R1[pad32((j + r * P::TV) * WS + c)];
     }
     fft_vec<LOGN, WS, true, NH>(v, R1, c, j, tw);
     float2 *dst = half + b * (long)N * (N / 2) + s0 + c;
 #pragma unroll
-    for (int m = 0; m < P::ML; ++m)
-#pragma unroll
-        for (int r = 0; r < P::RL; ++r) dst[(long)(j + m * P::TV + r * P::NSL) * (N / 2)] = v[m * P::RL + r];
+    for (int q = 0; q < P::E; ++q) dst[(long)(j + q * P::TV) * (N / 2)] = v[q];
 }
 
 // In place: row y of kap holds the half spectrum H(y, 0 .. n/2) as n/2 float2
@@ -565,23 +561,24 @@ __global__ void __launch_bounds__(PlanE<LOGN>::NT, PlanE<LOGN>::MINB)
 // staged by one bulk tensor copy.  Every read of the row precedes the
 // transform's first barrier, and every write follows it.
 template <int LOGN>
-__global__ void __launch_bounds__(256, 2) k_rows_inv32_c2r(float *kap, long total_rows, const float2 *__restrict__ tw,
+__global__ void __launch_bounds__(Plan32<LOGN - 1>::ROW_T, Plan32<LOGN - 1>::ROW_MINB)
+    k_rows_inv32_c2r(float *kap, long total_rows, const float2 *__restrict__ tw,
                                                            const float2 *__restrict__ tw2, float scale,
                                                            const __grid_constant__ CUtensorMap mk, int use_tma)
 {
     pdl_entry();
     using P = Plan32<LOGN - 1>;  // the length n/2 complex transform
     constexpr int N2 = P::N;
-    constexpr int RPC = P::TV >= kRowThreads ? 1 : kRowThreads / P::TV;
+    constexpr int RPC = P::RPC;
     extern __shared__ __align__(16) float2 sm32[];
     __shared__ uint64_t bar;
     float2 *smb = align128<float2>(sm32);
     const int vr = threadIdx.x / P::TV, j = threadIdx.x % P::TV;
     const long row = (long)blockIdx.x * RPC + vr;
-    float2 *sm = smb + vr * (N2 + N2 / 32);
+    float2 *sm = smb + vr * P::VS;
     const bool live = row < total_rows;
     const float2 *h = reinterpret_cast<const float2 *>(kap) + row * N2;
-    if constexpr (P::NPASS > 1) {
+    if constexpr (P::N >= 64) {
         if (use_tma) {
             if (threadIdx.x == 0) mbar_init(&bar, 1);
             __syncthreads();
@@ -593,9 +590,9 @@ __global__ void __launch_bounds__(256, 2) k_rows_inv32_c2r(float *kap, long tota
             h = smb + vr * N2;
         }
     }
-    float2 v[32];
+    float2 v[P::E];
 #pragma unroll
-    for (int r = 0; r < 32; ++r) {
+    for (int r = 0; r < P::E; ++r) {
         const int k = j + r * P::TV;
         float2 z = make_float2(0.f, 0.f);
         if (live) {
@@ -606,7 +603,7 @@ __global__ void __launch_bounds__(256, 2) k_rows_inv32_c2r(float *kap, long tota
                 const float2 hm = h[N2 - k];
                 const float2 ee = make_float2(hk.x + hm.x, hk.y - hm.y);  // H(k) + conj H(n/2 - k)
                 float2 od = make_float2(hk.x - hm.x, hk.y + hm.y);        // H(k) - conj H(n/2 - k)
-                od = cmul(od, twid<true>(tw, k));                         // times exp(+2 pi i k / n)
+                od = mul_tw<true>(od, tw + k);                            // times exp(+2 pi i k / n)
                 z = make_float2(ee.x - od.y, ee.y + od.x);
             }
         }
@@ -616,12 +613,7 @@ __global__ void __launch_bounds__(256, 2) k_rows_inv32_c2r(float *kap, long tota
     if (live) {
         float2 *out = reinterpret_cast<float2 *>(kap) + row * N2;  // (kappa(2m), kappa(2m + 1))
 #pragma unroll
-        for (int m = 0; m < P::ML; ++m)
-#pragma unroll
-            for (int r = 0; r < P::RL; ++r) {
-                const float2 z = v[m * P::RL + r];
-                out[j + m * P::TV + r * P::NSL] = make_float2(z.x * scale, z.y * scale);
-            }
+        for (int q = 0; q < P::E; ++q) out[j + q * P::TV] = make_float2(v[q].x * scale, v[q].y * scale);
     }
 }
 
@@ -657,20 +649,20 @@ static int ks32_real_impl(const float *in1, const float *in2, long in_bs, float 
     using P = Plan32<LOGN>;
     using P2 = Plan32<LOGN - 1>;
     using E = PlanE<LOGN>;
-    constexpr int RPC = P::TV >= kRowThreads ? 1 : kRowThreads / P::TV;
-    constexpr int RPC2 = P2::TV >= kRowThreads ? 1 : kRowThreads / P2::TV;
+    constexpr int RPC = P::RPC;
+    constexpr int RPC2 = P2::RPC;
     const long total_rows = (long)batch * P::N;
     const unsigned row_grid = (unsigned)((total_rows + RPC - 1) / RPC);
     const unsigned row2_grid = (unsigned)((total_rows + RPC2 - 1) / RPC2);
-    const size_t row_smem = (size_t)RPC * (P::N + P::N / 32) * sizeof(float2) + 128;
-    const size_t row2_smem = P2::NPASS > 1 ? (size_t)RPC2 * (P2::N + P2::N / 32) * sizeof(float2) + 128 : 0;
+    const size_t row_smem = (size_t)RPC * P::VS * sizeof(float2) + 128;
+    const size_t row2_smem = (size_t)RPC2 * P2::VS * sizeof(float2) + 128;
     const size_t col_smem = (size_t)(2 * E::RSZ) * sizeof(float2) + 128;
     const int col_threads = E::NT;
     const unsigned col_grid = (unsigned)((long)batch * (P::N / 2 / E::WS));
     auto krf = rotate ? k_rows_fwd32<LOGN, true, true> : k_rows_fwd32<LOGN, true, false>;
     FM_CUDA_TRY(fm::smem_attr((const void *)krf, row_smem));
     FM_CUDA_TRY(fm::smem_attr((const void *)k_cols_ks32_e<LOGN>, col_smem));
-    if (row2_smem) FM_CUDA_TRY(fm::smem_attr((const void *)k_rows_inv32_c2r<LOGN>, row2_smem));
+    FM_CUDA_TRY(fm::smem_attr((const void *)k_rows_inv32_c2r<LOGN>, row2_smem));
     CUtensorMap m1, m2, mc, mk;
     memset(&m1, 0, sizeof(m1));
     memset(&m2, 0, sizeof(m2));
@@ -688,7 +680,7 @@ static int ks32_real_impl(const float *in1, const float *in2, long in_bs, float 
         tma_in = (tma_mode & 2) && (in_bs == nn || (in_bs == 0 && RPC <= P::N)) &&
                  encode_map3d_f32(&m1, in1, dims, strides, box) && (!in2 || encode_map3d_f32(&m2, in2, dims, strides, box));
         // kappa's buffer as rows of n floats (= n/2 float2 of half spectrum)
-        if (P2::NPASS > 1 && (tma_mode & 4)) {
+        if (P2::N >= 64 && (tma_mode & 4)) {
             const uint64_t kdims[3] = {d0, (uint64_t)(P::N / d0), (uint64_t)total_rows};
             const uint32_t kbox[3] = {d0, (uint32_t)(P::N / d0), (uint32_t)RPC2};
             tma_out = encode_map3d_f32(&mk, out1, kdims, strides, kbox);
@@ -720,15 +712,15 @@ static int ks32_impl(const float *in1, const float *in2, long in_bs, float *out1
             return ks32_real_impl<LOGN>(in1, in2, in_bs, out1, work, batch, out_scale, seed, r0, rotate, tw, tw2, s);
     }
     using P = Plan32<LOGN>;
-    constexpr int RPC = P::TV >= kRowThreads ? 1 : kRowThreads / P::TV;
+    constexpr int RPC = P::RPC;
     const long total_rows = (long)batch * P::N;
     const unsigned row_grid = (unsigned)((total_rows + RPC - 1) / RPC);
     // exchange buffer (which also stages the TMA rows: RPC n floats per input
-    // array or RPC n float2 <= RPC (n + n/32) float2) + 128 bytes of alignment
-    const size_t row_smem = P::NPASS > 1 ? (size_t)RPC * (P::N + P::N / 32) * sizeof(float2) + 128 : 0;
+    // array or RPC n float2 <= RPC (n + n/16) float2) + 128 bytes of alignment
+    const size_t row_smem = (size_t)RPC * P::VS * sizeof(float2) + 128;
     const int col_threads = P::W * P::TV;
     // exchange buffer (also the TMA strip: n W float2) + 128 bytes of alignment
-    const size_t col_smem = P::NPASS > 1 ? (size_t)(P::N * P::W + P::N * P::W / 32 + 1) * sizeof(float2) + 128 : 0;
+    const size_t col_smem = (size_t)(P::N * P::W + P::N * P::W / 16 + 1) * sizeof(float2) + 128;
     const unsigned col_grid = (unsigned)((long)batch * (P::N / P::W));
     auto krf = rotate ? k_rows_fwd32<LOGN, false, true> : k_rows_fwd32<LOGN, false, false>;
     FM_CUDA_TRY(fm::smem_attr((const void *)krf, row_smem));
@@ -745,7 +737,7 @@ static int ks32_impl(const float *in1, const float *in2, long in_bs, float *out1
     memset(&mw, 0, sizeof(mw));
     int tma_in = 0, tma_out = 0;
     const int tma_mode = g_use_tma.load(std::memory_order_relaxed);
-    if (P::NPASS > 1 && (tma_mode & 6)) {
+    if (P::N >= 64 && (tma_mode & 6)) {
         const long nn = (long)P::N * P::N;
         const uint32_t d0 = P::N < 256 ? P::N : 256;
         const uint64_t rows = in_bs == 0 ? (uint64_t)P::N : (uint64_t)total_rows;
@@ -770,7 +762,7 @@ static int ks32_impl(const float *in1, const float *in2, long in_bs, float *out1
     CUtensorMap mc;
     memset(&mc, 0, sizeof(mc));
     int tma_col = 0;
-    if (P::NPASS > 1 && P::N >= 1024 && (tma_mode & 32)) {
+    if (P::N >= 1024 && (tma_mode & 32)) {
         const uint64_t cdims[3] = {(uint64_t)2 * P::N, (uint64_t)P::N, (uint64_t)batch};
         const uint64_t cstrides[2] = {(uint64_t)P::N * 8, (uint64_t)P::N * P::N * 8};
         const uint32_t cbox[3] = {(uint32_t)(2 * P::W), (uint32_t)(P::N < 256 ? P::N : 256), 1};

@@ -1,0 +1,59 @@
+// fft32_tables.cuh -- pass structure and twiddle tables of the fp32
+// register-resident FFT (fft32.cu), shared by the kernels and by the host
+// code that fills the tables (runtime.cu, noalloc.cu).
+//
+// A table for length n holds the natural table exp(-2 pi i t / n), t = 0 ..
+// n - 1, and after it one block per Stockham pass p >= 1 with the twiddles in
+// the order a warp reads them: entry [r - 1][k] = W^(r k) with k = 0 .. Ns - 1
+// consecutive, so a load of 32 neighbouring threads covers one or two cache
+// lines (taken from the natural table, the 16 threads of a pass with Ns = 16
+// gathered from up to 16 lines).
+#pragma once
+
+#include <math.h>
+
+#include <vector>
+
+#include "common.cuh"
+
+namespace fm {
+
+// elements a thread holds (the radix of all passes but the last) for n = 2^logn
+__host__ __device__ constexpr int fft_log_e(int logn) { return logn <= 8 ? 4 : 5; }
+
+// n = 2^LOGN split into radix-E passes and one last radix RL
+template <int LOGN> struct FftPlan {
+    static constexpr int N = 1 << LOGN;
+    static constexpr int LOGE = fft_log_e(LOGN), E = 1 << LOGE;  // elements per thread
+    static constexpr int TV = N / E;                             // threads per vector
+    static constexpr int NPASS = (LOGN + LOGE - 1) / LOGE;       // passes (all radix E but the last)
+    static constexpr int LOGRL = LOGN - LOGE * (NPASS - 1);      // log2 of the last radix
+    static constexpr int RL = 1 << LOGRL;
+    static constexpr int ML = E / RL;   // butterflies per thread in the last pass
+    static constexpr int NSL = N / RL;  // stride of the last pass outputs (= ML TV)
+    static_assert(NPASS >= 2, "at least two passes");
+    // first entry of pass p's block after the natural table: (E - 1) E^q
+    // entries for each earlier pass q = 1 .. p - 1
+    __host__ __device__ static constexpr int pass_off(int p) { return (1 << (LOGE * p)) - E; }
+};
+
+// the natural table and the blocks of passes 1 .. (their sizes sum to n - E)
+inline int fft32_table_elems(int n) { return 2 * n - (1 << fft_log_e(ilog2((unsigned)n))); }
+
+// fills fft32_table_elems(n) entries (FP64 on the host, rounded once)
+inline void fft32_fill_table(int n, float2 *t)
+{
+    auto w = [n](long e) {
+        const double ang = -2.0 * M_PI * (double)(e % n) / (double)n;
+        return make_float2((float)cos(ang), (float)sin(ang));
+    };
+    for (int i = 0; i < n; ++i) *t++ = w(i);
+    const int logn = ilog2((unsigned)n), loge = fft_log_e(logn), np = (logn + loge - 1) / loge;
+    for (int p = 1; p < np; ++p) {
+        const int ns = 1 << (loge * p), radix = p + 1 < np ? 1 << loge : n / ns;
+        for (int r = 1; r < radix; ++r)
+            for (int k = 0; k < ns; ++k) *t++ = w((long)r * k * (n / (ns * radix)));
+    }
+}
+
+}  // namespace fm

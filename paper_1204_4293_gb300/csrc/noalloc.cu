@@ -6,7 +6,7 @@
 // memory is reserved up front by another framework's pool, so that a fresh
 // allocation would fail, or a latency-critical loop that must never enter the
 // allocator.  fm_ks_invert_noalloc serves them: its work buffer and FFT
-// twiddle tables live in file-scope device arrays (32 MiB + 32 KiB per
+// twiddle tables live in file-scope device arrays (32 MiB + 63 KiB per
 // device).  The driver allocates them when it loads this file's module on a
 // device: under CUDA's default lazy module loading that happens at the first
 // call on that device (the set-up below), with eager loading when the
@@ -18,6 +18,7 @@
 #include <vector>
 
 #include "common.cuh"
+#include "fft32_tables.cuh"
 
 namespace fm {
 namespace {
@@ -25,7 +26,15 @@ namespace {
 constexpr long kNoallocWorkElems = 4l << 20;  // float2 elements: 32 MiB
 // batch * n^2 <= 4194304 caps n at 2048 (a batch of one)
 constexpr int kTwMinN = 32, kTwMaxN = 2048;
-constexpr int kTwElems = 2 * kTwMaxN - kTwMinN;  // tables n = 32, 64, ..., 2048 back to back
+// tables n = 32, 64, ..., 2048 back to back, 2 n entries 
+// at most (fft32_table_elems: the natural table and the pass tables)
+constexpr int kTwElems = 2 * (2 * kTwMaxN - kTwMinN);
+int tw_offset(int n)
+{
+    int off = 0;
+    for (int m = kTwMinN; m < n; m *= 2) off += fft32_table_elems(m);
+    return off;
+}
 
 static __device__ __align__(256) float2 g_noalloc_work[kNoallocWorkElems];
 static __device__ __align__(256) float2 g_noalloc_tw[kTwElems];
@@ -39,7 +48,7 @@ std::unordered_map<int, DevState> g_state;
 
 // Once per device, with that device current: take the arrays' device
 // addresses (their host-side names are only stand-ins) and fill the twiddle
-// tables exp(-2 pi i t / n), computed on the host in FP64, with a synchronous
+// tables (fft32_fill_table), computed on the host in FP64, with a synchronous
 // copy.  Nothing is allocated.
 int setup(int dev, DevState **out)
 {
@@ -53,11 +62,11 @@ int setup(int dev, DevState **out)
     FM_CUDA_TRY(cudaGetSymbolAddress((void **)&st.work, g_noalloc_work));
     FM_CUDA_TRY(cudaGetSymbolAddress((void **)&st.tw, g_noalloc_tw));
     std::vector<float2> host(kTwElems);
-    for (int n = kTwMinN, off = 0; n <= kTwMaxN; off += n, n *= 2)
-        for (int t = 0; t < n; ++t) {
-            const double ang = -2.0 * M_PI * (double)t / (double)n;
-            host[off + t] = make_float2((float)cos(ang), (float)sin(ang));
-        }
+    if (tw_offset(2 * kTwMaxN) > kTwElems) {
+        set_error("fm_ks_invert_noalloc: twiddle tables larger than their array");
+        return FM_ECUDA;
+    }
+    for (int n = kTwMinN; n <= kTwMaxN; n *= 2) fft32_fill_table(n, host.data() + tw_offset(n));
     FM_CUDA_TRY(cudaMemcpy(st.tw, host.data(), host.size() * sizeof(float2), cudaMemcpyHostToDevice));
     *out = &(g_state[dev] = st);
     return FM_OK;
@@ -96,9 +105,9 @@ extern "C" int fm_ks_invert_noalloc(const void *g1, const void *g2, void *kappa_
     DevState *st = nullptr;
     int r = setup(dev, &st);
     if (r != FM_OK) return r;
-    const float2 *tw = st->tw + (n - kTwMinN);  // sum of the smaller tables' sizes
+    const float2 *tw = st->tw + tw_offset(n);
     // the half-length table for the real-output inverse where it is the faster one
-    const float2 *tw2 = n >= 2 * kTwMinN && ks_real_for(n, false) ? st->tw + (n / 2 - kTwMinN) : nullptr;
+    const float2 *tw2 = n >= 2 * kTwMinN && ks_real_for(n, false) ? st->tw + tw_offset(n / 2) : nullptr;
     return launch_ks32((const float *)g1, (const float *)g2, (long)n * n, (float *)kappa_E, (float *)kappa_B, st->work,
                        n, batch, false, 0, 0, false, tw, tw2, (cudaStream_t)stream);
 }

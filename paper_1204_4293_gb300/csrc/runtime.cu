@@ -12,6 +12,7 @@
 #include <vector>
 
 #include "common.cuh"
+#include "fft32_tables.cuh"
 #include "tma.cuh"
 
 namespace fm {
@@ -115,18 +116,25 @@ static const void *twiddles_one(int n, int precision, cudaStream_t s, int *statu
     std::lock_guard<std::mutex> lk(g_tw_mu);
     auto it = g_tw.find(key);
     if (it != g_tw.end()) return it->second;
-    // exp(-2 pi i t / n) in FP64 on the host, rounded once to the element type
-    const size_t esz = precision == FM_F64 ? 16 : 8;
-    std::vector<unsigned char> host((size_t)n * esz);
-    for (int t = 0; t < n; ++t) {
-        const double ang = -2.0 * M_PI * (double)t / (double)n;
-        const double c = cos(ang), sn = sin(ang);
-        if (precision == FM_F64) {
-            double v[2] = {c, sn};
-            memcpy(&host[(size_t)t * esz], v, esz);
-        } else {
-            float v[2] = {(float)c, (float)sn};
-            memcpy(&host[(size_t)t * esz], v, esz);
+    // exp(-2 pi i t / n) in FP64 on the host, rounded once to the element type;
+    // fp32 lengths of the register-resident FFT carry its pass tables as well
+    std::vector<unsigned char> host;
+    if (precision == FM_F32 && n >= 32) {
+        host.resize((size_t)fft32_table_elems(n) * sizeof(float2));
+        fft32_fill_table(n, reinterpret_cast<float2 *>(host.data()));
+    } else {
+        const size_t esz = precision == FM_F64 ? 16 : 8;
+        host.resize((size_t)n * esz);
+        for (int t = 0; t < n; ++t) {
+            const double ang = -2.0 * M_PI * (double)t / (double)n;
+            const double c = cos(ang), sn = sin(ang);
+            if (precision == FM_F64) {
+                double v[2] = {c, sn};
+                memcpy(&host[(size_t)t * esz], v, esz);
+            } else {
+                float v[2] = {(float)c, (float)sn};
+                memcpy(&host[(size_t)t * esz], v, esz);
+            }
         }
     }
     void *d = nullptr;
