@@ -3,70 +3,123 @@
 // kurtosis over the pixels.
 //
 // Two passes over the pyramid: the first sums x per (map, array), the second
-// sums (x - mean)^2, ^3, ^4.  Each thread keeps fp32 partial sums over its
-// pixels, a block folds them in FP64 through warp shuffles and one FP64
-// atomic per block and quantity lands in the per-array sums; a last tiny
-// kernel forms the moments.
+// sums (x - mean)^2, ^3, ^4.  A strand is the run of at most 16 pixels S
+// apart (S = 256 ceil(nn / 4096)) whose sums are formed in fp32; strands are
+// added in pairs of floats (hi + lo by error-free two-sums) over a thread and
+// a block, and by one FP64 atomic per block and quantity; a last tiny kernel
+// forms the moments.
+//
+// The work is two reads of the pyramid.  FP64 adds are the scarce resource
+// otherwise (one warp instruction in 16 to 32 cycles an SM on GB300): an FP64
+// shuffle tree over every thread's sums kept the second pass at 219 us for 8
+// pyramids of 7 x 1024^2 (235 MB, 35 us a read).  The float pairs carry 48
+// bits and leave FP64 a few instructions a block; 16-byte loads, eight in
+// flight a thread.  Those 8 pyramids: 293 -> 88 us for the whole call.
+// Running both passes over 20 .. 80 MB groups of arrays, so that the second
+// read comes from L2, was no faster (154 .. 90 us: shorter launches).
+#include <algorithm>
+
 #include "common.cuh"
 
 namespace fm {
 
-__device__ __forceinline__ double warp_sum(double v)
+// hi + lo = the exact sum of the floats added so far, up to the rounding of
+// lo.  Sums of 2^100 and more (and infinities and NaN) move to FP64.
+struct FloatPair {  // (no initialisers: it is kept in shared memory too)
+    float hi, lo;
+    __device__ __forceinline__ void add(float p)
+    {
+        const float s = __fadd_rn(hi, p), b = __fsub_rn(s, hi);
+        lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, b)), __fsub_rn(p, b)));
+        hi = s;
+    }
+    __device__ __forceinline__ double value() const { return isfinite(hi) ? (double)hi + (double)lo : (double)hi; }
+    __device__ __forceinline__ bool large() const { return !(fabsf(hi) < 1.2676506e30f); }  // 2^100
+};
+
+// the sum over the first N lanes' pairs, in lane 0
+template <int N> __device__ __forceinline__ FloatPair lane_sum(FloatPair v)
 {
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+    for (int o = N / 2; o > 0; o >>= 1) {
+        const float h = __shfl_down_sync(0xffffffffu, v.hi, o), l = __shfl_down_sync(0xffffffffu, v.lo, o);
+        v.add(h);
+        v.lo = __fadd_rn(v.lo, l);
+    }
     return v;
 }
 
-// grid = (blocks per array, J, batch); sums[(b * J + j) * 4 + q]
-template <typename T, int PASS>
-__global__ void __launch_bounds__(256) k_moments(const T *__restrict__ pyr, long nn, int J, double *__restrict__ sums)
+// grid = (blocks per array, J, batch); sums[(b * J + j) * 4 + q].  A thread takes VW neighbouring
+// strands at a time (VW > 1: nn a multiple of VW and 16-byte aligned arrays).
+template <typename T, int PASS, int VW>
+__global__ void __launch_bounds__(256) k_moments(const T *__restrict__ pyr, long nn, long S, double inv_nn,
+                                                 double *__restrict__ sums)
 {
     pdl_entry();
-    const long b = blockIdx.z;
-    const int j = blockIdx.y;
-    const T *x = pyr + (b * J + j) * nn;
-    double *acc = sums + (b * J + j) * 4;
-    const float mean = PASS == 0 ? 0.f : (float)(acc[0] / (double)nn);
-    float s1 = 0.f, s2 = 0.f, s3 = 0.f;
-    for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < nn; i += (long)gridDim.x * blockDim.x) {
-        const float v = (float)x[i];
-        if (PASS == 0) {
-            s1 += v;
-        } else {
-            const float d = v - mean, d2 = d * d;
-            s1 += d2;
-            s2 += d2 * d;
-            s3 += d2 * d2;
+    constexpr int NQ = PASS == 0 ? 1 : 3;
+    struct alignas(VW * sizeof(T)) Vec {
+        T e[VW];
+    };
+    const long array = (long)blockIdx.z * gridDim.y + blockIdx.y;
+    const T *x = pyr + array * nn;
+    double *acc = sums + array * 4;
+    __shared__ float s_mean;
+    __shared__ FloatPair red[NQ][8];
+    float mean = 0.f;
+    if constexpr (PASS == 1) {
+        if (threadIdx.x == 0) s_mean = (float)(acc[0] * inv_nn);
+        __syncthreads();
+        mean = s_mean;
+    }
+    FloatPair tot[NQ];
+#pragma unroll
+    for (int q = 0; q < NQ; ++q) tot[q] = FloatPair{0.f, 0.f};
+    for (long v0 = ((long)blockIdx.x * 256 + threadIdx.x) * VW; v0 < S; v0 += (long)gridDim.x * 256 * VW) {
+        float s[VW][NQ] = {};
+        auto add = [&](const Vec &v) {
+#pragma unroll
+            for (int u = 0; u < VW; ++u) {
+                if constexpr (PASS == 0) {
+                    s[u][0] += (float)v.e[u];
+                } else {
+                    const float d = (float)v.e[u] - mean, d2 = d * d;
+                    s[u][0] += d2;
+                    s[u][1] += d2 * d;
+                    s[u][2] += d2 * d2;
+                }
+            }
+        };
+        long i = v0;
+        for (; i + 7 * S < nn; i += 8 * S) {  // eight loads in flight
+            Vec v[8];
+#pragma unroll
+            for (int k = 0; k < 8; ++k) v[k] = *reinterpret_cast<const Vec *>(x + i + k * S);
+#pragma unroll
+            for (int k = 0; k < 8; ++k) add(v[k]);
+        }
+        for (; i < nn; i += S) add(*reinterpret_cast<const Vec *>(x + i));
+#pragma unroll
+        for (int q = 0; q < NQ; ++q) {
+#pragma unroll
+            for (int u = 0; u < VW; ++u) {
+                tot[q].add(s[u][q]);
+                if (tot[q].large()) {
+                    atomicAdd(acc + PASS + q, tot[q].value());
+                    tot[q] = FloatPair{0.f, 0.f};
+                }
+            }
         }
     }
-    __shared__ double red[3][8];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    double r0 = warp_sum((double)s1), r1 = 0, r2 = 0;
-    if (PASS) {
-        r1 = warp_sum((double)s2);
-        r2 = warp_sum((double)s3);
-    }
-    if (lane == 0) {
-        red[0][warp] = r0;
-        red[1][warp] = r1;
-        red[2][warp] = r2;
+#pragma unroll
+    for (int q = 0; q < NQ; ++q) {
+        const FloatPair r = lane_sum<32>(tot[q]);
+        if (lane == 0) red[q][warp] = r;
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
-        double t0 = 0, t1 = 0, t2 = 0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
-            t0 += red[0][w];
-            t1 += red[1][w];
-            t2 += red[2][w];
-        }
-        if (PASS == 0) {
-            atomicAdd(acc + 0, t0);
-        } else {
-            atomicAdd(acc + 1, t0);
-            atomicAdd(acc + 2, t1);
-            atomicAdd(acc + 3, t2);
-        }
+    if (warp < NQ) {  // one quantity a warp
+        const FloatPair r = lane_sum<8>(lane < 8 ? red[warp][lane] : FloatPair{0.f, 0.f});
+        if (lane == 0) atomicAdd(acc + PASS + warp, r.value());
     }
 }
 
@@ -85,6 +138,23 @@ __global__ void k_moments_final(const double *__restrict__ sums, double *__restr
     o[3] = m2 > 0 ? m4 / (m2 * m2) - 3.0 : 0.0;
 }
 
+template <typename T, int VW>
+static int moments_impl(const T *pyr, double *sums, int J, int batch, long nn, cudaStream_t s)
+{
+    long per = (nn + 256 * 16 - 1) / (256 * 16);  // strands of ~16 pixels (fp32 partial sums)
+    if (per > 4096) per = 4096;
+    const long S = per * 256;
+    // about eight blocks an SM over all arrays (4 / 8: 93 / 88 us for 8
+    // pyramids of 7 x 1024^2), at least one an array
+    const long count = (long)J * batch;
+    const long bx = std::min<long>((S / VW + 255) / 256, std::max<long>(1, (152 * 8 + count - 1) / count));
+    const dim3 grid((unsigned)bx, J, batch);
+    const double inv_nn = 1.0 / (double)nn;
+    FM_LAUNCH(0, (k_moments<T, 0, VW>), grid, 256, 0, s, pyr, nn, S, inv_nn, sums);
+    FM_LAUNCH(0, (k_moments<T, 1, VW>), grid, 256, 0, s, pyr, nn, S, inv_nn, sums);
+    return FM_OK;
+}
+
 int launch_band_moments(const void *pyr, double *moments, int n, int J, int batch, int precision, void *scratch,
                         cudaStream_t s)
 {
@@ -92,16 +162,15 @@ int launch_band_moments(const void *pyr, double *moments, int n, int J, int batc
     double *sums = static_cast<double *>(scratch);
     const int count = batch * J;
     FM_CUDA_TRY(cudaMemsetAsync(sums, 0, sizeof(double) * 4 * (size_t)count, s));
-    long per = (nn + 256 * 16 - 1) / (256 * 16);  // ~16 pixels per thread (fp32 partial sums)
-    if (per > 4096) per = 4096;
-    const dim3 grid((unsigned)per, J, batch);
-    if (precision == FM_F64) {
-        FM_LAUNCH(0, (k_moments<double, 0>), grid, 256, 0, s, (const double *)pyr, nn, J, sums);
-        FM_LAUNCH(0, (k_moments<double, 1>), grid, 256, 0, s, (const double *)pyr, nn, J, sums);
-    } else {
-        FM_LAUNCH(0, (k_moments<float, 0>), grid, 256, 0, s, (const float *)pyr, nn, J, sums);
-        FM_LAUNCH(0, (k_moments<float, 1>), grid, 256, 0, s, (const float *)pyr, nn, J, sums);
-    }
+    const bool al = (reinterpret_cast<uintptr_t>(pyr) & 15) == 0;
+    int st;
+    if (precision == FM_F64)
+        st = al && nn % 2 == 0 ? moments_impl<double, 2>((const double *)pyr, sums, J, batch, nn, s)
+                               : moments_impl<double, 1>((const double *)pyr, sums, J, batch, nn, s);
+    else
+        st = al && nn % 4 == 0 ? moments_impl<float, 4>((const float *)pyr, sums, J, batch, nn, s)
+                               : moments_impl<float, 1>((const float *)pyr, sums, J, batch, nn, s);
+    if (st != FM_OK) return st;
     FM_LAUNCH(0, k_moments_final, (unsigned)((count + 127) / 128), 128, 0, s, sums, moments, nn, count);
     return FM_OK;
 }
