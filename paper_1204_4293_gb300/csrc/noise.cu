@@ -117,37 +117,114 @@ __device__ __forceinline__ void noise_sums(const void *acc, long nelem, long i, 
     }
 }
 
-template <typename T, bool KAHAN>
-__global__ void k_noise_final(const void *__restrict__ acc, const T *__restrict__ wdata, double *__restrict__ var,
-                              T *__restrict__ snr, long nelem, int R)
+__device__ __forceinline__ double snr_of(double w, double v) { return w / sqrt(v); }
+// fp32 result: w / sqrt(v) with v in FP64.  FP64 square root and division
+// are some 40 instructions of a pipe that takes one warp in 16 to 32 cycles,
+// so the usual case runs in fp32 pairs: v is split by its bits into hi (24
+// leading bits) + lo, y = rsqrt(hi) gets the residual e = 1 - v y^2 from
+// exact products (fma), and w y (1 + e / 2) is rounded once: its error is
+// that of the rounding plus 3/8 e^2 < 2^-43.  Values near the ends of the
+// fp32 range (and zeros, infinities, NaN) take the FP64 form.
+__device__ __forceinline__ float snr_of(float w, double v)
+{
+    const uint32_t vh = (uint32_t)__double2hiint(v), vl = (uint32_t)__double2loint(v);
+    const int ex = (int)(vh >> 20) - 1023;  // sign and exponent: negative v fails the test below
+    const float aw = fabsf(w);
+    if (ex >= -64 && ex <= 64 && aw >= 5.421011e-20f && aw <= 1.844674e19f) {  // 2^-64 .. 2^64
+        const float hi = __uint_as_float((uint32_t)(ex + 127) << 23 | (vh & 0xfffffu) << 3 | vl >> 29);
+        const float lo = (float)(vl & 0x1fffffffu) * __uint_as_float((uint32_t)(ex - 52 + 127) << 23);
+        const float y = rsqrtf(hi);
+        const float p = __fmul_rn(hi, y), pe = __fmaf_rn(hi, y, -p);  // hi y = p + pe
+        const float e = __fmaf_rn(-p, y, 1.f) - __fmul_rn(__fmaf_rn(lo, y, pe), y);
+        const float r = __fmul_rn(w, y), re = __fmaf_rn(w, y, -r);
+        return __fadd_rn(r, __fmaf_rn(r, 0.5f * e, re));
+    }
+    return (float)((double)w / sqrt(v));
+}
+
+// VW neighbouring elements a thread (nelem is a multiple of VW)
+template <typename T, bool KAHAN, int VW>
+__global__ void __launch_bounds__(256) k_noise_final(const void *__restrict__ acc, const T *__restrict__ wdata,
+                                                     double *__restrict__ var, T *__restrict__ snr, long nelem,
+                                                     double invR, double invR1)
 {
     pdl_entry();
-    const double invR = 1.0 / R, invR1 = 1.0 / (R - 1);
-    for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < nelem; i += (long)gridDim.x * blockDim.x) {
-        double a, q;
-        noise_sums<KAHAN>(acc, nelem, i, a, q);
-        double v = (q - a * a * invR) * invR1;
-        v = v < 0 ? 0 : v;
-        var[i] = v;
-        if (snr) snr[i] = (T)((double)wdata[i] / sqrt(v));
+    struct alignas(VW * sizeof(T)) Vec {
+        T e[VW];
+    };
+    struct alignas(16) Var {
+        double e[2];
+    };
+    for (long i = (blockIdx.x * (long)blockDim.x + threadIdx.x) * VW; i < nelem;
+         i += (long)gridDim.x * blockDim.x * VW) {
+        double v[VW], s1[VW], s2[VW];
+        if constexpr (VW == 2 && !KAHAN) {
+            const double *d = static_cast<const double *>(acc);
+            const Var a = *reinterpret_cast<const Var *>(d + i), q = *reinterpret_cast<const Var *>(d + nelem + i);
+            s1[0] = a.e[0];
+            s1[1] = a.e[1];
+            s2[0] = q.e[0];
+            s2[1] = q.e[1];
+        } else {
+#pragma unroll
+            for (int u = 0; u < VW; ++u) noise_sums<KAHAN>(acc, nelem, i + u, s1[u], s2[u]);
+        }
+#pragma unroll
+        for (int u = 0; u < VW; ++u) {
+            const double a = s1[u], q = s2[u];
+            v[u] = (q - a * a * invR) * invR1;
+            // v < 0 (rounding) by its bits, without an FP64 comparison; NaN stays
+            const uint32_t vh = (uint32_t)__double2hiint(v[u]);
+            if (vh >= 0x80000000u && vh <= 0xfff00000u) v[u] = 0;
+        }
+        if constexpr (VW == 1) {
+            var[i] = v[0];
+        } else {
+#pragma unroll
+            for (int u = 0; u < VW; u += 2) *reinterpret_cast<Var *>(var + i + u) = Var{{v[u], v[u + 1]}};
+        }
+        if (snr) {
+            Vec w = *reinterpret_cast<const Vec *>(wdata + i);
+#pragma unroll
+            for (int u = 0; u < VW; ++u) w.e[u] = snr_of(w.e[u], v[u]);
+            *reinterpret_cast<Vec *>(snr + i) = w;
+        }
     }
 }
 
+template <typename T, bool KAHAN, int VW>
+static int final_launch(const void *acc, const T *wdata, double *var, T *snr, long nelem, int R, cudaStream_t s)
+{
+    long g = (nelem / VW + 255) / 256;
+    if (g > 152L * 32) g = 152L * 32;
+    FM_LAUNCH(FM_K_NOISE_FINAL, (k_noise_final<T, KAHAN, VW>), (unsigned)g, 256, 0, s, acc, wdata, var, snr, nelem,
+              1.0 / R, 1.0 / (R - 1));
+    return FM_OK;
+}
+
+// Bound by HBM: 16 bytes of sums read and 8 (and 4 + 4 for the S/N) written
+// an element.  6 bands of 1024^2 with S/N: 269 -> NOISE_FINAL us (FP64
+// square root, division and comparison before).
 int launch_noise_finalize(const void *acc, const void *wdata, double *var, void *snr, long nelem, int R,
                           int precision, int accum, cudaStream_t s)
 {
-    long g = (nelem + 255) / 256;
-    if (g > 152L * 16) g = 152L * 16;
-    if (precision == FM_F64)
-        FM_LAUNCH(FM_K_NOISE_FINAL, (k_noise_final<double, false>), (unsigned)g, 256, 0, s, acc,
-                  (const double *)wdata, var, (double *)snr, nelem, R);
-    else if (accum == 1)
-        FM_LAUNCH(FM_K_NOISE_FINAL, (k_noise_final<float, true>), (unsigned)g, 256, 0, s, acc, (const float *)wdata,
-                  var, (float *)snr, nelem, R);
-    else
-        FM_LAUNCH(FM_K_NOISE_FINAL, (k_noise_final<float, false>), (unsigned)g, 256, 0, s, acc, (const float *)wdata,
-                  var, (float *)snr, nelem, R);
-    return FM_OK;
+    // two elements a thread where every array allows the wide accesses (the
+    // caller's pointers need not be aligned beyond their type)
+    auto al = [](const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; };
+    const bool wide = nelem % 2 == 0 && al(acc) && al(wdata) && al(var) && al(snr);
+    if (precision == FM_F64) {
+        const double *w = static_cast<const double *>(wdata);
+        double *o = static_cast<double *>(snr);
+        return wide ? final_launch<double, false, 2>(acc, w, var, o, nelem, R, s)
+                    : final_launch<double, false, 1>(acc, w, var, o, nelem, R, s);
+    }
+    const float *w = static_cast<const float *>(wdata);
+    float *o = static_cast<float *>(snr);
+    if (accum == 1)
+        return wide ? final_launch<float, true, 2>(acc, w, var, o, nelem, R, s)
+                    : final_launch<float, true, 1>(acc, w, var, o, nelem, R, s);
+    return wide ? final_launch<float, false, 2>(acc, w, var, o, nelem, R, s)
+                : final_launch<float, false, 1>(acc, w, var, o, nelem, R, s);
 }
 
 // ---- exact expected variance (periodic boundary) ----------------------------
