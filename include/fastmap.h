@@ -181,9 +181,11 @@ int fm_map_direct_masked(const void *g1, const void *g2, const void *weight, lon
  * (bands only) in L2-sized chunks alternating over the library's streams,
  * then one pass adds its bands to the FP64 sums (or, with cfg->accum = 1,
  * to fp32 sums with Kahan compensation) while the chunks run on into the
- * next batch (two pyramid buffers).  The whole call is recorded once into a
- * CUDA graph (keyed by pointers, sizes, R, seed, config and chunk plan) and
- * replayed as one launch.  Scratch: 16 (J-1) bytes per pixel of sums, the
+ * next batch (two pyramid buffers).  The realisations are recorded once into a
+ * CUDA graph (keyed by sizes, R, config and chunk plan; it reads copies of
+ * the shear and the seed, so it serves every buffer and seed of a shape) and
+ * replayed as one launch; calls of one shape on several streams follow each
+ * other.  Scratch: 16 (J-1) bytes per pixel of sums, the shear's copies, the
  * batches' pyramids and the chunks' intermediates, kept with the graph until
  * fm_trim or eviction. */
 int fm_map_noise(const void *g1, const void *g2, double *var_out, void *snr_out, int n, int J, int R, uint64_t seed,
@@ -324,7 +326,7 @@ int fm_device_error(void);
  *                        maps, so two chunks in flight stay in L2); 0 = no
  *                        chunking
  *   FM_TUNE_GRAPHS       1 = replay batched calls from cached CUDA graphs
- *                        (default), 0 = launch every kernel each call
+ *                        once their buffers come back (default), 0 = launch every kernel each call
  *   FM_TUNE_CHUNK_STREAMS number of streams chunks alternate on (1 to 4,
  *                        default 2)
  *   FM_TUNE_PDL          1 = launch kernels as programmatic dependents of
@@ -419,9 +421,10 @@ int fm_autotune_save(const char *path);
 int fm_autotune_load(const char *path);
 int fm_autotune_clear(void);
 
-/* Batched fm_map_starlet calls (when chunked) and fm_map_noise calls are
- * recorded once into CUDA graphs that keep their scratch (a few per kind,
- * least recently used dropped first).  fm_trim waits for the device and
+/* Batched fm_map_starlet calls (when chunked) that come back with the same
+ * buffers, and fm_map_noise calls by shape, are recorded once into CUDA graphs
+ * that keep their scratch (a few per kind, least recently used dropped
+ * first).  fm_trim waits for the device and
  * frees all of them. */
 int fm_trim(void);
 

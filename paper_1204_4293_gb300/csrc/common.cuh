@@ -177,10 +177,12 @@ int check_config(const fm_config &c);
 cudaError_t smem_attr(const void *kernel, size_t bytes);
 
 // ---- internal launchers (defined per .cu file) ------------------------------------
+// rotate: the noise maps' rotated shear; rot_seed is then the generator's seed
+// in device memory (so that a recorded graph serves every seed)
 // batched: a chunk of the batched KS + starlet pipeline (the real-output
 // inverse is chosen by ks_real_for(n, batched))
 int launch_ks(const void *in1, const void *in2, long in_bstride, void *out1, void *out2, void *work, int n, int batch,
-              int precision, bool forward, uint64_t rot_seed, int rot_r0, bool rotate, cudaStream_t s,
+              int precision, bool forward, const uint64_t *rot_seed, int rot_r0, bool rotate, cudaStream_t s,
               bool batched = false);
 // bands_only: the smooth array c_{J-1} is not written (noise realisations)
 int launch_starlet(const void *kappa, void *pyr, long pyr_bstride, int n, int J, int batch, const fm_config &cfg,
@@ -188,7 +190,7 @@ int launch_starlet(const void *kappa, void *pyr, long pyr_bstride, int n, int J,
 // tw2: the twiddle table of n/2 (the real-output inverse), or null for the
 // complex inverse
 int launch_ks32(const float *in1, const float *in2, long in_bs, float *out1, float *out2, float2 *work, int n,
-                int batch, bool forward, uint64_t seed, int r0, bool rotate, const float2 *tw, const float2 *tw2,
+                int batch, bool forward, const uint64_t *seed, int r0, bool rotate, const float2 *tw, const float2 *tw2,
                 cudaStream_t s);
 // Spectral operation of the column pass of the 2-D FFT pipeline
 // rows FFT -> columns FFT -> op -> columns IFFT -> rows IFFT (Re, Im):
@@ -199,10 +201,10 @@ int launch_ks32(const float *in1, const float *in2, long in_bs, float *out1, flo
 //   FFT_OP_SPECTRUM stop after the columns FFT: `work` holds the spectrum
 enum { FFT_OP_KS_INV = 0, FFT_OP_KS_FWD = 1, FFT_OP_FILTER = 2, FFT_OP_SPECTRUM = 3 };
 int launch_fft_op(const void *in1, const void *in2, long in_bstride, void *out1, void *out2, void *work, int n,
-                  int batch, int precision, int op, const void *filt, double out_scale, uint64_t rot_seed, int rot_r0,
+                  int batch, int precision, int op, const void *filt, double out_scale, const uint64_t *rot_seed, int rot_r0,
                   bool rotate, cudaStream_t s, bool real_ok = false);
 int launch_fft32(const float *in1, const float *in2, long in_bs, float *out1, float *out2, float2 *work, int n,
-                 int batch, int op, const float2 *filt, float out_scale, uint64_t seed, int r0, bool rotate,
+                 int batch, int op, const float2 *filt, float out_scale, const uint64_t *seed, int r0, bool rotate,
                  const float2 *tw, const float2 *tw2, cudaStream_t s);
 // inverse KS with a real output (kappa_E only) through the half spectrum
 // (FM_TUNE_KS_REAL): -1 = by size (default), 0 = never, 1 = whenever
@@ -256,6 +258,10 @@ int launch_band_moments(const void *pyr, double *moments, int n, int J, int batc
 // acc: FP64 S1, S2 (accum 0) or fp32 Kahan pairs s1, c1, s2, c2 (accum 1), bands * nn elements each
 int launch_noise_accum(const void *pyr, int nb, long pyr_bs, long nn, int bands, void *acc, int precision, int accum,
                        cudaStream_t s);
+// the seed into *dseed and, unless d1 is null, the two input maps (bytes each)
+// into the library's copies d1, d2
+int launch_noise_stage(const void *g1, const void *g2, void *d1, void *d2, size_t bytes, uint64_t seed,
+                       uint64_t *dseed, cudaStream_t s);
 int launch_noise_finalize(const void *acc, const void *wdata, double *var, void *snr, long nelem, int R,
                           int precision, int accum, cudaStream_t s);
 

@@ -105,7 +105,7 @@ template <typename T, int E>
 __global__ void __launch_bounds__(1024) k_rows_fwd(const T *__restrict__ in1, const T *__restrict__ in2,
                                                    long in_bstride, cplx_t<T> *__restrict__ work, int n, int logn,
                                                    int lognvec, long total_rows, const cplx_t<T> *__restrict__ tw,
-                                                   uint64_t seed, int r0, int rotate)
+                                                   const uint64_t *seed, int r0, int rotate)
 {
     pdl_entry();
     using V = cplx_t<T>;
@@ -114,6 +114,7 @@ __global__ void __launch_bounds__(1024) k_rows_fwd(const T *__restrict__ in1, co
     const int rows = 1 << lognvec;
     const int vstride = n + (n >> 3);
     const long row0 = (long)blockIdx.x * rows;
+    const uint64_t sd = rotate ? *seed : 0;
     for (int idx = threadIdx.x; idx < rows * n; idx += blockDim.x) {
         const int rr = idx >> logn, x = idx & (n - 1);
         const long grow = row0 + rr;
@@ -124,7 +125,7 @@ __global__ void __launch_bounds__(1024) k_rows_fwd(const T *__restrict__ in1, co
             const long off = b * in_bstride + (long)y * n + x;
             T a = in1[off];
             T c = in2 ? in2[off] : (T)0;
-            if (rotate) rotate_shear(a, c, seed, r0 + b, y, x, n);
+            if (rotate) rotate_shear(a, c, sd, r0 + b, y, x, n);
             val = cmake<V>(a, c);
         }
         buf[rr * vstride + x + (x >> 3)] = val;
@@ -234,7 +235,7 @@ __global__ void __launch_bounds__(1024) k_rows_inv(const cplx_t<T> *__restrict__
 // ---------------------------------------------------------------------------
 template <typename T>
 static int ks_impl(const T *in1, const T *in2, long in_bstride, T *out1, T *out2, cplx_t<T> *work, int n, int batch,
-                   int op, const cplx_t<T> *filt, T out_scale, uint64_t seed, int r0, bool rotate, cudaStream_t s)
+                   int op, const cplx_t<T> *filt, T out_scale, const uint64_t *seed, int r0, bool rotate, cudaStream_t s)
 {
     using V = cplx_t<T>;
     int st = FM_OK;
@@ -278,7 +279,7 @@ static int ks_impl(const T *in1, const T *in2, long in_bstride, T *out1, T *out2
 }
 
 int launch_fft_op(const void *in1, const void *in2, long in_bstride, void *out1, void *out2, void *work, int n,
-                  int batch, int precision, int op, const void *filt, double out_scale, uint64_t rot_seed, int rot_r0,
+                  int batch, int precision, int op, const void *filt, double out_scale, const uint64_t *rot_seed, int rot_r0,
                   bool rotate, cudaStream_t s, bool real_ok)
 {
     if (precision == FM_F64)
@@ -303,7 +304,7 @@ int launch_fft_op(const void *in1, const void *in2, long in_bstride, void *out1,
 }
 
 int launch_ks(const void *in1, const void *in2, long in_bstride, void *out1, void *out2, void *work, int n, int batch,
-              int precision, bool forward, uint64_t rot_seed, int rot_r0, bool rotate, cudaStream_t s, bool batched)
+              int precision, bool forward, const uint64_t *rot_seed, int rot_r0, bool rotate, cudaStream_t s, bool batched)
 {
     return launch_fft_op(in1, in2, in_bstride, out1, out2, work, n, batch, precision,
                          forward ? FFT_OP_KS_FWD : FFT_OP_KS_INV, nullptr, 1.0, rot_seed, rot_r0, rotate, s,

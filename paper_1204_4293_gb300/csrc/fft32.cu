@@ -181,7 +181,7 @@ template <int LOGN, bool SPLIT, bool ROT>
 __global__ void __launch_bounds__(Plan32<LOGN>::ROW_T, Plan32<LOGN>::ROW_MINB)
     k_rows_fwd32(const float *__restrict__ in1, const float *__restrict__ in2,
                                                        long in_bs, float2 *__restrict__ work, long total_rows,
-                                                       const float2 *__restrict__ tw, uint64_t seed, int r0,
+                                                       const float2 *__restrict__ tw, const uint64_t *__restrict__ seed, int r0,
                                                        const __grid_constant__ CUtensorMap m1,
                                                        const __grid_constant__ CUtensorMap m2, int use_tma)
 {
@@ -197,6 +197,8 @@ __global__ void __launch_bounds__(Plan32<LOGN>::ROW_T, Plan32<LOGN>::ROW_MINB)
     const bool live = row < total_rows;
     float2 v[P::E];
     bool staged = false;
+    uint64_t sd = 0;
+    if constexpr (ROT) sd = *seed;
     if constexpr (P::N >= 64) {
         if (use_tma) {
             float *st1 = reinterpret_cast<float *>(smb), *st2 = st1 + RPC * P::N;
@@ -217,7 +219,7 @@ __global__ void __launch_bounds__(Plan32<LOGN>::ROW_T, Plan32<LOGN>::ROW_MINB)
                 const int x = j + r * P::TV;
                 float a = st1[vr * P::N + x];
                 float cc = in2 ? st2[vr * P::N + x] : 0.f;
-                if constexpr (ROT) rotate_shear(a, cc, seed, r0 + b, y, x, P::N);
+                if constexpr (ROT) rotate_shear(a, cc, sd, r0 + b, y, x, P::N);
                 v[r] = make_float2(a, cc);
             }
             staged = true;  // fft_vec's first barrier orders these reads before the exchange writes
@@ -233,7 +235,7 @@ __global__ void __launch_bounds__(Plan32<LOGN>::ROW_T, Plan32<LOGN>::ROW_MINB)
             const int x = j + r * P::TV;
             float a = __ldcs(p1 + x);  // the shear is read once
             float cc = p2 ? __ldcs(p2 + x) : 0.f;
-            if constexpr (ROT) rotate_shear(a, cc, seed, r0 + b, y, x, P::N);
+            if constexpr (ROT) rotate_shear(a, cc, sd, r0 + b, y, x, P::N);
             v[r] = make_float2(a, cc);
         }
     } else if (!staged) {
@@ -643,7 +645,7 @@ bool ks_real_for(int n, bool batched)
 // float2, 16-byte aligned), the complex-to-real row pass in place there.
 template <int LOGN>
 static int ks32_real_impl(const float *in1, const float *in2, long in_bs, float *out1, float2 *work, int batch,
-                          float out_scale, uint64_t seed, int r0, bool rotate, const float2 *tw, const float2 *tw2,
+                          float out_scale, const uint64_t *seed, int r0, bool rotate, const float2 *tw, const float2 *tw2,
                           cudaStream_t s)
 {
     using P = Plan32<LOGN>;
@@ -704,7 +706,7 @@ static int ks32_real_impl(const float *in1, const float *in2, long in_bs, float 
 
 template <int LOGN>
 static int ks32_impl(const float *in1, const float *in2, long in_bs, float *out1, float *out2, float2 *work, int batch,
-                     int op, const float2 *filt, float out_scale, uint64_t seed, int r0, bool rotate,
+                     int op, const float2 *filt, float out_scale, const uint64_t *seed, int r0, bool rotate,
                      const float2 *tw, const float2 *tw2, cudaStream_t s)
 {
     if constexpr (LOGN >= 6) {
@@ -785,7 +787,7 @@ static int ks32_impl(const float *in1, const float *in2, long in_bs, float *out1
 // n = 32 .. 8192 (power of two); other sizes return FM_EINVAL to the caller,
 // which then uses the generic shared-memory Stockham kernels.
 int launch_fft32(const float *in1, const float *in2, long in_bs, float *out1, float *out2, float2 *work, int n,
-                 int batch, int op, const float2 *filt, float out_scale, uint64_t seed, int r0, bool rotate,
+                 int batch, int op, const float2 *filt, float out_scale, const uint64_t *seed, int r0, bool rotate,
                  const float2 *tw, const float2 *tw2, cudaStream_t s)
 {
 #define FM_KS32(L) \
@@ -808,7 +810,7 @@ int launch_fft32(const float *in1, const float *in2, long in_bs, float *out1, fl
 int fft_wait_error(bool clear) { return wait_error_flag(clear); }
 
 int launch_ks32(const float *in1, const float *in2, long in_bs, float *out1, float *out2, float2 *work, int n,
-                int batch, bool forward, uint64_t seed, int r0, bool rotate, const float2 *tw, const float2 *tw2,
+                int batch, bool forward, const uint64_t *seed, int r0, bool rotate, const float2 *tw, const float2 *tw2,
                 cudaStream_t s)
 {
     return launch_fft32(in1, in2, in_bs, out1, out2, work, n, batch, forward ? FFT_OP_KS_FWD : FFT_OP_KS_INV,

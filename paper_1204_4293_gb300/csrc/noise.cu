@@ -5,6 +5,40 @@
 
 namespace fm {
 
+// The inputs of one noise call into the library's buffers: the generator's
+// seed (read there by the row FFT) and, where d1 is given, the two shear maps
+// as `words` vectors V, so that a recorded graph reads neither the caller's
+// pointers nor a seed fixed at its recording.
+template <typename V>
+__global__ void __launch_bounds__(256) k_noise_stage(const V *__restrict__ g1, const V *__restrict__ g2,
+                                                     V *__restrict__ d1, V *__restrict__ d2, long words, uint64_t seed,
+                                                     uint64_t *__restrict__ dseed)
+{
+    pdl_entry();
+    const long i0 = blockIdx.x * (long)blockDim.x + threadIdx.x;
+    if (i0 == 0) *dseed = seed;
+    for (long i = i0; i < words; i += (long)gridDim.x * blockDim.x) {
+        d1[i] = g1[i];
+        d2[i] = g2[i];
+    }
+}
+
+int launch_noise_stage(const void *g1, const void *g2, void *d1, void *d2, size_t bytes, uint64_t seed,
+                       uint64_t *dseed, cudaStream_t s)
+{
+    if (!d1) bytes = 0;
+    const bool wide = ((reinterpret_cast<uintptr_t>(g1) | reinterpret_cast<uintptr_t>(g2) | bytes) & 15) == 0;
+    const long words = (long)(bytes / (wide ? 16 : 4));
+    const unsigned g = (unsigned)(words / 256 + 1 > 152 * 8 ? 152 * 8 : words / 256 + 1);
+    if (wide)
+        FM_LAUNCH(0, k_noise_stage<float4>, g, 256, 0, s, (const float4 *)g1, (const float4 *)g2, (float4 *)d1,
+                  (float4 *)d2, words, seed, dseed);
+    else
+        FM_LAUNCH(0, k_noise_stage<uint32_t>, g, 256, 0, s, (const uint32_t *)g1, (const uint32_t *)g2, (uint32_t *)d1,
+                  (uint32_t *)d2, words, seed, dseed);
+    return FM_OK;
+}
+
 // S1 += sum_b w, S2 += sum_b w^2 over a batch of `nb` (<= 32) realisations'
 // pyramids ([nb][J][n][n], bands 0..J-2 used).  The batch's partial sums are
 // formed in the element type (at most 32 terms) and added once to the FP64
@@ -203,7 +237,7 @@ static int final_launch(const void *acc, const T *wdata, double *var, T *snr, lo
 }
 
 // Bound by HBM: 16 bytes of sums read and 8 (and 4 + 4 for the S/N) written
-// an element.  6 bands of 1024^2 with S/N: 269 -> NOISE_FINAL us (FP64
+// an element.  6 bands of 1024^2 with S/N: 269 -> 42 us (FP64
 // square root, division and comparison before).
 int launch_noise_finalize(const void *acc, const void *wdata, double *var, void *snr, long nelem, int R,
                           int precision, int accum, cudaStream_t s)

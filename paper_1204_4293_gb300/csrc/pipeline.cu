@@ -101,9 +101,10 @@ ChunkPlan plan_chunks(int n, int J, int batch, const fm_config &cfg)
 
 // KS + starlet of maps b0 .. b0 + bc - 1 into their pyramids.  With `rotate`
 // every map of the chunk is the one input map rotated as realisation
-// r0 + (index in the chunk) of the noise generator (seed).
+// r0 + (index in the chunk) of the noise generator (seed in device memory).
 int run_chunk(const char *g1, const char *g2, char *pyr, int n, int J, int b0, int bc, const fm_config &cfg,
-              const ChunkPlan &p, char *slot, cudaStream_t s, bool rotate = false, uint64_t seed = 0, int r0 = 0)
+              const ChunkPlan &p, char *slot, cudaStream_t s, bool rotate = false,
+              const uint64_t *seed = nullptr, int r0 = 0)
 {
     const size_t es = cfg.precision == FM_F64 ? 8 : 4;
     const size_t nn = (size_t)n * n;
@@ -163,6 +164,33 @@ std::vector<GraphEntry> g_graphs;  // guarded by g_ds_mu
 uint64_t g_graph_clock = 0;
 constexpr size_t kMaxGraphs = 4;
 
+// Keys of the last calls that were launched without a graph (guarded by
+// g_ds_mu).  A call is recorded when its key comes back within them: programs
+// that keep their buffers replay from the third call on, and programs with new
+// buffers every call never pay for a recording (2 to 3 ms for 70 kernels, and
+// a device synchronisation once the graph cache is full) that no later call
+// would use.  Launched now, 32 maps of 1024^2 take 570 us, replayed 563.
+GraphKey g_seen[kMaxGraphs];
+size_t g_seen_n = 0;
+bool seen_before(const GraphKey &k)
+{
+    for (size_t i = 0; i < std::min(g_seen_n, kMaxGraphs); ++i)
+        if (g_seen[i] == k) return true;
+    g_seen[g_seen_n++ % kMaxGraphs] = k;
+    return false;
+}
+
+// A call that spreads over the internal streams cannot be part of a capture
+// of the caller's stream.
+int check_not_capturing(cudaStream_t s)
+{
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    FM_CUDA_TRY(cudaStreamIsCapturing(s, &cs));
+    if (cs == cudaStreamCaptureStatusNone) return FM_OK;
+    set_error("a call of several chunks cannot be captured into a graph");
+    return FM_ECUDA;
+}
+
 void drop_graph(GraphEntry &e)
 {
     cudaDeviceSynchronize();  // an evicted graph may still be running
@@ -198,9 +226,15 @@ static int map_starlet_dev(const void *g1, const void *g2, void *pyramid, int n,
     GraphKey key{g1, g2, pyramid, n, J, batch, 0, cfg, p.C, p.slots,
                  g_pdl.load() | ((g_tile_variant.load() + 1) << 1) | (g_use_tma.load() << 3) | (g_wait_test.load() << 10) | ((g_ks_real.load() + 1) << 11)};
     FM_CUDA_TRY(cudaGetDevice(&key.dev));
+    if ((st = check_not_capturing(s))) return st;
     GraphEntry *hit = nullptr;
     for (auto &e : g_graphs)
         if (e.key == key) hit = &e;
+    if (!hit && !seen_before(key)) {
+        Scratch sc;
+        if ((st = scratch_alloc(sc, p.slot_b * p.slots, s))) return st;
+        return run_chunks(g1, g2, pyramid, n, J, batch, cfg, p, (char *)sc.p, s, *ds);
+    }
     if (!hit) {
         if (g_graphs.size() >= kMaxGraphs) {
             auto lru = std::min_element(g_graphs.begin(), g_graphs.end(),
@@ -251,7 +285,8 @@ struct NoiseLayout {
     ChunkPlan p;    // KS + starlet of a batch, chunk by chunk
     int slots = 1;  // chunk slots in use: internal streams, or 1 on the caller's stream
     int pyr_bufs = 1;  // batch pyramid buffers: 2 lets the chunk streams run on during an accumulation
-    size_t acc_b = 0, pyr_b = 0, total = 0;
+    size_t acc_b = 0, pyr_b = 0, total = 0;  // total: + 256 bytes for the seed, at the end
+    size_t seed_off() const { return total - 256; }
 };
 constexpr int kNoisePyrBufs = 2;
 constexpr long kNoisePyrBatchBytes = 8L << 30;  // pyramids of one accumulation batch
@@ -278,24 +313,24 @@ NoiseLayout noise_layout(int n, int J, int R, const fm_config &cfg, bool multi_s
     L.pyr_bufs = L.slots > 1 && R > L.batch ? kNoisePyrBufs : 1;
     L.acc_b = ext_sums ? 0 : up(2 * (size_t)(J - 1) * nn * sizeof(double));
     L.pyr_b = up((size_t)L.batch * J * nn * es);
-    L.total = L.acc_b + (size_t)L.pyr_bufs * L.pyr_b + (size_t)L.slots * L.p.slot_b;
+    L.total = L.acc_b + (size_t)L.pyr_bufs * L.pyr_b + (size_t)L.slots * L.p.slot_b + 256;
     return L;
 }
 
-// Everything of one fm_map_noise call: zero the FP64 sums; every batch of
+// The bands of one fm_map_noise call: zero the FP64 sums; every batch of
 // rotated realisations through KS + starlet, chunk by chunk (over the
 // internal streams when `ds` is given, else on `s`), then S1 += w, S2 += w^2
-// over the batch's pyramids on `s`; the unrotated pass for S/N; the finalize
-// kernel.  With internal streams and more than one batch, two pyramid
-// buffers alternate so that the chunk streams run on into the next batch
-// while `s` accumulates (R = 1000 at 1024^2: 32.2 -> 31.6 ms; the
+// over the batch's pyramids on `s`; with_data: the unrotated pass for S/N into
+// the first pyramid.  With internal streams and more than one batch, two
+// pyramid buffers alternate so that the chunk streams run on into the next
+// batch while `s` accumulates (R = 1000 at 1024^2: 32.2 -> 31.6 ms; the
 // accumulation's pyramid loads are streaming, evict-first: 31.5 ms).
+// The seed is read from scr + L.seed_off() (launch_noise_stage).
 // ext_sums (partial accumulation): the caller's FP64 sums, added to without
-// zeroing and without the S/N pass and finalize; realisations rbase ..
-// rbase + R - 1.
-int noise_submit(const void *g1, const void *g2, double *var_out, void *snr_out, int n, int J, int R, uint64_t seed,
-                 const fm_config &cfg, const NoiseLayout &L, char *scr, cudaStream_t s, DevStreams *ds,
-                 double *ext_sums = nullptr, int rbase = 0)
+// zeroing and without the S/N pass; realisations rbase .. rbase + R - 1.
+int noise_submit(const void *g1, const void *g2, bool with_data, int n, int J, int R, const fm_config &cfg,
+                 const NoiseLayout &L, char *scr, cudaStream_t s, DevStreams *ds, double *ext_sums = nullptr,
+                 int rbase = 0)
 {
     const size_t es = cfg.precision == FM_F64 ? 8 : 4;
     const long nn = (long)n * n;
@@ -305,6 +340,7 @@ int noise_submit(const void *g1, const void *g2, double *var_out, void *snr_out,
     char *pyr = scr + L.acc_b, *slots = pyr + (size_t)L.pyr_bufs * L.pyr_b;
     const ChunkPlan &p = L.p;
     const bool multi = ds && L.slots > 1;
+    const uint64_t *seed = reinterpret_cast<const uint64_t *>(scr + L.seed_off());
     const char *c1 = static_cast<const char *>(g1), *c2 = static_cast<const char *>(g2);
     int r;
     if (!ext_sums) FM_CUDA_TRY(cudaMemsetAsync(acc, 0, (size_t)2 * nb * sizeof(double), s));
@@ -336,30 +372,42 @@ int noise_submit(const void *g1, const void *g2, double *var_out, void *snr_out,
         if ((r = launch_noise_accum(pb, b, (long)J * nn, nn, J - 1, acc, cfg.precision, cfg.accum, s))) return r;
         if (multi && L.pyr_bufs > 1) FM_CUDA_TRY(cudaEventRecord(ds->acc[buf], s));
     }
-    if (ext_sums) return FM_OK;
     // S/N needs the unrotated bands; finalize reads them from the first pyramid
     // (every chunk stream has joined `s` after the last batch)
-    if (snr_out && (r = run_chunk(c1, c2, pyr, n, J, 0, 1, cfg, p, slots, s))) return r;
-    return launch_noise_finalize(acc, snr_out ? pyr : nullptr, var_out, snr_out, nb, R, cfg.precision, cfg.accum, s);
+    if (with_data) return run_chunk(c1, c2, pyr, n, J, 0, 1, cfg, p, slots, s);
+    return FM_OK;
 }
 
+int noise_finish(const NoiseLayout &L, char *scr, double *var_out, void *snr_out, int n, int J, int R,
+                 const fm_config &cfg, cudaStream_t s)
+{
+    return launch_noise_finalize(scr, snr_out ? scr + L.acc_b : nullptr, var_out, snr_out, (long)(J - 1) * n * n, R,
+                                 cfg.precision, cfg.accum, s);
+}
+
+// A recorded noise call: its graph reads the shear and the seed from the
+// copies at the end of its scratch, so one graph serves every call of the
+// shape whatever the buffers and the seed (recorded per pointer and seed, a
+// call with new outputs paid 2.6 ms of recording for 2.5 ms of work at
+// 1024^2, R = 100).  The copy, the replay and the finalize kernel go to the
+// caller's stream; `done` orders a call after the previous use of the scratch
+// on whatever stream that ran.
 struct NoiseKey {
-    const void *g1, *g2, *var, *snr;
     int n, J, R, dev;
-    uint64_t seed;
+    bool with_data;
     fm_config cfg;
     int chunk, slots, pdl;  // the plan and launch mode the graph was recorded with
     bool operator==(const NoiseKey &o) const
     {
-        return g1 == o.g1 && g2 == o.g2 && var == o.var && snr == o.snr && n == o.n && J == o.J && R == o.R &&
-               dev == o.dev && seed == o.seed && memcmp(&cfg, &o.cfg, sizeof(cfg)) == 0 && chunk == o.chunk &&
-               slots == o.slots && pdl == o.pdl;
+        return n == o.n && J == o.J && R == o.R && dev == o.dev && with_data == o.with_data &&
+               memcmp(&cfg, &o.cfg, sizeof(cfg)) == 0 && chunk == o.chunk && slots == o.slots && pdl == o.pdl;
     }
 };
 struct NoiseGraph {
     NoiseKey key;
     cudaGraphExec_t exec = nullptr;
     void *scratch = nullptr;
+    cudaEvent_t done = nullptr;
     uint64_t used = 0;
     int64_t kernels = 0;
 };
@@ -371,15 +419,17 @@ void drop_noise_graph(NoiseGraph &e)
     cudaDeviceSynchronize();
     if (e.exec) cudaGraphExecDestroy(e.exec);
     if (e.scratch) cudaFree(e.scratch);
+    if (e.done) cudaEventDestroy(e.done);
     e.exec = nullptr;
     e.scratch = nullptr;
+    e.done = nullptr;
 }
 
 }  // namespace
 
-// allow_graph: record the whole call once into a CUDA graph (kept with its
-// scratch, LRU of two) and replay it; otherwise launch eagerly with
-// stream-ordered scratch (the serving path, whose buffers change per call).
+// allow_graph: record the realisations of a shape once into a CUDA graph
+// (kept with its scratch, LRU of two) and replay it; otherwise launch eagerly
+// with stream-ordered scratch (the serving path, which bounds its memory).
 int map_noise_run(const void *g1, const void *g2, double *var_out, void *snr_out, int n, int J, int R, uint64_t seed,
                   const fm_config &cfg, cudaStream_t s, bool allow_graph, bool multi_eager)
 {
@@ -393,19 +443,29 @@ int map_noise_run(const void *g1, const void *g2, double *var_out, void *snr_out
         std::lock_guard<std::mutex> lk(g_ds_mu);
         DevStreams *ds = nullptr;
         if ((st = dev_streams(&ds))) return st;
-        return noise_submit(g1, g2, var_out, snr_out, n, J, R, seed, cfg, L, (char *)sc.p, s, ds);
+        char *scr = (char *)sc.p;
+        if ((st = launch_noise_stage(g1, g2, nullptr, nullptr, 0, seed, (uint64_t *)(scr + L.seed_off()), s)) ||
+            (st = noise_submit(g1, g2, snr_out != nullptr, n, J, R, cfg, L, scr, s, ds)))
+            return st;
+        return noise_finish(L, scr, var_out, snr_out, n, J, R, cfg, s);
     }
     if (!allow_graph || g_prof_kid.load() != 0 || !g_use_graphs.load()) {
         const NoiseLayout L = noise_layout(n, J, R, cfg, false);
         Scratch sc;
         if ((st = scratch_alloc(sc, L.total, s))) return st;
-        return noise_submit(g1, g2, var_out, snr_out, n, J, R, seed, cfg, L, (char *)sc.p, s, nullptr);
+        char *scr = (char *)sc.p;
+        if ((st = launch_noise_stage(g1, g2, nullptr, nullptr, 0, seed, (uint64_t *)(scr + L.seed_off()), s)) ||
+            (st = noise_submit(g1, g2, snr_out != nullptr, n, J, R, cfg, L, scr, s, nullptr)))
+            return st;
+        return noise_finish(L, scr, var_out, snr_out, n, J, R, cfg, s);
     }
+    if ((st = check_not_capturing(s))) return st;
     const NoiseLayout L = noise_layout(n, J, R, cfg, true);
     std::lock_guard<std::mutex> lk(g_ds_mu);
     DevStreams *ds = nullptr;
     if ((st = dev_streams(&ds))) return st;
-    NoiseKey key{g1, g2, var_out, snr_out, n, J, R, 0, seed, cfg, L.p.C, L.slots,
+    const size_t in_b = ((size_t)n * n * (cfg.precision == FM_F64 ? 8 : 4) + 255) / 256 * 256;
+    NoiseKey key{n, J, R, 0, snr_out != nullptr, cfg, L.p.C, L.slots,
                  g_pdl.load() | ((g_tile_variant.load() + 1) << 1) | (g_use_tma.load() << 3) | (g_wait_test.load() << 10) | ((g_ks_real.load() + 1) << 11)};
     FM_CUDA_TRY(cudaGetDevice(&key.dev));
     NoiseGraph *hit = nullptr;
@@ -420,7 +480,7 @@ int map_noise_run(const void *g1, const void *g2, double *var_out, void *snr_out
         }
         NoiseGraph e;
         e.key = key;
-        cudaError_t ce = dev_malloc(&e.scratch, L.total);
+        cudaError_t ce = dev_malloc(&e.scratch, L.total + 2 * in_b);
         if (ce != cudaSuccess) return cuda_fail(ce, "cudaMalloc (noise graph scratch)");
         cudaGraph_t graph = nullptr;
         ce = cudaStreamBeginCapture(ds->cap, cudaStreamCaptureModeRelaxed);
@@ -429,7 +489,8 @@ int map_noise_run(const void *g1, const void *g2, double *var_out, void *snr_out
             return cuda_fail(ce, "cudaStreamBeginCapture");
         }
         const int64_t before = g_launches.load();
-        st = noise_submit(g1, g2, var_out, snr_out, n, J, R, seed, cfg, L, (char *)e.scratch, ds->cap, ds);
+        char *scr = (char *)e.scratch;
+        st = noise_submit(scr + L.total, scr + L.total + in_b, key.with_data, n, J, R, cfg, L, scr, ds->cap, ds);
         e.kernels = g_launches.load() - before;
         g_launches.fetch_sub(e.kernels);
         ce = cudaStreamEndCapture(ds->cap, &graph);
@@ -439,6 +500,10 @@ int map_noise_run(const void *g1, const void *g2, double *var_out, void *snr_out
             if (ce != cudaSuccess) st = cuda_fail(ce, "cudaGraphInstantiate");
         }
         if (graph) cudaGraphDestroy(graph);
+        if (st == FM_OK) {
+            ce = cudaEventCreateWithFlags(&e.done, cudaEventDisableTiming);
+            if (ce != cudaSuccess) st = cuda_fail(ce, "cudaEventCreate (noise graph)");
+        }
         if (st != FM_OK) {
             if (e.exec) cudaGraphExecDestroy(e.exec);
             cudaFree(e.scratch);
@@ -448,9 +513,16 @@ int map_noise_run(const void *g1, const void *g2, double *var_out, void *snr_out
         hit = &g_noise_graphs.back();
     }
     hit->used = ++g_graph_clock;
+    char *scr = (char *)hit->scratch;
+    FM_CUDA_TRY(cudaStreamWaitEvent(s, hit->done, 0));  // the scratch's previous use, on any stream
+    if ((st = launch_noise_stage(g1, g2, scr + L.total, scr + L.total + in_b, (size_t)n * n * (cfg.precision == FM_F64 ? 8 : 4),
+                                 seed, (uint64_t *)(scr + L.seed_off()), s)))
+        return st;
     FM_CUDA_TRY(cudaGraphLaunch(hit->exec, s));
     g_launches.fetch_add(hit->kernels);
-    return FM_OK;
+    st = noise_finish(L, scr, var_out, snr_out, n, J, R, cfg, s);
+    FM_CUDA_TRY(cudaEventRecord(hit->done, s));
+    return st;
 }
 
 // Realisations r0 .. r0 + R - 1 added to the caller's FP64 sums, on `s`
@@ -463,14 +535,16 @@ int map_noise_accumulate_run(const void *g1, const void *g2, double *sums, int n
     const NoiseLayout L = noise_layout(n, J, R, cfg, false, true);
     Scratch sc;
     if ((st = scratch_alloc(sc, L.total, s))) return st;
-    return noise_submit(g1, g2, nullptr, nullptr, n, J, R, seed, cfg, L, (char *)sc.p, s, nullptr, sums, r0);
+    char *scr = (char *)sc.p;
+    if ((st = launch_noise_stage(g1, g2, nullptr, nullptr, 0, seed, (uint64_t *)(scr + L.seed_off()), s))) return st;
+    return noise_submit(g1, g2, false, n, J, R, cfg, L, scr, s, nullptr, sums, r0);
 }
 
 // scratch of a noise call on the caller's stream (the serving path)
 size_t noise_scratch_bytes(int n, int J, int R, const fm_config &cfg, bool with_snr, bool multi_stream)
 {
     (void)with_snr;
-    return noise_layout(n, J, R, cfg, multi_stream).total + 256;
+    return noise_layout(n, J, R, cfg, multi_stream).total;  // the seed's 256 bytes among them
 }
 
 int map_starlet_run(const void *g1, const void *g2, void *pyramid, int n, int J, int batch, const fm_config &cfg,
