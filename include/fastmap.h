@@ -349,13 +349,8 @@ int fm_device_error(void);
  *                        (within about 0.1 s), the tile leaves its outputs
  *                        unwritten and fm_device_error reports 1; 0 = off
  *                        (default)
- *   FM_TUNE_DIRECT       kernel of the fp32 direct M_ap without weights:
- *                        0 = scalar FMAs with synchronous row staging,
- *                        1 = packed two-lane FMAs with asynchronous row
- *                        staging, 4 rows x 8 columns per lane, 4 warps;
- *                        2, 3, 4 = the same with 2 x 8 per lane and 4 warps,
- *                        4 x 8 and 2 warps, 2 x 8 and 8 warps; default: 2
- *                        below a 48-pixel cut radius, else 3
+ *   FM_TUNE_DIRECT       accepted (0 .. 4) and without effect: the direct M_ap
+ *                        has one kernel form
  *   FM_TUNE_KS_REAL      inverse KS without kappa_B: 1 = compute only the
  *                        Hermitian half of kappa_E's spectrum (real-output
  *                        column and row passes; fp32, n >= 64, kappa_E

@@ -5,40 +5,60 @@
 // M(x) = sum_{0 < |d| <= R} Q(|d|) gamma_t(x + d; x),
 // gamma_t = -(gamma1 cos 2 phi_d + gamma2 sin 2 phi_d), so with per-offset
 // weights A(d) = -Q cos 2 phi = -Q (dx^2 - dy^2) / |d|^2 and
-// B(d) = -Q sin 2 phi = -Q 2 dx dy / |d|^2 (built on the host in FP64) the map
-// is the 2-D correlation M = A * gamma1 + B * gamma2, zero outside the field.
+// B(d) = -Q sin 2 phi = -Q 2 dx dy / |d|^2 (FP64, rounded once) the map is the
+// 2-D correlation M = A * gamma1 + B * gamma2, zero outside the field.
 //
-// Kernel layout: a CTA owns TY = NW*RY output rows x TX = 32*CX columns; warp
-// w owns RY rows, lane l owns CX adjacent columns.  The CTA walks the input
-// rows iy covering its rows +- R; each input row (both components, halo R)
-// is staged once in shared memory and serves every output row within R of
-// it: output row y uses it with the weight row dy = iy - y.  Within a warp
-// all lanes share the output rows, so the dy tests and dx loop bounds are
-// warp-uniform, and weights are warp-wide broadcast loads.  The staged row
-// is stored with one pad slot per 8 so that the lanes' 8-column windows hit
-// distinct banks.  FP32 cores (FFMA), no tensor cores: not a contraction the
-// tensor cores can take at this precision.
+// A(dx, -dy) = A(dx, dy) and B(dx, -dy) = -B(dx, dy), so the rows y + dy and
+// y - dy enter together: with s = gamma1(y + dy) + gamma1(y - dy) and
+// d = gamma2(y + dy) - gamma2(y - dy),
+//   M(x, y) = sum_{dy >= 0} sum_dx A(dx, dy) s(x + dx) + B(dx, dy) d(x + dx),
+// half the multiplications of the plain sum.
+//
+// Kernel layout: one warp owns one output row of 32 CX columns (CX adjacent
+// ones a lane) and shares nothing with the others.  For each dy it forms the
+// folded row (s, d) in its own piece of shared memory, as blocks of CX
+// columns padded by 16 bytes (the lanes' 16-byte loads of CX neighbouring
+// blocks then hit distinct banks), and walks dx in groups of CX taps: a lane
+// keeps two blocks in registers, loads one more per group and spends CX^2
+// packed two-lane FMAs (fma.rn.f32x2: A s and B d in one instruction) on it.
+// The groups at the rim of the disc skip the taps outside it, so a pixel
+// beyond the radius never meets a weight.  Sums are two-level (a dy's taps,
+// then the total).  With few rows the dy are dealt out to P warps (dy = p,
+// p + P, ...: equal shares) whose sums k_direct_sum adds in order.
+//
+// What bounds it: the FP32 pipe and the shared-memory loads together (1024^2,
+// R = 32: 52.7 M warp FMAs of two lanes, 84 us at two a cycle and SM; ncu: FMA
+// pipe 56 %, shared-memory and L1 data path 69 %, 20 warps an SM).  One 1024^2
+// map, starlet Q theta = 16 (R = 32): 372 -> 209 us; S98 theta = 64 1246 ->
+// 658, masked 3050 -> 866; masked 2 x 1000^2 S98 theta = 16 445 -> 236; fp64
+// 512^2 S98 theta = 16 3079 -> 472 (the plain sum over all rows, with a CTA's
+// warps sharing each staged row behind a barrier).  16 columns a lane halve
+// the window loads but need 116 to 142 registers: 225 us; groups of four taps
+// instead of eight 260 us.
 //
 // Missing data (Sec. 4.3, Sec. 4.5): with pixel weights w >= 0 (0 = masked)
-// the same pass also forms D(x) = sum w(x+d) over the in-field offsets
-// 0 < |d| <= R (a third staged component and a 0/1 disc table), stages
-// w gamma1, w gamma2 instead of the shear, and writes
-// M = N_R S / D (0 where D <= 0) and optionally coverage = D / N_R, N_R the
+// the folded row is that of w gamma, and the same pass forms D(x) = sum
+// w(x+d) over the in-field offsets 0 < |d| <= R.  D needs no multiplication:
+// a lane's CX windows of one dy share all but CX - 1 columns at each end, so
+// it adds the common part once (whole blocks from their sums) and the ends as
+// running sums; additions of weights only, no differences.  The result is
+// M = N_R S / D (0 where D <= 0), optionally coverage = D / N_R, N_R the
 // aperture's pixel count.
 #include <math.h>
 
+#include <algorithm>
 #include <atomic>
-#include <vector>
+#include <type_traits>
 
 #include "common.cuh"
 
 namespace fm {
 
-// ---- filters (Sec. 4), FP64 on the host --------------------------------------
-static double cube(double v) { return v * v * v; }
+// ---- filters (Sec. 4), FP64 ----------------------------------------------------
+__device__ static double cube(double v) { return v * v * v; }
 
 // starlet Q(eta) printed in Sec. 4.2; the direct sum never evaluates eta = 0.
-static double q_starlet(double e)
+__device__ static double q_starlet(double e)
 {
     const double e2 = e * e;
     double s = -279.0 * e2 * cube(fabs(e));
@@ -51,7 +71,7 @@ static double q_starlet(double e)
     return s / (45.0 * e2);
 }
 
-static double q_of(int filter, double v, double theta, int ell)
+__device__ static double q_of(int filter, double v, double theta, int ell)
 {
     const double t2 = theta * theta;
     switch (filter) {
@@ -59,7 +79,10 @@ static double q_of(int filter, double v, double theta, int ell)
     case FM_FILTER_S98: {  // eq. sch
         if (v > theta) return 0.0;
         const double x2 = v * v / t2;
-        return (1.0 + ell) * (2.0 + ell) / (M_PI * t2) * x2 * pow(1.0 - x2, (double)ell);
+        double pw = 1.0, base = 1.0 - x2;
+        for (int k = ell; k > 0; k >>= 1, base *= base)
+            if (k & 1) pw *= base;
+        return (1.0 + ell) * (2.0 + ell) / (M_PI * t2) * x2 * pw;
     }
     case FM_FILTER_JBJ04:
     case FM_FILTER_VW98: {  // eq. mexhat with A = 1
@@ -73,465 +96,452 @@ static double q_of(int filter, double v, double theta, int ell)
 
 static double default_cut(int filter) { return filter == FM_FILTER_STARLET ? 2.0 : filter == FM_FILTER_S98 ? 1.0 : 5.0; }
 
-// ---- kernel -------------------------------------------------------------------
-__device__ __forceinline__ int padc(int c) { return c + (c >> 3); }
-__device__ __forceinline__ uint32_t smem_u32_md(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
+// largest dx with dx^2 + dy^2 <= R^2 (dy <= R)
+__host__ __device__ static int disc_half_width(int dy, double R2)
+{
+    int dx = (int)sqrt(R2 - (double)dy * dy > 0 ? R2 - (double)dy * dy : 0.0);
+    while (((double)(dx + 1) * (dx + 1)) + (double)dy * dy <= R2) ++dx;
+    while (dx > 0 && (double)dx * dx + (double)dy * dy > R2) --dx;
+    return dx;
+}
 
-template <typename T, int CX, int RY, int NW, bool MASK>
-__global__ void __launch_bounds__(NW * 32) k_map_direct(const T *__restrict__ g1, const T *__restrict__ g2,
-                                                        const T *__restrict__ wgt, long w_bs,
-                                                        const cplx_t<T> *__restrict__ taps,
-                                                        const T *__restrict__ disc, int tw,
-                                                        const int *__restrict__ dxmax, T *__restrict__ out,
-                                                        T *__restrict__ cov, int n, int Ri, T n_r)
+// columns a lane owns, and the folded row's layout in shared memory
+template <typename T> struct DirectRow {
+    using V = cplx_t<T>;
+    static constexpr int CX = sizeof(T) == 4 ? 8 : 4;
+    static constexpr int TX = 32 * CX;
+    static constexpr int BS = CX + 16 / (int)sizeof(V);  // elements of a padded block: 80 bytes
+    // radius rounded up to whole blocks, blocks of a row, taps of a table row
+    static int rp(int Ri) { return (Ri + CX - 1) / CX * CX; }
+    static int blocks(int Ri) { return 32 + 2 * rp(Ri) / CX + 1; }
+    static int tap_width(int Ri) { return 2 * rp(Ri) + CX; }
+    // shared memory of a warp: (s, d); weights: w folded (blocks of CX + 1) and its block sums
+    static size_t bytes(int Ri, bool mask)
+    {
+        const size_t nb = blocks(Ri);
+        const size_t b = nb * BS * sizeof(V) + (mask ? nb * (CX + 2) * sizeof(T) : 0);
+        return (b + 15) / 16 * 16;
+    }
+};
+
+// Weights (A, B) of the rows dy = 0 .. Ri (the others follow by symmetry),
+// dx = -rp .. rp + CX - 1, zero outside 0 < |d| <= R; and each row's half width.
+// On the device: no copy from host memory, so a call can be captured, and the
+// host's share of a call no longer grows with R^2 (0.1 ms at R = 32).
+template <typename T>
+__global__ void __launch_bounds__(64) k_direct_taps(cplx_t<T> *__restrict__ taps, int *__restrict__ dxmax, int Ri,
+                                                    int rp, int tw, double R2, int filter, double theta, int ell)
+{
+    pdl_entry();
+    const int dy = blockIdx.y, dx = blockIdx.x * blockDim.x + threadIdx.x;
+    cplx_t<T> *row = taps + (long)dy * tw + rp;
+    if (dx == 0) dxmax[dy] = disc_half_width(dy, R2);
+    if (dx >= tw - rp) return;
+    const double r2 = (double)dx * dx + (double)dy * dy;
+    double a = 0, b = 0;
+    if (r2 > 0 && r2 <= R2) {
+        const double q = q_of(filter, sqrt(r2), theta, ell);
+        a = -q * ((double)dx * dx - (double)dy * dy) / r2;
+        b = -q * 2.0 * dx * dy / r2;
+    }
+    row[dx] = cmake<cplx_t<T>>((T)a, (T)b);
+    if (dx > 0 && dx <= rp) row[-dx] = cmake<cplx_t<T>>((T)a, (T)-b);
+}
+
+__device__ __forceinline__ void tap_fma(float2 &acc, float2 ab, float2 w) { acc = __ffma2_rn(ab, w, acc); }
+__device__ __forceinline__ void tap_fma(double2 &acc, double2 ab, double2 w)
+{
+    acc.x = fma(ab.x, w.x, acc.x);
+    acc.y = fma(ab.y, w.y, acc.y);
+}
+// a block of CX columns of the folded row (16-byte loads)
+template <typename V, int CX> __device__ __forceinline__ void load_block(V (&w)[CX], const V *p)
+{
+#pragma unroll
+    for (int k = 0; k < CX; k += 16 / (int)sizeof(V)) {
+        if constexpr (sizeof(V) == 8) {
+            const float4 q = *reinterpret_cast<const float4 *>(p + k);
+            w[k] = make_float2(q.x, q.y);
+            w[k + 1] = make_float2(q.z, q.w);
+        } else {
+            w[k] = p[k];
+        }
+    }
+}
+
+// CX taps of a table row (16-byte aligned: rows hold 2 rp + CX taps)
+template <typename V, int CX> __device__ __forceinline__ void load_taps(V (&ab)[CX], const V *p)
+{
+    if constexpr (sizeof(V) == 8) {
+#pragma unroll
+        for (int k = 0; k < CX; k += 2) {
+            const float4 q = __ldg(reinterpret_cast<const float4 *>(p + k));
+            ab[k] = make_float2(q.x, q.y);
+            ab[k + 1] = make_float2(q.z, q.w);
+        }
+    } else {
+#pragma unroll
+        for (int k = 0; k < CX; ++k) ab[k] = __ldg(p + k);
+    }
+}
+
+// grid = (ceil(n / warps), ceil(n / TX), maps * P), one output row a warp.
+// P = 1: writes out (and cov); P > 1: the part's sums to parts[p][map] and,
+// MASK, partw[p][map].
+template <typename T, bool MASK>
+__global__ void __launch_bounds__(128, sizeof(T) == 4 ? 5 : 3)
+    k_map_direct(const T *__restrict__ g1, const T *__restrict__ g2, const T *__restrict__ wgt, long w_bs,
+                 const cplx_t<T> *__restrict__ taps, const int *__restrict__ dxmax, T *__restrict__ out,
+                 T *__restrict__ cov, T *__restrict__ parts, T *__restrict__ partw, int n, int Ri, int rp, int nblocks,
+                 int warp_bytes, int P, int maps, T n_r)
 {
     pdl_entry();
     using V = cplx_t<T>;
-    constexpr int TX = 32 * CX, TY = NW * RY;
-    constexpr int NC = MASK ? 3 : 2;  // staged components
+    using D = DirectRow<T>;
+    constexpr int CX = D::CX, BS = D::BS;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int width = TX + 2 * Ri + 8;
-    const int pw = padc(width) + 1;
-    T *s1 = reinterpret_cast<T *>(smem_raw);  // [2 buffers][NC comps][pw]
-    const int x0 = blockIdx.x * TX, y0 = blockIdx.y * TY;
-    const long nn = (long)n * n;
-    const long b = blockIdx.z;
-    g1 += b * nn;
-    g2 += b * nn;
-    out += b * nn;
-    if (MASK) {
-        wgt += b * w_bs;
-        if (cov) cov += b * nn;
-    }
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int yw = y0 + warp * RY;
-    const int lc = lane * CX;
-
-    T acc[RY][CX], accw[MASK ? RY : 1][CX];
-#pragma unroll
-    for (int k = 0; k < RY; ++k)
-#pragma unroll
-        for (int o = 0; o < CX; ++o) {
-            acc[k][o] = (T)0;
-            if (MASK) accw[k][o] = (T)0;
-        }
-
-    const int iy_lo = y0 - Ri, iy_hi = y0 + TY - 1 + Ri;
-    for (int iy = iy_lo; iy <= iy_hi; ++iy) {
-        T *buf = s1 + ((iy - iy_lo) & 1) * NC * pw;
-        const bool rin = iy >= 0 && iy < n;
-        for (int c = threadIdx.x; c < width; c += blockDim.x) {
-            const int gx = x0 - Ri + c;
-            T a = (T)0, bb = (T)0, ww = (T)0;
-            if (rin && gx >= 0 && gx < n) {
-                a = g1[(long)iy * n + gx];
-                bb = g2[(long)iy * n + gx];
-                if (MASK) {
-                    ww = wgt[(long)iy * n + gx];
-                    a *= ww;
-                    bb *= ww;
-                }
-            }
-            buf[padc(c)] = a;
-            buf[pw + padc(c)] = bb;
-            if (MASK) buf[2 * pw + padc(c)] = ww;
-        }
-        __syncthreads();
-
-        int dy[RY];
-        bool act[RY];
-        int dxm = -1;
-#pragma unroll
-        for (int k = 0; k < RY; ++k) {
-            dy[k] = iy - (yw + k);
-            act[k] = dy[k] >= -Ri && dy[k] <= Ri && (yw + k) < n;
-            if (act[k]) {
-                const int m = __ldg(dxmax + dy[k] + Ri);
-                dxm = m > dxm ? m : dxm;
-            }
-        }
-        if (dxm >= 0) {
-            // two-level sum: this input row's taps first, then into the total
-            T part[RY][CX], partw[MASK ? RY : 1][CX];
-#pragma unroll
-            for (int k = 0; k < RY; ++k)
-#pragma unroll
-                for (int o = 0; o < CX; ++o) {
-                    part[k][o] = (T)0;
-                    if (MASK) partw[k][o] = (T)0;
-                }
-            for (int dx0 = -dxm; dx0 <= dxm; dx0 += 8) {
-                T w1[CX + 7], w2[CX + 7], w3[MASK ? CX + 7 : 1];
-                const int base = lc + dx0 + Ri;
-#pragma unroll
-                for (int q = 0; q < CX + 7; ++q) {
-                    w1[q] = buf[padc(base + q)];
-                    w2[q] = buf[pw + padc(base + q)];
-                    if (MASK) w3[q] = buf[2 * pw + padc(base + q)];
-                }
-#pragma unroll
-                for (int k = 0; k < RY; ++k) {
-                    if (!act[k]) continue;
-                    const long toff = (long)(dy[k] + Ri) * tw + (dx0 + Ri);
-                    const V *trow = taps + toff;
-#pragma unroll
-                    for (int t = 0; t < 8; ++t) {
-                        const V ab = __ldg(trow + t);
-#pragma unroll
-                        for (int o = 0; o < CX; ++o) {
-                            part[k][o] = fma(ab.x, w1[o + t], part[k][o]);
-                            part[k][o] = fma(ab.y, w2[o + t], part[k][o]);
-                        }
-                        if (MASK) {
-                            const T in_disc = __ldg(disc + toff + t);
-#pragma unroll
-                            for (int o = 0; o < CX; ++o) partw[k][o] = fma(in_disc, w3[o + t], partw[k][o]);
-                        }
-                    }
-                }
-            }
-#pragma unroll
-            for (int k = 0; k < RY; ++k)
-#pragma unroll
-                for (int o = 0; o < CX; ++o) {
-                    acc[k][o] += part[k][o];
-                    if (MASK) accw[k][o] += partw[k][o];
-                }
-        }
-    }
-#pragma unroll
-    for (int k = 0; k < RY; ++k) {
-        const int y = yw + k;
-        if (y >= n) continue;
-#pragma unroll
-        for (int o = 0; o < CX; ++o) {
-            const int x = x0 + lc + o;
-            if (x >= n) continue;
-            if (MASK) {
-                const T d = accw[k][o];
-                out[(long)y * n + x] = d > (T)0 ? n_r * acc[k][o] / d : (T)0;
-                if (cov) cov[(long)y * n + x] = d / n_r;
-            } else {
-                out[(long)y * n + x] = acc[k][o];
-            }
-        }
-    }
-}
-
-// ---- fp32 form without weights ------------------------------------------------
-// The same walk over input rows with two changes: the next input row arrives
-// by asynchronous 4-byte copies (cp.async, zero-filled outside the field)
-// into the other buffer while the CTA works on the current one, so the
-// global-memory latency of the staging is hidden; and the two components are
-// staged interleaved, (gamma1, gamma2) per column, so that one packed
-// two-lane FMA (fma.rn.f32x2) per tap adds A gamma1 into lane x and
-// B gamma2 into lane y of a partial sum; the lanes are added when the input
-// row is done.  Half the FMA instructions of the scalar form.
-__device__ __forceinline__ void cp_async4(void *dst, const void *src, int src_bytes)
-{
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(smem_u32_md(dst)), "l"(src), "r"(src_bytes)
-                 : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
-
-//
-// With P > 1 the input rows a tile needs (TY + 2R of them) are split into P
-// consecutive parts, one CTA each (blockIdx.z = b P + p), so that a single
-// map with a large radius still gives the GPU several waves of CTAs; part p
-// writes its sums to part_out[p][b] and k_sum_parts adds the parts in order
-// (the same order whatever the batch, so a map's result does not depend on
-// the maps beside it).
-template <int CX, int RY, int NW>
-__global__ void __launch_bounds__(NW * 32) k_map_direct_f2(const float *__restrict__ g1, const float *__restrict__ g2,
-                                                           const float2 *__restrict__ taps, int tw,
-                                                           const int *__restrict__ dxmax, float *__restrict__ out,
-                                                           int n, int Ri, int P, int batch)
-{
-    pdl_entry();
-    constexpr int TX = 32 * CX, TY = NW * RY;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int width = TX + 2 * Ri + 8;
-    const int pw = padc(width) + 1;
-    float2 *s2 = reinterpret_cast<float2 *>(smem_raw);  // [2 buffers][pw] of (gamma1, gamma2)
-    const int x0 = blockIdx.x * TX, y0 = blockIdx.y * TY;
-    const long nn = (long)n * n;
-    const long b = blockIdx.z / P;
+    const int y = blockIdx.x * (blockDim.x >> 5) + warp;
+    if (y >= n) return;  // warps share nothing
+    V *buf = reinterpret_cast<V *>(smem_raw + (size_t)warp * warp_bytes);
+    T *sw = reinterpret_cast<T *>(buf + nblocks * BS);  // folded weights, CX + 1 a block
+    T *sb = sw + nblocks * (CX + 1);                    // their block sums
+    const int x0 = blockIdx.y * D::TX;
+    const long nn = (long)n * n, b = blockIdx.z / P;
     const int p = blockIdx.z % P;
     g1 += b * nn;
     g2 += b * nn;
-    out += ((long)p * batch + b) * nn;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int yw = y0 + warp * RY;
-    const int lc = lane * CX;
-    const int rows = TY + 2 * Ri, chunk = (rows + P - 1) / P;
-    const int iy_lo = y0 - Ri + p * chunk;
-    const int iy_end = y0 + TY - 1 + Ri;
-    const int iy_hi = iy_lo + chunk - 1 < iy_end ? iy_lo + chunk - 1 : iy_end;
+    if (MASK) wgt += b * w_bs;
+    const int tw = 2 * rp + CX;
 
-    auto stage = [&](int iy) {  // this thread's copies of input row iy into its buffer
-        float *buf = reinterpret_cast<float *>(s2 + ((iy - iy_lo) & 1) * pw);
-        const bool rin = iy >= 0 && iy < n;
-        for (int c = threadIdx.x; c < width; c += NW * 32) {
-            const int gx = x0 - Ri + c;
-            const bool in = rin && gx >= 0 && gx < n;
-            const long off = in ? (long)iy * n + gx : 0;
-            cp_async4(buf + 2 * padc(c), g1 + off, in ? 4 : 0);
-            cp_async4(buf + 2 * padc(c) + 1, g2 + off, in ? 4 : 0);
-        }
-        cp_async_commit();
-    };
-
-    float acc[RY][CX];
+    T acc[CX], accw[MASK ? CX : 1];
 #pragma unroll
-    for (int k = 0; k < RY; ++k)
-#pragma unroll
-        for (int o = 0; o < CX; ++o) acc[k][o] = 0.f;
-
-    if (iy_lo <= iy_hi) stage(iy_lo);
-    for (int iy = iy_lo; iy <= iy_hi; ++iy) {
-        cp_async_wait_all();  // this thread's copies of row iy have landed
-        __syncthreads();      // everyone's have; the other buffer is no longer read
-        if (iy < iy_hi) stage(iy + 1);
-        const float2 *buf = s2 + ((iy - iy_lo) & 1) * pw;
-
-        int dy[RY];
-        bool act[RY];
-        int dxm = -1;
-#pragma unroll
-        for (int k = 0; k < RY; ++k) {
-            dy[k] = iy - (yw + k);
-            act[k] = dy[k] >= -Ri && dy[k] <= Ri && (yw + k) < n;
-            if (act[k]) {
-                const int m = __ldg(dxmax + dy[k] + Ri);
-                dxm = m > dxm ? m : dxm;
-            }
-        }
-        if (dxm < 0) continue;
-        float2 part[RY][CX];
-#pragma unroll
-        for (int k = 0; k < RY; ++k)
-#pragma unroll
-            for (int o = 0; o < CX; ++o) part[k][o] = make_float2(0.f, 0.f);
-        for (int dx0 = -dxm; dx0 <= dxm; dx0 += 8) {
-            float2 w[CX + 7];
-            const int base = lc + dx0 + Ri;
-#pragma unroll
-            for (int q = 0; q < CX + 7; ++q) w[q] = buf[padc(base + q)];
-#pragma unroll
-            for (int k = 0; k < RY; ++k) {
-                if (!act[k]) continue;
-                const float2 *trow = taps + (long)(dy[k] + Ri) * tw + (dx0 + Ri);
-#pragma unroll
-                for (int t = 0; t < 8; ++t) {
-                    const float2 ab = __ldg(trow + t);
-#pragma unroll
-                    for (int o = 0; o < CX; ++o) part[k][o] = __ffma2_rn(ab, w[o + t], part[k][o]);
-                }
-            }
-        }
-#pragma unroll
-        for (int k = 0; k < RY; ++k)
-#pragma unroll
-            for (int o = 0; o < CX; ++o) acc[k][o] += part[k][o].x + part[k][o].y;
+    for (int o = 0; o < CX; ++o) {
+        acc[o] = (T)0;
+        if (MASK) accw[o] = (T)0;
     }
+    for (int dy = p; dy <= Ri; dy += P) {
+        const bool up = y + dy < n, dn = dy > 0 && y - dy >= 0;
+        if (!up && !dn) break;  // larger dy leave the field too
+        const int dxm = __ldg(dxmax + dy);
+        const int glo = (rp - dxm) / CX, ghi = (rp + dxm) / CX;  // groups of taps that meet the disc
+        // the folded row, columns of the blocks glo .. 32 + ghi: rows and
+        // addresses are fixed before the loop, whose body is loads, the fold
+        // and stores at compile-time offsets
+        const int c0 = glo * CX + lane, c_end = (33 + ghi) * CX;
+        const int gx0 = x0 - rp + c0;
+        __syncwarp();  // the last dy's reads
+        auto fold = [&](auto up_, auto dn_, auto edge_) {
+            constexpr bool UP = decltype(up_)::value, DN = decltype(dn_)::value, EDGE = decltype(edge_)::value;
+            const long iu = (long)(y + dy) * n + gx0, id = (long)(y - dy) * n + gx0;
+            const T *u1 = g1 + iu, *u2 = g2 + iu, *d1 = g1 + id, *d2 = g2 + id;
+            [[maybe_unused]] const T *uw = MASK ? wgt + iu : nullptr, *dw = MASK ? wgt + id : nullptr;
+            V *dst = buf + c0 / CX * BS + c0 % CX;
+            [[maybe_unused]] T *dsw = sw + c0 / CX * (CX + 1) + c0 % CX, *dsb = sb + c0 / CX;
+            int gx = gx0, left = c_end - c0;
+#pragma unroll 4
+            for (int t = (c_end - glo * CX + 31) / 32; t > 0; --t) {
+                T a = (T)0, d = (T)0;
+                [[maybe_unused]] T w = (T)0;
+                if (!EDGE || (unsigned)gx < (unsigned)n) {
+                    if constexpr (UP) {
+                        a = __ldg(u1);
+                        d = __ldg(u2);
+                        if constexpr (MASK) {
+                            w = __ldg(uw);
+                            a *= w;
+                            d *= w;
+                        }
+                    }
+                    if constexpr (DN) {
+                        T a2 = __ldg(d1), e2 = __ldg(d2);
+                        if constexpr (MASK) {
+                            const T w2 = __ldg(dw);
+                            a2 *= w2;
+                            e2 *= w2;
+                            w += w2;
+                        }
+                        a += a2;
+                        d -= e2;
+                    }
+                }
+                if (left > 0) *dst = cmake<V>(a, d);
+                if constexpr (MASK) {
+                    if (left > 0) *dsw = w;
 #pragma unroll
-    for (int k = 0; k < RY; ++k) {
-        const int y = yw + k;
-        if (y >= n) continue;
+                    for (int o = 1; o < CX; o *= 2) w += __shfl_xor_sync(0xffffffffu, w, o);
+                    if (lane % CX == 0 && left > 0) *dsb = w;
+                    uw += 32;
+                    dw += 32;
+                    dsw += 32 / CX * (CX + 1);
+                    dsb += 32 / CX;
+                }
+                u1 += 32;
+                u2 += 32;
+                d1 += 32;
+                d2 += 32;
+                dst += 32 / CX * BS;
+                gx += 32;
+                left -= 32;
+            }
+        };
+        // columns past c_end (the last 32 of a row may overhang it) are loaded
+        // but not stored: they count for the field's edge as well
+        const int cl = (c_end - glo * CX + 31) / 32 * 32;
+        const bool edge = x0 - rp + glo * CX < 0 || x0 - rp + glo * CX + cl > n;
+        using Yes = std::true_type;
+        using No = std::false_type;
+        if (up && dn) {
+            if (edge)
+                fold(Yes(), Yes(), Yes());
+            else
+                fold(Yes(), Yes(), No());
+        } else if (up) {
+            fold(Yes(), No(), Yes());
+        } else {
+            fold(No(), Yes(), Yes());
+        }
+        __syncwarp();
+        V part[CX];
 #pragma unroll
-        for (int o = 0; o < CX; ++o) {
-            const int x = x0 + lc + o;
-            if (x < n) out[(long)y * n + x] = acc[k][o];
+        for (int o = 0; o < CX; ++o) part[o] = cmake<V>((T)0, (T)0);
+        const V *trow = taps + (long)dy * tw, *src = buf + lane * BS;
+        // taps g CX .. g CX + CX - 1 over the columns in a (block lane + g) and b (the next):
+        // all of them, or at the rim those of the disc
+        auto full = [&](int g, const V (&a)[CX], const V (&b)[CX]) {
+            V ab[CX];
+            load_taps<V, CX>(ab, trow + g * CX);
+#pragma unroll
+            for (int k = 0; k < CX; ++k)
+#pragma unroll
+                for (int o = 0; o < CX; ++o) tap_fma(part[o], ab[k], o + k < CX ? a[o + k] : b[o + k - CX]);
+        };
+        auto rim = [&](int g, const V (&a)[CX], const V (&b)[CX]) {
+            const int lo = rp - dxm - g * CX, hi = rp + dxm - g * CX;
+            V ab[CX];
+            load_taps<V, CX>(ab, trow + g * CX);
+#pragma unroll
+            for (int k = 0; k < CX; ++k)
+                if (k >= lo && k <= hi) {
+#pragma unroll
+                    for (int o = 0; o < CX; ++o) tap_fma(part[o], ab[k], o + k < CX ? a[o + k] : b[o + k - CX]);
+                }
+        };
+        V wa[CX], wb[CX];
+        load_block<V, CX>(wa, src + glo * BS);
+        load_block<V, CX>(wb, src + (glo + 1) * BS);
+        rim(glo, wa, wb);
+        int g = glo + 1;  // wb holds block lane + g
+        for (; g + 1 < ghi; g += 2) {
+            load_block<V, CX>(wa, src + (g + 1) * BS);
+            full(g, wb, wa);
+            load_block<V, CX>(wb, src + (g + 2) * BS);
+            full(g + 1, wa, wb);
+        }
+        if (g < ghi) {
+            load_block<V, CX>(wa, src + (g + 1) * BS);
+            full(g, wb, wa);
+#pragma unroll
+            for (int k = 0; k < CX; ++k) wb[k] = wa[k];
+        }
+        if (ghi > glo) {
+            load_block<V, CX>(wa, src + (ghi + 1) * BS);
+            rim(ghi, wb, wa);
+        }
+#pragma unroll
+        for (int o = 0; o < CX; ++o) acc[o] += part[o].x + part[o].y;
+        if constexpr (MASK) {
+            // this dy's weights within |dx| <= dxm of each of the lane's columns
+            // (dx = 0 left out at dy = 0); column c from the lane's first one
+            const T *ws = sw + lane * (CX + 1);
+            auto at = [&](int c) { return ws[rp + c + (rp + c) / CX]; };
+            if (dxm < CX - 1) {
+#pragma unroll
+                for (int o = 0; o < CX; ++o) {
+                    T t = (T)0;
+                    for (int dx = -dxm; dx <= dxm; ++dx)
+                        if (dx != 0 || dy != 0) t += at(o + dx);
+                    accw[o] += t;
+                }
+            } else {
+                // columns lo .. hi, whole blocks by their sums
+                auto span = [&](int lo, int hi) {
+                    T t = (T)0;
+                    int u = rp + lo;
+                    const int e = rp + hi + 1;  // blocks count from -rp
+                    for (; u < e && u % CX != 0; ++u) t += ws[u + u / CX];
+                    for (; u + CX <= e; u += CX) t += sb[lane + u / CX];
+                    for (; u < e; ++u) t += ws[u + u / CX];
+                    return t;
+                };
+                T mid[CX];
+                if (dy == 0) {
+                    const T common = span(CX - 1 - dxm, -1) + span(CX, dxm);
+                    T run = (T)0;
+#pragma unroll
+                    for (int o = 0; o < CX; ++o) {  // own column left out: those before it, then those after it
+                        mid[o] = common + run;
+                        run += at(o);
+                    }
+                    run = (T)0;
+#pragma unroll
+                    for (int o = CX - 1; o >= 0; --o) {
+                        mid[o] += run;
+                        run += at(o);
+                    }
+                } else {
+                    const T common = span(CX - 1 - dxm, dxm);
+#pragma unroll
+                    for (int o = 0; o < CX; ++o) mid[o] = common;
+                }
+                T left = (T)0, right = (T)0;
+#pragma unroll
+                for (int o = CX - 2; o >= 0; --o) {
+                    left += at(o - dxm);
+                    mid[o] += left;
+                }
+#pragma unroll
+                for (int o = 1; o < CX; ++o) {
+                    right += at(o + dxm);
+                    mid[o] += right;
+                }
+#pragma unroll
+                for (int o = 0; o < CX; ++o) accw[o] += mid[o];
+            }
+        }
+    }
+    const long row = (P > 1 ? (long)p * maps + b : b) * nn + (long)y * n;
+#pragma unroll
+    for (int o = 0; o < CX; ++o) {
+        const int x = x0 + lane * CX + o;
+        if (x >= n) continue;
+        if (P > 1) {
+            parts[row + x] = acc[o];
+            if (MASK) partw[row + x] = accw[o];
+        } else if constexpr (MASK) {
+            const T d = accw[o];
+            out[row + x] = d > (T)0 ? n_r * acc[o] / d : (T)0;
+            if (cov) cov[row + x] = d / n_r;
+        } else {
+            out[row + x] = acc[o];
         }
     }
 }
 
-// out[i] = sum over p of part[p][i], p in order (float4 where the size allows)
-__global__ void k_sum_parts(const float *__restrict__ part, float *__restrict__ out, long total, int P)
+// the parts' sums in order, p = 0 .. P - 1, over `total` pixels
+template <typename T, bool MASK>
+__global__ void __launch_bounds__(256) k_direct_sum(const T *__restrict__ parts, const T *__restrict__ partw,
+                                                    T *__restrict__ out, T *__restrict__ cov, long total, int P,
+                                                    T n_r)
 {
     pdl_entry();
-    const long i4 = ((long)blockIdx.x * blockDim.x + threadIdx.x) * 4;
-    // float4 access needs `out` 16-byte aligned and every part's start too
-    // (`part` is 256-byte aligned scratch, part p starts p * total floats on)
-    const bool vec = (reinterpret_cast<uintptr_t>(out) & 15) == 0 && (total & 3) == 0;
-    if (vec && i4 + 3 < total) {
-        float4 a = *reinterpret_cast<const float4 *>(part + i4);
-        for (int p = 1; p < P; ++p) {
-            const float4 v = *reinterpret_cast<const float4 *>(part + (long)p * total + i4);
-            a.x += v.x;
-            a.y += v.y;
-            a.z += v.z;
-            a.w += v.w;
+    for (long i = (long)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (long)gridDim.x * blockDim.x) {
+        T a = (T)0, d = (T)0;
+        for (int q = 0; q < P; ++q) {
+            a += parts[(long)q * total + i];
+            if (MASK) d += partw[(long)q * total + i];
         }
-        *reinterpret_cast<float4 *>(out + i4) = a;
-    } else {
-        for (long i = i4; i < total && i < i4 + 4; ++i) {
-            float a = part[i];
-            for (int p = 1; p < P; ++p) a += part[(long)p * total + i];
+        if (MASK) {
+            out[i] = d > (T)0 ? n_r * a / d : (T)0;
+            if (cov) cov[i] = d / n_r;
+        } else {
             out[i] = a;
         }
     }
 }
 
-// kernel form of the unmasked fp32 direct map: 0 = scalar FMAs (k_map_direct),
-// 1 .. 4 = k_map_direct_f2 shapes (fm_tune FM_TUNE_DIRECT), -1 = by radius:
-// measured on one 1024^2 map (ms, forms 1 / 2 / 3 / 4), S98 theta = 8:
-// 0.084 / 0.062 / 0.068 / 0.070, theta = 32: 0.531 / 0.435 / 0.484 / 0.496,
-// theta = 64: 1.53 / 1.48 / 1.46 / 1.52, starlet Q theta = 64 (R = 128):
-// 5.01 / 5.08 / 4.99 / 5.13; the scalar form 0.091, 0.597, 1.98, 7.01
+// FM_TUNE_DIRECT: kept for its callers; every value runs the one kernel form
 std::atomic<int> g_direct_form{-1};
-static int direct_form(int Ri)
-{
-    const int f = g_direct_form.load();
-    return f >= 0 ? f : (Ri < 48 ? 2 : 3);
-}
 
-// parts of the input-row walk: about 16 rows each, at most 16 (a function of
-// the tile height and radius only, so results never depend on the batch).
-// Measured on one 1024^2 map (ms), parts of ~32 rows (at most 8) / ~16 (16) /
-// ~64 (4): S98 theta = 64 1.41 / 1.33 / 1.65, starlet Q theta = 64 4.83 /
-// 4.71 / 5.19, JBJ04 theta = 16 (cut 5 theta) 2.01 / 1.92 / 2.46.
-static int direct_parts(int TY, int Ri)
+// Parts of the dy: a function of n and the radius only, so that a map's
+// result does not depend on the maps beside it.  Enough warps for two full
+// loads of the GPU (152 SMs x 20 warps), at least four dy a part, at most 16.
+static int direct_parts(int n, int Ri, int TX)
 {
-    const int P = (TY + 2 * Ri) / 16;
-    return P < 1 ? 1 : (P > 16 ? 16 : P);
+    const long warps = (long)n * ((n + TX - 1) / TX);
+    long P = (2 * 152 * 20 + warps - 1) / warps;
+    P = std::min<long>({P, 16, (Ri + 1) / 4});
+    return P < 1 ? 1 : (int)P;
 }
 // maps per launch pair when the parts go through scratch: at most 256 MiB of
 // partial sums (the order of the sums is per map, so the slicing of a batch
 // does not change any result)
-static int direct_slice(int P, int n, int batch)
+static int direct_slice(int P, int n, int batch, size_t es)
 {
-    if (P <= 1) return batch;
-    const long per_map = (long)P * n * n * (long)sizeof(float);
-    long m = (256L << 20) / per_map;
-    m = m < 1 ? 1 : m;
-    return m < batch ? (int)m : batch;
+    // the grid's third dimension holds maps x parts
+    const int most = std::min(batch, 65535 / P);
+    if (P <= 1) return most;
+    const long m = (256L << 20) / ((long)P * n * n * (long)es);
+    return (int)std::max<long>(1, std::min<long>(m, most));
 }
 
-template <int RY, int NW>
-static int launch_direct_f2(const float *g1, const float *g2, const float2 *dtaps, int tw, const int *ddx, float *map,
-                            float *parts, int n, int batch, int Ri, cudaStream_t s)
-{
-    constexpr int CX = 8, TX = 32 * CX, TY = NW * RY;
-    const int width = TX + 2 * Ri + 8;
-    const int pw = width + (width >> 3) + 1;
-    const size_t smem = 2ull * pw * sizeof(float2);
-    const int P = direct_parts(TY, Ri);
-    const int slice = direct_slice(P, n, batch);
-    auto k = k_map_direct_f2<CX, RY, NW>;
-    FM_CUDA_TRY(fm::smem_attr((const void *)k, smem));
-    const long nn = (long)n * n;
-    for (int b0 = 0; b0 < batch; b0 += slice) {
-        const int bs = batch - b0 < slice ? batch - b0 : slice;
-        dim3 grid((n + TX - 1) / TX, (n + TY - 1) / TY, bs * P);
-        FM_LAUNCH(FM_K_MAP_DIRECT, k, grid, NW * 32, smem, s, g1 + b0 * nn, g2 + b0 * nn, dtaps, tw, ddx,
-                  P > 1 ? parts : map + b0 * nn, n, Ri, P, bs);
-        if (P > 1) {
-            const long total = (long)bs * nn;
-            const unsigned g = (unsigned)((total / 4 + 255) / 256 + 1);
-            FM_LAUNCH(FM_K_MAP_DIRECT, k_sum_parts, g, 256, 0, s, (const float *)parts, map + b0 * nn, total, P);
-        }
-    }
-    return FM_OK;
-}
-
-static size_t direct_parts_bytes(int form, int n, int batch, int Ri)
-{
-    const int TY = form == 2 ? 8 : form == 3 ? 8 : 16;
-    const int P = direct_parts(TY, Ri);
-    return P > 1 ? (size_t)P * direct_slice(P, n, batch) * n * n * sizeof(float) : 0;
-}
-
-template <typename T>
+template <typename T, bool MASK>
 static int map_direct_impl(const T *g1, const T *g2, const T *wgt, long w_bs, T *map, T *cov, int n, int batch,
                            int filter, double theta, int ell, double cut, cudaStream_t s)
 {
     using V = cplx_t<T>;
-    const bool mask = wgt != nullptr;
-    const double R = (cut > 0 ? cut : default_cut(filter)) * theta;
-    const int Ri = (int)floor(R);
-    const int tw = 2 * Ri + 8;  // weight row: dx = -Ri .. Ri + 7 (zeros beyond R)
-    const size_t ntap = (size_t)(2 * Ri + 1) * tw;
-    std::vector<V> htaps(ntap);
-    std::vector<T> hdisc(mask ? ntap : 0);
-    std::vector<int> hdx(2 * Ri + 1);
+    using D = DirectRow<T>;
+    const double R = (cut > 0 ? cut : default_cut(filter)) * theta, R2 = R * R;
+    const int Ri = (int)floor(R), rp = D::rp(Ri), tw = D::tap_width(Ri);
     long n_r = 0;  // lattice offsets 0 < |d| <= R
-    for (int dy = -Ri; dy <= Ri; ++dy) {
-        const double m2 = R * R - (double)dy * dy;
-        hdx[dy + Ri] = m2 >= 0 ? (int)floor(sqrt(m2)) : -1;
-        for (int c = 0; c < tw; ++c) {
-            const int dx = c - Ri;
-            const double r2 = (double)dx * dx + (double)dy * dy;
-            V ab;
-            ab.x = ab.y = 0;
-            const bool in = r2 > 0 && r2 <= R * R;
-            if (in) {
-                const double q = q_of(filter, sqrt(r2), theta, ell);
-                ab.x = (decltype(ab.x))(-q * ((double)dx * dx - (double)dy * dy) / r2);
-                ab.y = (decltype(ab.y))(-q * 2.0 * dx * dy / r2);
-                ++n_r;
-            }
-            htaps[(size_t)(dy + Ri) * tw + c] = ab;
-            if (mask) hdisc[(size_t)(dy + Ri) * tw + c] = in ? (T)1 : (T)0;
-        }
+    if (MASK) {
+        for (int dy = 0; dy <= Ri; ++dy) n_r += (dy ? 2 : 1) * (2L * disc_half_width(dy, R2) + 1);
+        n_r -= 1;
     }
-    Scratch sc;
+    const int P = direct_parts(n, Ri, D::TX), slice = direct_slice(P, n, batch, sizeof(T));
     auto up = [](size_t b) { return ((b + 255) / 256) * 256; };
-    const size_t tap_bytes = htaps.size() * sizeof(V);
-    const size_t disc_bytes = hdisc.size() * sizeof(T);
-    const size_t dx_bytes = hdx.size() * sizeof(int);
-    const int form = direct_form(Ri);
-    const size_t part_bytes = (sizeof(T) == 4 && !mask && form > 0) ? direct_parts_bytes(form, n, batch, Ri) : 0;
-    int st = scratch_alloc(sc, up(tap_bytes) + up(disc_bytes) + up(dx_bytes) + part_bytes, s);
+    const size_t tap_b = up((size_t)(Ri + 1) * tw * sizeof(V)), dx_b = up((size_t)(Ri + 1) * sizeof(int));
+    const long nn = (long)n * n;
+    const size_t part_b = P > 1 ? up((size_t)P * slice * nn * sizeof(T)) : 0;
+    Scratch sc;
+    int st = scratch_alloc(sc, tap_b + dx_b + (MASK ? 2 : 1) * part_b, s);
     if (st != FM_OK) return st;
     char *base = static_cast<char *>(sc.p);
-    V *dtaps = reinterpret_cast<V *>(base);
-    T *ddisc = mask ? reinterpret_cast<T *>(base + up(tap_bytes)) : nullptr;
-    int *ddx = reinterpret_cast<int *>(base + up(tap_bytes) + up(disc_bytes));
-    float *dparts = reinterpret_cast<float *>(base + up(tap_bytes) + up(disc_bytes) + up(dx_bytes));
-    FM_CUDA_TRY(cudaMemcpyAsync(dtaps, htaps.data(), tap_bytes, cudaMemcpyHostToDevice, s));
-    if (mask) FM_CUDA_TRY(cudaMemcpyAsync(ddisc, hdisc.data(), disc_bytes, cudaMemcpyHostToDevice, s));
-    FM_CUDA_TRY(cudaMemcpyAsync(ddx, hdx.data(), dx_bytes, cudaMemcpyHostToDevice, s));
-
-    constexpr int CX = 8, NW = 4;
-    const int width = 32 * CX + 2 * Ri + 8;
-    const int pw = width + (width >> 3) + 1;
-    if constexpr (sizeof(T) == 4) {
-        const float2 *ft = reinterpret_cast<const float2 *>(dtaps);
-        if (!mask && form == 1) return launch_direct_f2<4, 4>(g1, g2, ft, tw, ddx, map, dparts, n, batch, Ri, s);
-        if (!mask && form == 2) return launch_direct_f2<2, 4>(g1, g2, ft, tw, ddx, map, dparts, n, batch, Ri, s);
-        if (!mask && form == 3) return launch_direct_f2<4, 2>(g1, g2, ft, tw, ddx, map, dparts, n, batch, Ri, s);
-        if (!mask && form == 4) return launch_direct_f2<2, 8>(g1, g2, ft, tw, ddx, map, dparts, n, batch, Ri, s);
-    }
-    if (!mask) {
-        constexpr int RY = 4, TX = 32 * CX, TY = NW * RY;
-        const size_t smem = 2ull * 2 * pw * sizeof(T);
-        auto k = k_map_direct<T, CX, RY, NW, false>;
-        FM_CUDA_TRY(fm::smem_attr((const void *)k, smem));
-        dim3 grid((n + TX - 1) / TX, (n + TY - 1) / TY, batch);
-        FM_LAUNCH(FM_K_MAP_DIRECT, k, grid, NW * 32, smem, s, g1, g2, (const T *)nullptr, 0l, dtaps,
-                  (const T *)nullptr, tw, ddx, map, (T *)nullptr, n, Ri, (T)n_r);
-    } else {
-        constexpr int RY = 2, TX = 32 * CX, TY = NW * RY;
-        const size_t smem = 2ull * 3 * pw * sizeof(T);
-        auto k = k_map_direct<T, CX, RY, NW, true>;
-        FM_CUDA_TRY(fm::smem_attr((const void *)k, smem));
-        dim3 grid((n + TX - 1) / TX, (n + TY - 1) / TY, batch);
-        FM_LAUNCH(FM_K_MAP_DIRECT, k, grid, NW * 32, smem, s, g1, g2, wgt, w_bs, dtaps, ddisc, tw, ddx, map, cov,
-                  n, Ri, (T)n_r);
+    V *taps = reinterpret_cast<V *>(base);
+    int *dxmax = reinterpret_cast<int *>(base + tap_b);
+    T *parts = reinterpret_cast<T *>(base + tap_b + dx_b);
+    T *partw = reinterpret_cast<T *>(base + tap_b + dx_b + part_b);
+    FM_LAUNCH(FM_K_MAP_DIRECT, k_direct_taps<T>, dim3((unsigned)((tw - rp + 63) / 64), (unsigned)(Ri + 1)), 64, 0, s,
+              taps, dxmax, Ri, rp, tw, R2, filter, theta, ell);
+    // four warps a CTA, fewer where their rows would leave the SM with few CTAs
+    const size_t wb = D::bytes(Ri, MASK);
+    const int nw = 4 * wb <= 56 * 1024 ? 4 : 2 * wb <= 110 * 1024 ? 2 : 1;
+    auto k = k_map_direct<T, MASK>;
+    FM_CUDA_TRY(fm::smem_attr((const void *)k, nw * wb));
+    for (int b0 = 0; b0 < batch; b0 += slice) {
+        const int bs = batch - b0 < slice ? batch - b0 : slice;
+        const dim3 grid((n + nw - 1) / nw, (n + D::TX - 1) / D::TX, bs * P);
+        T *o = map + b0 * nn, *oc = cov ? cov + b0 * nn : nullptr;
+        FM_LAUNCH(FM_K_MAP_DIRECT, k, grid, nw * 32, nw * wb, s, g1 + b0 * nn, g2 + b0 * nn,
+                  MASK ? wgt + b0 * w_bs : nullptr, w_bs, (const V *)taps, (const int *)dxmax, o, oc, parts, partw, n,
+                  Ri, rp, D::blocks(Ri), (int)wb, P, bs, (T)n_r);
+        if (P > 1) {
+            const long total = (long)bs * nn;
+            const unsigned g = (unsigned)std::min<long>((total + 255) / 256, 152L * 32);
+            FM_LAUNCH(FM_K_MAP_DIRECT, (k_direct_sum<T, MASK>), g, 256, 0, s, (const T *)parts, (const T *)partw, o, oc,
+                      total, P, (T)n_r);
+        }
     }
     return FM_OK;
+}
+
+template <typename T>
+static int map_direct_typed(const void *g1, const void *g2, const void *weight, long w_bs, void *map, void *coverage,
+                            int n, int batch, int filter, double theta, int ell, double cut, cudaStream_t s)
+{
+    const T *a = static_cast<const T *>(g1), *b = static_cast<const T *>(g2), *w = static_cast<const T *>(weight);
+    T *m = static_cast<T *>(map), *c = static_cast<T *>(coverage);
+    return w ? map_direct_impl<T, true>(a, b, w, w_bs, m, c, n, batch, filter, theta, ell, cut, s)
+             : map_direct_impl<T, false>(a, b, w, w_bs, m, c, n, batch, filter, theta, ell, cut, s);
 }
 
 int launch_map_direct(const void *g1, const void *g2, const void *weight, long w_bs, void *map, void *coverage, int n,
                       int batch, int filter, double theta, int ell, double cut, int precision, cudaStream_t s)
 {
-    if (precision == FM_F64)
-        return map_direct_impl<double>((const double *)g1, (const double *)g2, (const double *)weight, w_bs,
-                                       (double *)map, (double *)coverage, n, batch, filter, theta, ell, cut, s);
-    return map_direct_impl<float>((const float *)g1, (const float *)g2, (const float *)weight, w_bs, (float *)map,
-                                  (float *)coverage, n, batch, filter, theta, ell, cut, s);
+    return precision == FM_F64 ? map_direct_typed<double>(g1, g2, weight, w_bs, map, coverage, n, batch, filter, theta,
+                                                          ell, cut, s)
+                               : map_direct_typed<float>(g1, g2, weight, w_bs, map, coverage, n, batch, filter, theta,
+                                                         ell, cut, s);
 }
 
 }  // namespace fm
