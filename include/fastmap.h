@@ -82,8 +82,8 @@ typedef struct {
                        (the plain one-scale-per-pass form) */
     int large_path; /* scales after the fused ones: 0 = automatic (the
                        autotuned plan, else 4 where it applies after at
-                       least two fused scales, 3 after fused small scales
-                       on maps up to 256^2, 1 otherwise),
+                       least two fused scales and n >= 64, 3 after fused
+                       small scales on maps up to 256^2, 1 otherwise),
                        1 = one row pass + one column pass per scale, 2 = all
                        large scales in one row kernel + one column-strip
                        kernel, 3 = the column pass of each scale fused with
@@ -91,8 +91,8 @@ typedef struct {
                        kernel per scale; the pyramid's smooth-array slot
                        serves as scratch until its final write), 4 = one
                        pass per scale that row-filters c_{j-1} from shared
-                       memory (fp32, n a multiple of 512, scales with
-                       spacing 4..128 px; otherwise the form 1) */
+                       memory (fp32, n a multiple of 4, scales with spacing
+                       4..128 px; the form 1 for the others) */
 } fm_config;
 
 /* ---- Kaiser-Squires (Sec. 4.5) ---------------------------------------------

@@ -35,6 +35,13 @@ template <typename T> struct B3 {
     }
 };
 
+// fp32: integer taps and one exact scaling, the rounding of the packed filters
+// (tap5) below whatever the kernel
+template <> __device__ __forceinline__ float B3<float>::apply(float m2, float m1, float c, float p1, float p2)
+{
+    return fmaf(6.f, c, fmaf(4.f, m1 + p1, m2 + p2)) * 0.0625f;
+}
+
 // 16-byte vectors: 4 floats or 2 doubles
 template <typename T> struct Vec16;
 template <> struct Vec16<float> {
@@ -726,114 +733,141 @@ __global__ void __launch_bounds__(128) k_st_col(const T *__restrict__ r, long r_
 }
 
 // ---------------------------------------------------------------------------
-// One large scale in one pass (fp32, large_path 4: maps whose arrays stream
-// through HBM).  A CTA owns 512 columns (128 threads x float4) and KR output
-// rows y_k = r0 + s (mb + k) of one map, like k_st_col.  Its KR + 4 window
-// rows of c_{j-1} (rows r0 + s (mb + t - 2), folded at the map's top and
-// bottom) arrive by one bulk tensor copy each, 512 + 4s columns wide
-// (x0 - 2s .. x0 + 512 + 2s; mc views c_{j-1} as {2s, n / 2s, rows}), into
-// shared memory; halo columns outside the map are then loaded folded.  Each
-// thread row-filters its window rows there (taps +-s, +-2s) into a five-row
-// register window and filters that down the column: c_j, and w_j = c_{j-1} -
-// c_j with c_{j-1} the centre of the window row.  The row-filtered map never
-// goes through memory (the pair k_st_row + k_st_col moves 24 bytes per pixel,
-// this pass 8 + 4 (KR + 4) / KR (512 + 4s) / 512).  c_next must not alias
-// c_prev: other CTAs read its rows and halo columns.  4 <= s <= 128.
-template <int KR>
-__global__ void __launch_bounds__(128) k_st_scale(const float *c_prev, float *c_next, long next_bs,
-                                                  float *__restrict__ w_out, long w_bs, int n, int s, int boundary,
-                                                  const __grid_constant__ CUtensorMap mc)
+// One large scale in one pass (fp32, large_path 4).  A CTA owns CW = 4 NT
+// columns (NT threads x float4) and KR output rows y_k = r0 + S (mb + k) of
+// one map, like k_st_col.  Its KR + 4 window rows of c_{j-1} (rows r0 + S (mb
+// + t - 2), folded at the map's top and bottom) arrive in shared memory by K
+// bulk tensor copies of B columns each (x0 - 2S on; columns outside the map
+// arrive as zeros and are then folded).  Each thread row-filters its window
+// rows there (taps +-S, +-2S) into a five-row register window and filters
+// that down the column: c_j, and w_j = c_{j-1} - c_j with c_{j-1} the centre
+// of the window row.  The row-filtered map never goes through memory (the pair
+// k_st_row + k_st_col moves 24 bytes per pixel, this pass 8 + 4 (KR + 4) / KR
+// (CW + 4S) / CW).  c_next must not alias c_prev: other CTAs read its rows and
+// halo columns.
+//
+// What bounds it: instruction issue and the latency of one wave on L2-sized
+// chunks, HBM on large maps.  The spacing is a template parameter, so every
+// shared-memory offset is an immediate, and the filters run on packed pairs of
+// fp32 (taps 1, 4, 6, 4, 1, one exact 1 / 256).  Against a run-time spacing and
+// scalar filters, 32 x 1024^2 J = 7 through the pipeline 562 -> 551 us, 64 x
+// 512^2 284 -> 275; 3 x 1500^2 alone (row and column passes before) 145 -> 118.
+template <int S, int CW> struct ScaleBox {
+    static constexpr int K = (CW + 4 * S + 255) / 256;                     // copies per row (a box is at most 256 wide)
+    static constexpr int B = ((CW + 4 * S + K - 1) / K + 31) / 32 * 32;    // columns of one: 128-byte multiples
+    static constexpr int RW = K * B;                                       // floats per staged row
+    static constexpr size_t smem(int KR) { return 128 + (size_t)(KR + 4) * RW * sizeof(float); }
+};
+
+struct Pair4 {  // four columns as two packed pairs
+    float2 a, b;
+};
+__device__ __forceinline__ Pair4 p4(const float *p)
+{
+    const float4 v = f4(p);
+    return Pair4{make_float2(v.x, v.y), make_float2(v.z, v.w)};
+}
+// (a + e) + 4 (b + d) + 6 c on packed pairs, the rounding of tap5
+__device__ __forceinline__ float2 tap5(float2 a, float2 b, float2 c, float2 d, float2 e)
+{
+    return __ffma2_rn(make_float2(6.f, 6.f), c, __ffma2_rn(make_float2(4.f, 4.f), __fadd2_rn(b, d), __fadd2_rn(a, e)));
+}
+__device__ __forceinline__ Pair4 tap5(const Pair4 &a, const Pair4 &b, const Pair4 &c, const Pair4 &d, const Pair4 &e)
+{
+    return Pair4{tap5(a.a, b.a, c.a, d.a, e.a), tap5(a.b, b.b, c.b, d.b, e.b)};
+}
+
+template <int S, int KR, int NT>
+__global__ void __launch_bounds__(NT) k_st_scale(const float *c_prev, float *c_next, long next_bs,
+                                                 float *__restrict__ w_out, long w_bs, int n, int boundary,
+                                                 const __grid_constant__ CUtensorMap mc)
 {
     pdl_entry();
+    constexpr int CW = 4 * NT;
+    using X = ScaleBox<S, CW>;
+    constexpr int RW = X::RW;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ uint64_t bar;
-    const int RW = (512 + 4 * s + 31) & ~31;  // floats per staged row: 512 + 4s, padded so that every row (a
-                                              // bulk tensor copy destination) starts 128-byte aligned
-    float *sw = align128<float>(smem_raw);    // [KR + 4][RW]
-    const int x0 = blockIdx.x * 512;
-    const int r0 = blockIdx.y % s, mb = (blockIdx.y / s) * KR;
+    float *sw = align128<float>(smem_raw);  // [KR + 4][RW]
+    const int x0 = blockIdx.x * CW;
+    const int r0 = blockIdx.y % S, mb = (blockIdx.y / S) * KR;
+    if (r0 + S * mb >= n) return;  // the whole CTA: no row of this residue left
     const long b = blockIdx.z;
-    const float *cb = c_prev + b * (long)n * n;
     if (threadIdx.x == 0) mbar_init(&bar, 1);
     __syncthreads();
     // one window row per lane of the first warp, after lane 0 announced the bytes
     static_assert(KR + 4 <= 32, "window rows per warp");
     if (threadIdx.x < 32) {
-        if (threadIdx.x == 0) mbar_expect_tx(&bar, (uint32_t)((KR + 4) * (512 + 4 * s) * sizeof(float)));
+        if (threadIdx.x == 0) mbar_expect_tx(&bar, (uint32_t)((KR + 4) * RW * sizeof(float)));
         __syncwarp();
         const int t = threadIdx.x;
         if (t < KR + 4) {
-            const int y = fold_index(r0 + s * (mb + t - 2), n, boundary);
-            tma_load_3d(sw + t * RW, &mc, 0, x0 / (2 * s) - 1, (int)(b * n + y), &bar);
+            const int y = fold_index(r0 + S * (mb + t - 2), n, boundary);
+#pragma unroll
+            for (int k = 0; k < X::K; ++k)
+                tma_load_3d(sw + t * RW + k * X::B, &mc, x0 - 2 * S + k * X::B, (int)(b * n + y), 0, &bar);
         }
     }
     if (!tma_wait_all(&bar, 0)) return;  // the copies never completed (flagged)
-    if ((x0 == 0 || x0 + 512 == n) && boundary != FM_PERIODIC) {
-        // halo columns outside the map (the copies filled them with zeros):
-        // with 2s <= 256 < 512 only the first CTA's left halo and the last
-        // one's right halo leave the map.  Mirrored, staged column 2s + x of
-        // map column x (x0 = 0) gets column -x, and map column n + h
-        // (x0 = n - 512) gets n - 2 - h; both lie inside the map and were
-        // staged by this CTA.
-        const bool lo = x0 == 0, hi = x0 + 512 == n;
-        for (int h = threadIdx.x; h < 2 * s; h += blockDim.x) {
+    const int over = x0 + CW + 2 * S - n;  // window columns right of the map
+    if (x0 == 0 || over > 0) {
+        // Halo columns outside the map.  Mirrored, staged column 2S + x of map
+        // column x < 0 gets column -x, and map column n + h gets n - 2 - h;
+        // both were staged by this CTA (n > 2S, and a CTA's first column is
+        // inside the map) and are not themselves rewritten, as far as a thread
+        // inside the map reads.  Periodic ones wrap to the map's other edge and
+        // come from global memory.
+        const int hr = over < 0 ? 0 : over < 2 * S ? over : 2 * S;  // of the right halo
+        const int e0 = n - x0 + 2 * S;                              // staged index of map column n
+        if (boundary != FM_PERIODIC) {
+            for (int h = threadIdx.x; h < 2 * S; h += NT) {
 #pragma unroll
-            for (int t = 0; t < KR + 4; ++t) {
-                float *row = sw + t * RW;
-                if (lo) row[h] = row[4 * s - h];
-                if (hi) row[512 + 2 * s + h] = row[510 + 2 * s - h];
+                for (int t = 0; t < KR + 4; ++t) {
+                    float *row = sw + t * RW;
+                    if (x0 == 0) row[h] = row[4 * S - h];
+                    if (h < hr) row[e0 + h] = row[e0 - 2 - h];
+                }
             }
-        }
-        __syncthreads();
-    } else if (x0 - 2 * s < 0 || x0 + 512 + 2 * s > n) {
-        // periodic: halo columns outside the map wrap to its other edge and
-        // come from global memory
-        for (int e = threadIdx.x; e < (KR + 4) * 4 * s; e += blockDim.x) {
-            const int t = e / (4 * s), h = e % (4 * s);
-            const int xl = h < 2 * s ? h : 512 + h;  // left halo, then right halo
-            const int x = x0 - 2 * s + xl;
-            if (x < 0 || x >= n) {
-                const int xf = fold_index(x, n, boundary);
-                if (boundary == FM_PERIODIC) {
-                    const int y = fold_index(r0 + s * (mb + t - 2), n, boundary);
-                    sw[t * RW + xl] = cb[(long)y * n + xf];
-                } else {
-                    sw[t * RW + xl] = sw[t * RW + xf - x0 + 2 * s];
+        } else {
+            const float *cb = c_prev + b * (long)n * n;
+            for (int h = threadIdx.x; h < 2 * S; h += NT) {
+                for (int t = 0; t < KR + 4; ++t) {
+                    float *row = sw + t * RW;
+                    const float *src = cb + (long)fold_index(r0 + S * (mb + t - 2), n, boundary) * n;
+                    if (x0 == 0) row[h] = src[n - 2 * S + h];
+                    if (h < hr) row[e0 + h] = src[h];
                 }
             }
         }
         __syncthreads();
     }
-    const int xl = 2 * s + 4 * threadIdx.x, x = x0 + 4 * threadIdx.x;
-    float4 win[5], ctr[3];
+    const int x = x0 + 4 * threadIdx.x;
+    if (x >= n) return;  // n is a multiple of 4: the whole vector is inside or outside
+    const float *base = sw + 2 * S + 4 * threadIdx.x;
+    const long px0 = (long)(r0 + S * mb) * n + x;
+    float *wp = w_out + b * w_bs + px0, *cp = c_next ? c_next + b * next_bs + px0 : nullptr;
+    const long step = (long)S * n;
+    const int rows = (n - 1 - r0) / S - mb + 1;  // of this residue, from mb on
+    Pair4 win[5], ctr[3];
 #pragma unroll
     for (int t = 0; t < KR + 4; ++t) {
-        const float *row = sw + t * RW + xl;
-        const float4 m2 = f4(row - 2 * s), m1 = f4(row - s), c0 = f4(row), p1 = f4(row + s), p2 = f4(row + 2 * s);
-        // the same arithmetic as k_st_row
-        win[t % 5] = make_float4(B3<float>::apply(m2.x, m1.x, c0.x, p1.x, p2.x),
-                                 B3<float>::apply(m2.y, m1.y, c0.y, p1.y, p2.y),
-                                 B3<float>::apply(m2.z, m1.z, c0.z, p1.z, p2.z),
-                                 B3<float>::apply(m2.w, m1.w, c0.w, p1.w, p2.w));
+        const float *row = base + t * RW;
+        const Pair4 c0 = p4(row);
+        win[t % 5] = tap5(p4(row - 2 * S), p4(row - S), c0, p4(row + S), p4(row + 2 * S));
         ctr[t % 3] = c0;
         if (t >= 4) {
             const int k = t - 4;
-            const int y = r0 + s * (mb + k);
-            if (y < n) {
-                // the same arithmetic as k_st_col
-                const float4 &a = win[k % 5], &bq = win[(k + 1) % 5], &c = win[(k + 2) % 5], &d = win[(k + 3) % 5],
-                             &e = win[(k + 4) % 5];
-                alignas(16) float cj[4] = {B3<float>::apply(a.x, bq.x, c.x, d.x, e.x),
-                                           B3<float>::apply(a.y, bq.y, c.y, d.y, e.y),
-                                           B3<float>::apply(a.z, bq.z, c.z, d.z, e.z),
-                                           B3<float>::apply(a.w, bq.w, c.w, d.w, e.w)};
-                const float4 p = ctr[(k + 2) % 3];
-                alignas(16) float w[4] = {p.x - cj[0], p.y - cj[1], p.z - cj[2], p.w - cj[3]};
-                const long px = (long)y * n + x;
-                // n is a multiple of 512: the whole vector is inside
-                st16cs(w_out + b * w_bs + px, w);
-                if (c_next) st16(c_next + b * next_bs + px, cj);
+            if (k < rows) {
+                const Pair4 f = tap5(win[k % 5], win[(k + 1) % 5], win[(k + 2) % 5], win[(k + 3) % 5], win[(k + 4) % 5]);
+                const Pair4 p = ctr[(k + 2) % 3];
+                const float2 sc = make_float2(1.f / 256.f, 1.f / 256.f), m1 = make_float2(-1.f, -1.f);
+                const float2 ca = __fmul2_rn(f.a, sc), cbb = __fmul2_rn(f.b, sc);
+                const float2 wa = __ffma2_rn(ca, m1, p.a), wb = __ffma2_rn(cbb, m1, p.b);
+                __stcs(reinterpret_cast<float4 *>(wp), make_float4(wa.x, wa.y, wb.x, wb.y));
+                if (cp) *reinterpret_cast<float4 *>(cp) = make_float4(ca.x, ca.y, cbb.x, cbb.y);
             }
+            wp += step;
+            if (cp) cp += step;
         }
     }
 }
@@ -1103,16 +1137,16 @@ static int auto_fuse(int n, int J, const fm_config &cfg)
 }
 
 // Large-scale path when cfg.large_path = 0: the autotuned plan's, else one
-// pass per scale (k_st_scale) where it applies (n a multiple of 512, large
-// scales of spacing 4..128 px; fp32 only, fp64 takes the form 1), else the
-// column pass fused with the next row pass on maps up to 256^2 after fused
-// small scales, else one row and one column pass per scale.  One pass per
-// scale against the row + column pair (KS + starlet per batch, ms): 32 x
-// 1024^2 J = 7 0.818 -> 0.715, 16 x 2048^2 J = 8 1.99 -> 1.78, 16 x 4096^2
-// J = 9 10.52 -> 8.25, 1 x 8192^2 J = 9 3.16 -> 2.56.
+// pass per scale (k_st_scale) after two or more fused scales on sides that are
+// multiples of 4 (fp32 only, fp64 takes the form 1), else the column pass
+// fused with the next row pass on small maps, else one row and one column pass
+// per scale.  The three forms 1 / 3 / 4, starlet alone (us): 256 x 128^2 J = 5
+// 113 / 94 / 50, 1 x 256^2 J = 6 27 / 22 / 18, 128 x 256^2 184 / 163 / 81,
+// 40 x 300^2 84 / 78 / 56, 3 x 1500^2 J = 7 133 / 133 / 91, 3000^2 J = 9 213 /
+// 212 / 146; KS + starlet (ms, 1 / 4) 32 x 1024^2 J = 7 0.818 / 0.715.
 int starlet_builtin_large_path(int n, int J, int fuse)
 {
-    if (fuse >= 2 && n % 512 == 0 && (1 << (J - 2)) <= 128) return 4;
+    if (fuse >= 2 && n % 4 == 0 && n >= 64) return 4;
     return fuse >= 1 && n <= 256 ? 3 : 1;
 }
 
@@ -1228,6 +1262,53 @@ static int tile_dispatch(int f, const T *in, T *w_out, long w_bs, long w_ss, T *
     return FM_EINVAL;
 }
 
+// One pass of the scale of spacing S: KR rows a CTA, CW = 4 NT columns.
+constexpr int kScaleRefused = -1000;  // no tensor map for this layout
+template <int S, int KR, int NT>
+static int scale_launch_t(const float *c_in, float *c_out, long out_bs, float *w, long w_bs, int n, int bnd, int batch,
+                          cudaStream_t s)
+{
+    using X = ScaleBox<S, 4 * NT>;
+    CUtensorMap map;
+    const uint64_t dims[3] = {(uint64_t)n, (uint64_t)batch * n, 1};
+    const uint64_t str[2] = {(uint64_t)n * 4, (uint64_t)batch * n * n * 4};
+    const uint32_t box[3] = {X::B, 1, 1};
+    if (!encode_map3d_f32(&map, c_in, dims, str, box)) return kScaleRefused;
+    auto k = k_st_scale<S, KR, NT>;
+    FM_CUDA_TRY(fm::smem_attr((const void *)k, X::smem(KR)));
+    const dim3 grid((n + 4 * NT - 1) / (4 * NT), S * ((((n + S - 1) / S) + KR - 1) / KR), batch);
+    FM_LAUNCH(FM_K_STARLET_COL, k, grid, NT, X::smem(KR), s, c_in, c_out, out_bs, w, w_bs, n, bnd, map);
+    return FM_OK;
+}
+template <int S>
+static int scale_launch_s(const float *c_in, float *c_out, long out_bs, float *w, long w_bs, int n, int bnd, int batch,
+                          cudaStream_t s)
+{
+    // 16 rows a CTA for wide halos (S >= 32), so that the window's four extra
+    // rows are re-read less often, where a residue has that many rows; 256
+    // columns a CTA where 512 would leave the map
+    const bool tall = S >= 32 && n >= 16 * S;
+    if (n <= 256)
+        return tall ? scale_launch_t<S, 16, 64>(c_in, c_out, out_bs, w, w_bs, n, bnd, batch, s)
+                    : scale_launch_t<S, 8, 64>(c_in, c_out, out_bs, w, w_bs, n, bnd, batch, s);
+    return tall ? scale_launch_t<S, 16, 128>(c_in, c_out, out_bs, w, w_bs, n, bnd, batch, s)
+                : scale_launch_t<S, 8, 128>(c_in, c_out, out_bs, w, w_bs, n, bnd, batch, s);
+}
+constexpr int kScaleMinN = 32;
+static int scale_launch(const float *c_in, float *c_out, long out_bs, float *w, long w_bs, int n, int sp, int bnd,
+                        int batch, cudaStream_t s)
+{
+    switch (sp) {
+    case 4: return scale_launch_s<4>(c_in, c_out, out_bs, w, w_bs, n, bnd, batch, s);
+    case 8: return scale_launch_s<8>(c_in, c_out, out_bs, w, w_bs, n, bnd, batch, s);
+    case 16: return scale_launch_s<16>(c_in, c_out, out_bs, w, w_bs, n, bnd, batch, s);
+    case 32: return scale_launch_s<32>(c_in, c_out, out_bs, w, w_bs, n, bnd, batch, s);
+    case 64: return scale_launch_s<64>(c_in, c_out, out_bs, w, w_bs, n, bnd, batch, s);
+    case 128: return scale_launch_s<128>(c_in, c_out, out_bs, w, w_bs, n, bnd, batch, s);
+    }
+    return kScaleRefused;
+}
+
 static bool aligned16(const void *p) { return ((uintptr_t)p & 15u) == 0; }
 
 template <typename T>
@@ -1285,48 +1366,25 @@ static int starlet_impl(const T *kappa, T *pyr, long pyr_bs, int n, int J, int b
 #undef FM_COLS_MULTI
         return FM_OK;
     }
+    int j0 = f + 1;  // first scale left for the passes below, its input and the free scratch map
+    const T *c_in = f >= 1 ? A : kappa;
     if constexpr (sizeof(T) == 4) {
-        // large_path 4: one pass per large scale, row filter from shared memory
-        const int s_lo = 1 << f, s_hi = 1 << (J - 2);  // spacing of the first and last large scale
-        if (K >= 1 && lpath == 4 && vec_ok && n % 512 == 0 && s_lo >= 4 && s_hi <= 128 && Bb) {
-            constexpr int KRS = 8;
-            // c_j alternates between A and Bb (never in place); the last goes to
-            // the smooth-array slot.  Tensor maps first: if the driver refuses
-            // one, the two-pass path below runs instead.
-            const T *srcs[20];
-            T *dsts[20];
-            CUtensorMap maps[20];
-            bool ok = true;
-            const T *src = f >= 1 ? A : kappa;
-            for (int j = f + 1; j <= J - 1 && ok; ++j) {
-                const int sp = 1 << (j - 1);
-                T *dst = j == J - 1 ? (bands_only ? nullptr : last) : (src == Bb ? A : Bb);
-                const uint64_t dims[3] = {(uint64_t)(2 * sp), (uint64_t)(n / (2 * sp)), (uint64_t)batch * n};
-                const uint64_t str[2] = {(uint64_t)(2 * sp) * 4, (uint64_t)n * 4};
-                const uint32_t box[3] = {(uint32_t)(2 * sp), (uint32_t)(256 / sp + 2), 1};
-                ok = encode_map3d_f32(&maps[j], src, dims, str, box);
-                srcs[j] = src;
-                dsts[j] = dst;
-                src = dst;
-            }
-            if (ok) {
-                for (int j = f + 1; j <= J - 1; ++j) {
-                    const int sp = 1 << (j - 1);
-                    const long dst_bs = j == J - 1 ? pyr_bs : nn;
-                    // wide halos (s >= 32): 16 output rows a CTA, so that the
-                    // window's four extra rows are re-read less often
-                    const int kr = sp >= 32 ? 16 : KRS;
-                    auto ksc = kr == 16 ? k_st_scale<16> : k_st_scale<KRS>;
-                    const size_t ssm = 128 + (size_t)(kr + 4) * ((512 + 4 * sp + 31) & ~31) * sizeof(float);
-                    FM_CUDA_TRY(fm::smem_attr((const void *)ksc, ssm));
-                    const unsigned gys = (unsigned)(sp * ((((n + sp - 1) / sp) + kr - 1) / kr));
-                    FM_LAUNCH(FM_K_STARLET_COL, ksc, dim3(n / 512, gys, batch), 128, ssm, s, (const float *)srcs[j],
-                              (float *)dsts[j], dst_bs, (float *)(pyr + (long)(j - 1) * nn), pyr_bs, n, sp, bnd,
-                              maps[j]);
-                }
-                return FM_OK;
-            }
+        // large_path 4: one pass per large scale of spacing 4 .. 128, row filter
+        // from shared memory.  c_j alternates between A and Bb (never in
+        // place); the last goes to the smooth-array slot.  Scales the driver
+        // refuses a tensor map for, and larger ones, take the passes below.
+        for (; j0 <= J - 1 && lpath == 4 && vec_ok && Bb && n >= kScaleMinN; ++j0) {
+            const int sp = 1 << (j0 - 1);
+            if (sp < 4 || sp > 128) break;
+            T *dst = j0 == J - 1 ? (bands_only ? nullptr : last) : (c_in == Bb ? A : Bb);
+            int st = scale_launch(c_in, dst, j0 == J - 1 ? pyr_bs : nn, pyr + (long)(j0 - 1) * nn, pyr_bs, n, sp, bnd,
+                                  batch, s);
+            if (st == kScaleRefused) break;
+            if (st != FM_OK) return st;
+            c_in = dst;
         }
+        if (j0 > J - 1) return FM_OK;
+        if (c_in == Bb) std::swap(A, Bb);  // the passes below keep c in A
     }
     const unsigned gx = (unsigned)((n + 128 * VW - 1) / (128 * VW));
     // row pass: up to 256 threads (1024 fp32 pixels) of one row per CTA, so
@@ -1352,14 +1410,14 @@ static int starlet_impl(const T *kappa, T *pyr, long pyr_bs, int n, int J, int b
     // between Bb and the pyramid's smooth-array slot (unused until the last
     // column pass writes c_{J-1} there), placed so that r_{J-1} is in Bb.
     auto r_in_last = [&](int j) { return colrow && (J - 1 - j) % 2 == 1; };
-    for (int j = f + 1; j <= J - 1; ++j) {
+    for (int j = j0; j <= J - 1; ++j) {
         const int sp = 1 << (j - 1);
         const T *c_prev = j == 1 ? kappa : A;
         T *c_next = j == J - 1 ? (bands_only ? nullptr : last) : A;
         const long next_bs = j == J - 1 ? pyr_bs : nn;
         T *rj = r_in_last(j) ? last : Bb;
         const long rj_bs = r_in_last(j) ? pyr_bs : nn;
-        if (!colrow || j == f + 1)
+        if (!colrow || j == j0)
             FM_LAUNCH(FM_K_STARLET_ROW, k_st_row<T>, dim3(gxr, n, batch), rt, 0, s, c_prev, nn, rj, rj_bs, n, sp, bnd,
                       vec_ok ? 1 : 0);
         if (colrow && j < J - 1) {
