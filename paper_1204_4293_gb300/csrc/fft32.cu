@@ -61,7 +61,10 @@
 
 namespace fm {
 
-__device__ __forceinline__ int pad16(int a) { return a + (a >> 4); }
+// shared-memory slot of element a of a transform of length 2^LOGN: one slot of
+// padding per E, so that E-strided stores of W interleaved vectors hit every
+// bank (the stride E W + W is W modulo 16 eight-byte slots)
+template <int LOGN> __device__ __forceinline__ constexpr int padded(int a) { return a + (a >> FftPlan<LOGN>::LOGE); }
 
 // threads of a row-pass CTA (RPC rows of TV threads; one row when TV is
 // larger)
@@ -76,7 +79,7 @@ template <int LOGN> struct Plan32 : FftPlan<LOGN> {
     static constexpr int ROW_T = RPC * TV;
     static constexpr int THREADS = 16384 / B::E;  // threads of an SM: 1024 (64 registers) with 16 elements each, 512 (128) with 32
     static constexpr int ROW_MINB = THREADS / ROW_T < 1 ? 1 : (THREADS / ROW_T > 24 ? 24 : THREADS / ROW_T);
-    static constexpr int VS = N + N / 16;  // exchange buffer of one vector (elements)
+    static constexpr int VS = N + N / B::E;  // exchange buffer of one vector (elements)
     // column strip width: 64 B row segments at n = 1024, 32 B at 2048 and
     // 4096 (one full sector), 16 B at 8192
     static constexpr int W = N <= 512 ? 16 : (N >= 8192 ? 2 : (N == 4096 ? 4 : 8192 / N));
@@ -103,7 +106,7 @@ template <bool INV> __device__ __forceinline__ float2 mul_tw(float2 a, const flo
 }
 
 // In: v[q] = x[j + q TV].  Out: v[q] = X[j + q TV].
-// Element i of vector c (of W) lives at sm[pad16(i W + c)] between passes.
+// Element i of vector c (of W) lives at sm[padded(i W + c)] between passes.
 // tw: the pass tables of length N (FftPlan's layout, after the natural table).
 // Every thread taking part must call this (it holds barriers).
 template <int LOGN, int W, bool INV, int NB = 0>
@@ -113,19 +116,18 @@ __device__ __forceinline__ void fft_vec(float2 (&v)[FftPlan<LOGN>::E], float2 *s
     using P = FftPlan<LOGN>;
     constexpr int E = P::E;
     // Padded addresses split into one base a thread and compile-time offsets
-    // (immediates of the loads and stores): exact as long as 16 divides the
-    // strides, i.e. TV W >= 16; smaller vectors take the formula itself.
-    constexpr bool LIN = P::TV * W >= 16;
-    constexpr int TVS = P::TV * W + P::TV * W / 16;  // padded stride of TV elements
-    float2 *rd = sm + pad16(j * W + c);              // x[j], then + q TVS
-    auto load = [&](int q) { return LIN ? rd[q * TVS] : sm[pad16((j + q * P::TV) * W + c)]; };
+    // (immediates of the loads and stores): exact, since TV W and E divide one
+    // another and the base stays below TV W.
+    static_assert(W <= E, "padding");
+    constexpr int TVW = P::TV * W;
+    float2 *rd = sm + padded<LOGN>(j * W + c);  // x[j]
+    auto load = [&](int q) { return rd[padded<LOGN>(q * TVW)]; };
     Dft<E, INV, float2>::run(v);  // pass 0: Ns = 1, no twiddles; outputs at E j + r
     part_sync<NB>();              // the buffer may still be read by an earlier pass
     {
-        static_assert(W <= 16 && (E * W) % 16 == 0, "padding");
-        float2 *wr = sm + j * (E * W + E * W / 16) + c;
+        float2 *wr = sm + j * (E * W + W) + c;
 #pragma unroll
-        for (int r = 0; r < E; ++r) wr[r * W + ((r * W) >> 4)] = v[r];
+        for (int r = 0; r < E; ++r) wr[padded<LOGN>(r * W)] = v[r];
     }
     part_sync<NB>();
     // middle passes: radix E, Ns = E, E^2
@@ -140,9 +142,9 @@ __device__ __forceinline__ void fft_vec(float2 (&v)[FftPlan<LOGN>::E], float2 *s
         for (int r = 1; r < E; ++r) v[r] = mul_tw<INV>(v[r], t + (r - 1) * NS);
         Dft<E, INV, float2>::run(v);
         part_sync<NB>();
-        float2 *wr = sm + pad16(((j - k) * E + k) * W + c);
+        float2 *wr = sm + padded<LOGN>(((j - k) * E + k) * W + c);
 #pragma unroll
-        for (int r = 0; r < E; ++r) wr[r * (NS * W + NS * W / 16)] = v[r];
+        for (int r = 0; r < E; ++r) wr[padded<LOGN>(r * NS * W)] = v[r];
         part_sync<NB>();
     }
     // last pass: radix RL, Ns = NSL, butterfly b = j + m TV (< NSL), twiddle W_n^(r b)
@@ -247,7 +249,7 @@ __global__ void __launch_bounds__(Plan32<LOGN>::ROW_T, Plan32<LOGN>::ROW_MINB)
         // Z through the exchange buffer so that Z(kx) and Z(n - kx) meet
         __syncthreads();  // the last pass's reads of the buffer
 #pragma unroll
-        for (int q = 0; q < P::E; ++q) sm[pad16(j + q * P::TV)] = v[q];
+        for (int q = 0; q < P::E; ++q) sm[padded<LOGN>(j + q * P::TV)] = v[q];
         __syncthreads();
         if (live) {
             // slot kx of the row: (Gamma1(kx), Gamma2(kx)) as one 16-byte element
@@ -255,12 +257,12 @@ __global__ void __launch_bounds__(Plan32<LOGN>::ROW_T, Plan32<LOGN>::ROW_MINB)
 #pragma unroll
             for (int t = 0; t < P::E / 2; ++t) {
                 const int kx = j + t * P::TV;
-                const float2 a = sm[pad16(kx)];
+                const float2 a = sm[padded<LOGN>(kx)];
                 if (kx == 0) {
-                    const float2 h = sm[pad16(P::N / 2)];
+                    const float2 h = sm[padded<LOGN>(P::N / 2)];
                     d[0] = make_float4(a.x, h.x, a.y, h.y);
                 } else {
-                    const float2 bm = sm[pad16(P::N - kx)];  // Z(n - kx); B = conj of it
+                    const float2 bm = sm[padded<LOGN>(P::N - kx)];  // Z(n - kx); B = conj of it
                     d[kx] = make_float4(0.5f * (a.x + bm.x), 0.5f * (a.y - bm.y), 0.5f * (a.y + bm.y),
                                         -0.5f * (a.x - bm.x));
                 }
@@ -436,7 +438,7 @@ __global__ void __launch_bounds__(Plan32<LOGN>::COL_T, Plan32<LOGN>::COL_MINB)
 template <int LOGN> struct PlanE {
     static constexpr int N = 1 << LOGN;
     static constexpr int WS = N <= 256 ? 16 : (N == 512 ? 8 : (N == 1024 ? 4 : (N <= 4096 ? 2 : 1)));
-    static constexpr int RSZ = (N * WS + N * WS / 16 + 1 + 15) & ~15;  // float2 per region, 128-byte multiple
+    static constexpr int RSZ = (N * WS + N * WS / FftPlan<LOGN>::E + 1 + 15) & ~15;  // float2 per region, 128-byte multiple
     // the corner strip's dense exchange (2n elements): with WS >= 2 both
     // halves go to the Gamma1 region after its transform (the Gamma2 region
     // carries the other slots' hand-over); with WS = 1 the strip is the
@@ -718,11 +720,11 @@ static int ks32_impl(const float *in1, const float *in2, long in_bs, float *out1
     const long total_rows = (long)batch * P::N;
     const unsigned row_grid = (unsigned)((total_rows + RPC - 1) / RPC);
     // exchange buffer (which also stages the TMA rows: RPC n floats per input
-    // array or RPC n float2 <= RPC (n + n/16) float2) + 128 bytes of alignment
+    // array or RPC n float2 <= RPC (n + n/E) float2) + 128 bytes of alignment
     const size_t row_smem = (size_t)RPC * P::VS * sizeof(float2) + 128;
     const int col_threads = P::W * P::TV;
     // exchange buffer (also the TMA strip: n W float2) + 128 bytes of alignment
-    const size_t col_smem = (size_t)(P::N * P::W + P::N * P::W / 16 + 1) * sizeof(float2) + 128;
+    const size_t col_smem = (size_t)(P::N * P::W + P::N * P::W / P::E + 1) * sizeof(float2) + 128;
     const unsigned col_grid = (unsigned)((long)batch * (P::N / P::W));
     auto krf = rotate ? k_rows_fwd32<LOGN, false, true> : k_rows_fwd32<LOGN, false, false>;
     FM_CUDA_TRY(fm::smem_attr((const void *)krf, row_smem));
