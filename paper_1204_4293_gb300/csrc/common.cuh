@@ -57,6 +57,9 @@ extern std::atomic<int> g_direct_form;
 int starlet_wait_error(bool clear);
 int fft_wait_error(bool clear);
 int einval(const std::string &msg);  // records msg as the last error, returns FM_EINVAL
+// Kernels that stage by bulk copies do what touches no other kernel's results
+// first (barrier initialisation, the tensor maps' prefetch), so that it runs
+// while the kernel before drains.
 __device__ __forceinline__ void pdl_entry()
 {
 #if defined(__CUDA_ARCH__) && __CUDA_ARCH__ >= 900

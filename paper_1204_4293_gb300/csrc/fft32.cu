@@ -187,12 +187,18 @@ __global__ void __launch_bounds__(Plan32<LOGN>::ROW_T, Plan32<LOGN>::ROW_MINB)
                                                        const __grid_constant__ CUtensorMap m1,
                                                        const __grid_constant__ CUtensorMap m2, int use_tma)
 {
-    pdl_entry();
     using P = Plan32<LOGN>;
     constexpr int RPC = P::RPC;
     extern __shared__ __align__(16) float2 sm32[];
     __shared__ uint64_t bar;
     float2 *smb = align128<float2>(sm32);
+    if (use_tma && threadIdx.x == 0) {
+        mbar_init(&bar, 1);
+        tma_prefetch_map(&m1);
+        if (in2) tma_prefetch_map(&m2);
+    }
+    __syncthreads();
+    pdl_entry();
     const int vr = threadIdx.x / P::TV, j = threadIdx.x % P::TV;
     const long row = (long)blockIdx.x * RPC + vr;
     float2 *sm = smb + vr * P::VS;
@@ -204,8 +210,6 @@ __global__ void __launch_bounds__(Plan32<LOGN>::ROW_T, Plan32<LOGN>::ROW_MINB)
     if constexpr (P::N >= 64) {
         if (use_tma) {
             float *st1 = reinterpret_cast<float *>(smb), *st2 = st1 + RPC * P::N;
-            if (threadIdx.x == 0) mbar_init(&bar, 1);
-            __syncthreads();
             if (threadIdx.x == 0) {
                 const long row0 = (long)blockIdx.x * RPC;
                 const int z = (int)(in_bs == 0 ? (row0 & (P::N - 1)) : row0);
@@ -289,12 +293,17 @@ __global__ void __launch_bounds__(Plan32<LOGN>::ROW_T, Plan32<LOGN>::ROW_MINB)
                                                        const float2 *__restrict__ tw, float scale,
                                                        const __grid_constant__ CUtensorMap mw, int use_tma)
 {
-    pdl_entry();
     using P = Plan32<LOGN>;
     constexpr int RPC = P::RPC;
     extern __shared__ __align__(16) float2 sm32[];
     __shared__ uint64_t bar;
     float2 *smb = align128<float2>(sm32);
+    if (use_tma && threadIdx.x == 0) {
+        mbar_init(&bar, 1);
+        tma_prefetch_map(&mw);
+    }
+    __syncthreads();
+    pdl_entry();
     const int vr = threadIdx.x / P::TV, j = threadIdx.x % P::TV;
     const long row = (long)blockIdx.x * RPC + vr;
     float2 *sm = smb + vr * P::VS;
@@ -303,8 +312,6 @@ __global__ void __launch_bounds__(Plan32<LOGN>::ROW_T, Plan32<LOGN>::ROW_MINB)
     bool staged = false;
     if constexpr (P::N >= 64) {
         if (use_tma) {
-            if (threadIdx.x == 0) mbar_init(&bar, 1);
-            __syncthreads();
             if (threadIdx.x == 0) {
                 mbar_expect_tx(&bar, (uint32_t)(RPC * P::N * sizeof(float2)));
                 tma_load_3d(smb, &mw, 0, 0, (int)((long)blockIdx.x * RPC), &bar);
@@ -345,23 +352,26 @@ __global__ void __launch_bounds__(Plan32<LOGN>::COL_T, Plan32<LOGN>::COL_MINB)
                                                    int op_arg, const float2 *__restrict__ filt,
                                                    const __grid_constant__ CUtensorMap mw, int use_tma)
 {
-    pdl_entry();
     const int op = KSINV ? FFT_OP_KS_INV : op_arg;
     using P = Plan32<LOGN>;
     constexpr int W = P::W, N = P::N;
     constexpr int STRIPS = N / W;
     extern __shared__ __align__(16) unsigned char smem_col[];
     float2 *sm32 = align128<float2>(smem_col);
+    __shared__ uint64_t bar;
+    if (use_tma && threadIdx.x == 0) {
+        mbar_init(&bar, 1);
+        tma_prefetch_map(&mw);
+    }
+    __syncthreads();
+    pdl_entry();
     const long b = blockIdx.x / STRIPS;
     const int x0 = (blockIdx.x % STRIPS) * W;
     const int c = threadIdx.x % W, j = threadIdx.x / W;
     float2 *base = work + b * (long)N * N + x0 + c;
     float2 v[P::E];
     if (use_tma & 1) {
-        __shared__ uint64_t bar;
         constexpr int BR = N < 256 ? N : 256;  // rows per copy
-        if (threadIdx.x == 0) mbar_init(&bar, 1);
-        __syncthreads();
         if (threadIdx.x == 0) {
             mbar_expect_tx(&bar, (uint32_t)(N * W * sizeof(float2)));
             for (int k = 0; k < N / BR; ++k) tma_load_3d(sm32 + k * BR * W, &mw, 2 * x0, k * BR, (int)b, &bar);
@@ -459,7 +469,6 @@ __global__ void __launch_bounds__(PlanE<LOGN>::NT, PlanE<LOGN>::MINB)
     k_cols_ks32_e(const float2 *__restrict__ work, float2 *__restrict__ half, const float2 *__restrict__ tw,
                   const __grid_constant__ CUtensorMap mw, int use_tma)
 {
-    pdl_entry();
     using P = Plan32<LOGN>;
     using E = PlanE<LOGN>;
     constexpr int N = P::N, WS = E::WS, NH = E::NH;
@@ -467,6 +476,13 @@ __global__ void __launch_bounds__(PlanE<LOGN>::NT, PlanE<LOGN>::MINB)
     extern __shared__ __align__(16) unsigned char smem_col[];
     float2 *R1 = align128<float2>(smem_col);
     float2 *R2 = R1 + E::RSZ;
+    __shared__ uint64_t bar;
+    if (use_tma && threadIdx.x == 0) {
+        mbar_init(&bar, 1);
+        tma_prefetch_map(&mw);
+    }
+    __syncthreads();
+    pdl_entry();
     float2 *U1 = R1, *U2 = WS == 1 ? R2 : R1 + N;  // corner exchange
     const long b = blockIdx.x / STRIPS;
     const int s0 = (blockIdx.x % STRIPS) * WS;
@@ -474,10 +490,7 @@ __global__ void __launch_bounds__(PlanE<LOGN>::NT, PlanE<LOGN>::MINB)
     float2 *R = hf ? R2 : R1;  // this half's strip and exchange region
     float2 v[P::E];
     if (use_tma) {
-        __shared__ uint64_t bar;
         constexpr int BR = N < 256 ? N : 256;  // rows per copy
-        if (tid == 0) mbar_init(&bar, 1);
-        __syncthreads();
         if (tid == 0) {
             // the strip, [n][WS] (Gamma1, Gamma2) pairs, over both regions
             mbar_expect_tx(&bar, (uint32_t)(2 * N * WS * sizeof(float2)));
@@ -570,13 +583,18 @@ __global__ void __launch_bounds__(Plan32<LOGN - 1>::ROW_T, Plan32<LOGN - 1>::ROW
                                                            const float2 *__restrict__ tw2, float scale,
                                                            const __grid_constant__ CUtensorMap mk, int use_tma)
 {
-    pdl_entry();
     using P = Plan32<LOGN - 1>;  // the length n/2 complex transform
     constexpr int N2 = P::N;
     constexpr int RPC = P::RPC;
     extern __shared__ __align__(16) float2 sm32[];
     __shared__ uint64_t bar;
     float2 *smb = align128<float2>(sm32);
+    if (use_tma && threadIdx.x == 0) {
+        mbar_init(&bar, 1);
+        tma_prefetch_map(&mk);
+    }
+    __syncthreads();
+    pdl_entry();
     const int vr = threadIdx.x / P::TV, j = threadIdx.x % P::TV;
     const long row = (long)blockIdx.x * RPC + vr;
     float2 *sm = smb + vr * P::VS;
@@ -584,8 +602,6 @@ __global__ void __launch_bounds__(Plan32<LOGN - 1>::ROW_T, Plan32<LOGN - 1>::ROW
     const float2 *h = reinterpret_cast<const float2 *>(kap) + row * N2;
     if constexpr (P::N >= 64) {
         if (use_tma) {
-            if (threadIdx.x == 0) mbar_init(&bar, 1);
-            __syncthreads();
             if (threadIdx.x == 0) {
                 mbar_expect_tx(&bar, (uint32_t)(RPC * N2 * sizeof(float2)));
                 tma_load_3d(smb, &mk, 0, 0, (int)((long)blockIdx.x * RPC), &bar);

@@ -474,7 +474,6 @@ __global__ void __launch_bounds__(256, F >= 4 ? 1 : 3)
                   float *__restrict__ c_out, long c_bs, int n, int boundary, int tiles_x, int tiles_per_map,
                   int vec_ok, const __grid_constant__ CUtensorMap tmap, int use_tma)
 {
-    pdl_entry();
     constexpr int TS = 64;
     constexpr int H = (1 << (F + 1)) - 2;
     constexpr int HP = ((H + 3) / 4) * 4;
@@ -484,6 +483,12 @@ __global__ void __launch_bounds__(256, F >= 4 ? 1 : 3)
     float *b0 = align128<float>(smem_raw);  // c_0, c_2, ... (a bulk copy destination)
     float *b1 = b0 + P * P;                 // c_1, c_3, ...
     uint64_t *bar = reinterpret_cast<uint64_t *>(b1 + P * P);
+    if ((use_tma & 1) && threadIdx.x == 0) {
+        mbar_init(bar, 1);
+        tma_prefetch_map(&tmap);
+    }
+    __syncthreads();
+    pdl_entry();
     const long b = blockIdx.x / tiles_per_map;
     const int t = blockIdx.x - (int)(b * tiles_per_map);
     const int ty0 = (t / tiles_x) * TS;
@@ -497,8 +502,6 @@ __global__ void __launch_bounds__(256, F >= 4 ? 1 : 3)
         // (use_tma bit 1, a test hook: 16 bytes more are announced than the
         // copy delivers, so the bounded wait runs out and is flagged).  Box
         // columns and rows outside the map arrive as zeros.
-        if (threadIdx.x == 0) mbar_init(bar, 1);
-        __syncthreads();
         if (threadIdx.x == 0) {
             mbar_expect_tx(bar, (uint32_t)(P * P * sizeof(float)) + ((use_tma & 2) ? 16u : 0u));
             tma_load_3d(b0, &tmap, tx0 - HP, ty0 - HP, (int)b, bar);
@@ -782,7 +785,6 @@ __global__ void __launch_bounds__(NT) k_st_scale(const float *c_prev, float *c_n
                                                  float *__restrict__ w_out, long w_bs, int n, int boundary,
                                                  const __grid_constant__ CUtensorMap mc)
 {
-    pdl_entry();
     constexpr int CW = 4 * NT;
     using X = ScaleBox<S, CW>;
     constexpr int RW = X::RW;
@@ -791,10 +793,14 @@ __global__ void __launch_bounds__(NT) k_st_scale(const float *c_prev, float *c_n
     float *sw = align128<float>(smem_raw);  // [KR + 4][RW]
     const int x0 = blockIdx.x * CW;
     const int r0 = blockIdx.y % S, mb = (blockIdx.y / S) * KR;
+    if (threadIdx.x == 0) {
+        mbar_init(&bar, 1);
+        tma_prefetch_map(&mc);
+    }
+    __syncthreads();
+    pdl_entry();
     if (r0 + S * mb >= n) return;  // the whole CTA: no row of this residue left
     const long b = blockIdx.z;
-    if (threadIdx.x == 0) mbar_init(&bar, 1);
-    __syncthreads();
     // one window row per lane of the first warp, after lane 0 announced the bytes
     static_assert(KR + 4 <= 32, "window rows per warp");
     if (threadIdx.x < 32) {
