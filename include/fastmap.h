@@ -92,7 +92,9 @@ typedef struct {
                        serves as scratch until its final write), 4 = one
                        pass per scale that row-filters c_{j-1} from shared
                        memory (fp32, n a multiple of 4, scales with spacing
-                       4..128 px; the form 1 for the others) */
+                       4..128 px; the form 1 for the others); in fp64,
+                       automatic or 4: one pass for every scale that an
+                       explicit fuse_depth leaves (n even) */
 } fm_config;
 
 /* ---- Kaiser-Squires (Sec. 4.5) ---------------------------------------------

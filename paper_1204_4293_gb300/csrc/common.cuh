@@ -33,10 +33,9 @@ extern std::atomic<int64_t> g_launches;
 void prof_before(int kid, cudaStream_t s);
 void prof_after(int kid, cudaStream_t s);
 
-// Programmatic dependent launch: every kernel of the library starts with
-// pdl_entry(), which waits until the kernel it depends on in the stream has
-// finished (a no-op when launched without the attribute) and then lets the
-// next kernel's CTAs be scheduled into SMs this grid leaves idle in its tail.
+// Programmatic dependent launch: every kernel of the library waits in
+// pdl_entry() (or pdl_wait()) until the kernel before it in the stream has
+// finished (a no-op when launched without the attribute).
 extern std::atomic<int> g_pdl;
 // fp32 fused-scale tile kernel: 0 = shared row-filtered buffer, 1 = register
 // window, -1 = automatic (the autotuned plan, else the register window)
@@ -60,11 +59,27 @@ int einval(const std::string &msg);  // records msg as the last error, returns F
 // Kernels that stage by bulk copies do what touches no other kernel's results
 // first (barrier initialisation, the tensor maps' prefetch), so that it runs
 // while the kernel before drains.
+__device__ __forceinline__ void pdl_wait()
+{
+#if defined(__CUDA_ARCH__) && __CUDA_ARCH__ >= 900
+    cudaGridDependencySynchronize();
+#endif
+}
+// pdl_entry() also lets the next kernel's CTAs onto the SMs at once, where that
+// is worth it: beside a tiny grid there are free SMs, and behind one of several
+// CTAs an SM, as a chunk's kernels have, they fill its tail.  Behind a grid of
+// about one CTA an SM they crowd onto the SMs that happen to have room and stay
+// there, and the next kernel runs unevenly.  With the early trigger everywhere
+// / nowhere (us): one 256^2 map 27 / 30, one 1024^2 map 54.7 / 42.9, 32 maps of
+// 1024^2 (chunks of 4 on two streams) 538 / 541, one 8192^2 map (4096 CTAs and
+// more) 1896 / 1877.  The fp64 kernels, whose SMs are busy with few warps, never
+// trigger early (one 1024^2 map 614 / 420).
 __device__ __forceinline__ void pdl_entry()
 {
 #if defined(__CUDA_ARCH__) && __CUDA_ARCH__ >= 900
     cudaGridDependencySynchronize();
-    cudaTriggerProgrammaticLaunchCompletion();
+    const unsigned ctas = gridDim.x * gridDim.y * gridDim.z;
+    if (ctas <= 64u || (ctas >= 512u && ctas < 4096u)) cudaTriggerProgrammaticLaunchCompletion();
 #endif
 }
 
@@ -209,6 +224,10 @@ int launch_fft_op(const void *in1, const void *in2, long in_bstride, void *out1,
 int launch_fft32(const float *in1, const float *in2, long in_bs, float *out1, float *out2, float2 *work, int n,
                  int batch, int op, const float2 *filt, float out_scale, const uint64_t *seed, int r0, bool rotate,
                  const float2 *tw, const float2 *tw2, cudaStream_t s);
+// the fp64 form, n = 64 .. 2048 (fft64.cu)
+int launch_fft64(const double *in1, const double *in2, long in_bs, double *out1, double *out2, double2 *work, int n,
+                 int batch, int op, const double2 *filt, double out_scale, const uint64_t *seed, int r0, bool rotate,
+                 const double2 *tw, const double2 *tw2, cudaStream_t s);
 // inverse KS with a real output (kappa_E only) through the half spectrum
 // (FM_TUNE_KS_REAL): -1 = by size (default), 0 = never, 1 = whenever
 // possible (fp32, n >= 64)

@@ -1,5 +1,7 @@
 // fft.cu -- batched 2-D FFT staged in shared memory, with the Kaiser-Squires
-// multiplier fused between the column passes (Sec. 4.5).
+// multiplier fused between the column passes (Sec. 4.5), for the sizes that
+// the register-resident transforms (fft32.cu, fft64.cu) leave out; and the
+// dispatch to those.
 //
 // Three kernels per transform, each one HBM read and one HBM write:
 //   rows_fwd : pack (gamma1 + i gamma2) [optionally rotated by a per-pixel
@@ -282,6 +284,18 @@ int launch_fft_op(const void *in1, const void *in2, long in_bstride, void *out1,
                   int batch, int precision, int op, const void *filt, double out_scale, const uint64_t *rot_seed, int rot_r0,
                   bool rotate, cudaStream_t s, bool real_ok)
 {
+    if (precision == FM_F64 && n >= 64 && n <= 2048) {  // register-resident radix-8 path (fft64.cu)
+        int st = FM_OK;
+        const double2 *tw = static_cast<const double2 *>(twiddles(n, FM_F64, s, &st));
+        if (!tw) return st;
+        const double2 *tw2 = nullptr;  // the half-length table of the real-output inverse
+        if (op == FFT_OP_KS_INV && !out2 && g_ks_real.load(std::memory_order_relaxed) != 0 &&
+            !(tw2 = static_cast<const double2 *>(twiddles(n / 2, FM_F64, s, &st))))
+            return st;
+        return launch_fft64((const double *)in1, (const double *)in2, in_bstride, (double *)out1, (double *)out2,
+                            (double2 *)work, n, batch, op, (const double2 *)filt, out_scale, rot_seed, rot_r0, rotate,
+                            tw, tw2, s);
+    }
     if (precision == FM_F64)
         return ks_impl<double>((const double *)in1, (const double *)in2, in_bstride, (double *)out1, (double *)out2,
                                (double2 *)work, n, batch, op, (const double2 *)filt, out_scale, rot_seed, rot_r0,

@@ -1,6 +1,7 @@
-// fft32_tables.cuh -- pass structure and twiddle tables of the fp32
-// register-resident FFT (fft32.cu), shared by the kernels and by the host
-// code that fills the tables (runtime.cu, noalloc.cu).
+// fft32_tables.cuh -- pass structure and twiddle tables of the
+// register-resident FFTs (fft32.cu; fft64.cu shares the tables' layout), for
+// the kernels and for the host code that fills the tables (runtime.cu,
+// noalloc.cu).
 //
 // A table for length n holds the natural table exp(-2 pi i t / n), t = 0 ..
 // n - 1, and after it one block per Stockham pass p >= 1 with the twiddles in
@@ -37,23 +38,32 @@ template <int LOGN> struct FftPlan {
     __host__ __device__ static constexpr int pass_off(int p) { return (1 << (LOGE * p)) - E; }
 };
 
-// the natural table and the blocks of passes 1 .. (their sizes sum to n - E)
-inline int fft32_table_elems(int n) { return 2 * n - (1 << fft_log_e(ilog2((unsigned)n))); }
+// fp64 (fft64.cu): radix 8 throughout
+constexpr int kFft64LogE = 3;
 
-// fills fft32_table_elems(n) entries (FP64 on the host, rounded once)
-inline void fft32_fill_table(int n, float2 *t)
+// elements of a table: the natural one and the blocks of passes 1 .. (their
+// sizes sum to n - E)
+inline int fft_table_elems(int n, int loge) { return 2 * n - (1 << loge); }
+inline int fft32_table_elems(int n) { return fft_table_elems(n, fft_log_e(ilog2((unsigned)n))); }
+
+// fills fft_table_elems(n, loge) entries (FP64 on the host, rounded once)
+template <typename V> inline void fft_fill_table(int n, int loge, V *t)
 {
     auto w = [n](long e) {
         const double ang = -2.0 * M_PI * (double)(e % n) / (double)n;
-        return make_float2((float)cos(ang), (float)sin(ang));
+        V v;
+        v.x = (decltype(v.x))cos(ang);
+        v.y = (decltype(v.y))sin(ang);
+        return v;
     };
     for (int i = 0; i < n; ++i) *t++ = w(i);
-    const int logn = ilog2((unsigned)n), loge = fft_log_e(logn), np = (logn + loge - 1) / loge;
+    const int logn = ilog2((unsigned)n), np = (logn + loge - 1) / loge;
     for (int p = 1; p < np; ++p) {
         const int ns = 1 << (loge * p), radix = p + 1 < np ? 1 << loge : n / ns;
         for (int r = 1; r < radix; ++r)
             for (int k = 0; k < ns; ++k) *t++ = w((long)r * k * (n / (ns * radix)));
     }
 }
+inline void fft32_fill_table(int n, float2 *t) { fft_fill_table(n, fft_log_e(ilog2((unsigned)n)), t); }
 
 }  // namespace fm

@@ -95,12 +95,12 @@ std::unordered_map<uint64_t, void *> g_tw;  // key: device, precision, n
 
 static const void *twiddles_one(int n, int precision, cudaStream_t s, int *status);
 
-// The table of n and, for fp32 n >= 64, the one of n / 2 as well, which the
+// The table of n and, for n >= 64, the one of n / 2 as well, which the
 // real-output inverse transform uses: both exist once this returns, so a call
 // before a stream capture leaves nothing to allocate inside it.
 const void *twiddles(int n, int precision, cudaStream_t s, int *status)
 {
-    if (precision == FM_F32 && n >= 64 && !twiddles_one(n / 2, precision, s, status)) return nullptr;
+    if (n >= 64 && !twiddles_one(n / 2, precision, s, status)) return nullptr;
     return twiddles_one(n, precision, s, status);
 }
 
@@ -117,25 +117,23 @@ static const void *twiddles_one(int n, int precision, cudaStream_t s, int *statu
     auto it = g_tw.find(key);
     if (it != g_tw.end()) return it->second;
     // exp(-2 pi i t / n) in FP64 on the host, rounded once to the element type;
-    // fp32 lengths of the register-resident FFT carry its pass tables as well
+    // lengths of the register-resident FFTs carry their pass tables as well
     std::vector<unsigned char> host;
-    if (precision == FM_F32 && n >= 32) {
-        host.resize((size_t)fft32_table_elems(n) * sizeof(float2));
-        fft32_fill_table(n, reinterpret_cast<float2 *>(host.data()));
+    if (precision == FM_F32) {
+        host.resize((size_t)(n >= 32 ? fft32_table_elems(n) : n) * sizeof(float2));
+        float2 *t = reinterpret_cast<float2 *>(host.data());
+        if (n >= 32)
+            fft32_fill_table(n, t);
+        else
+            for (int i = 0; i < n; ++i)
+                t[i] = make_float2((float)cos(-2.0 * M_PI * i / n), (float)sin(-2.0 * M_PI * i / n));
     } else {
-        const size_t esz = precision == FM_F64 ? 16 : 8;
-        host.resize((size_t)n * esz);
-        for (int t = 0; t < n; ++t) {
-            const double ang = -2.0 * M_PI * (double)t / (double)n;
-            const double c = cos(ang), sn = sin(ang);
-            if (precision == FM_F64) {
-                double v[2] = {c, sn};
-                memcpy(&host[(size_t)t * esz], v, esz);
-            } else {
-                float v[2] = {(float)c, (float)sn};
-                memcpy(&host[(size_t)t * esz], v, esz);
-            }
-        }
+        host.resize((size_t)(n >= 32 ? fft_table_elems(n, kFft64LogE) : n) * sizeof(double2));
+        double2 *t = reinterpret_cast<double2 *>(host.data());
+        if (n >= 32)
+            fft_fill_table(n, kFft64LogE, t);
+        else
+            for (int i = 0; i < n; ++i) t[i] = make_double2(cos(-2.0 * M_PI * i / n), sin(-2.0 * M_PI * i / n));
     }
     void *d = nullptr;
     e = dev_malloc(&d, host.size());

@@ -879,6 +879,105 @@ __global__ void __launch_bounds__(NT) k_st_scale(const float *c_prev, float *c_n
 }
 
 // ---------------------------------------------------------------------------
+// One scale in one pass, fp64, any spacing.  A warp owns 64 columns (two a
+// lane) and KR output rows at stride s: it row-filters its KR + 4 window rows
+// of c_{j-1} straight from global memory (L1 and L2 serve the taps) into a
+// five-row register window and filters that down the column, like k_st_scale.
+// What bounds it is the FP64 pipe (one warp instruction in 16 cycles or more an
+// SM): 4 operations a filter (taps 1, 4, 6, 4, 1), 1.25 row filters and one
+// column filter a pixel, one difference; the scaling by 1 / 256 works on the
+// exponent field.  A tile of three fused scales computes its halo again (2.39 M
+// FP64 warp instructions for 1024^2 against 1.0 M), and a row and a column pass
+// read and write the row-filtered map.  No shared memory and one-warp CTAs, so
+// that the few hundred of a single map spread evenly.  One 1024^2 map, J = 7: the
+// starlet 257 -> 164 us (fused tile of three scales 158, a large scale 32, now
+// 30 each).
+__device__ __forceinline__ double tap5(double a, double b, double c, double d, double e)
+{
+    return fma(6.0, c, fma(4.0, b + d, a + e));
+}
+__device__ __forceinline__ double over256(double v)
+{
+    const int hi = __double2hiint(v), ex = hi & 0x7ff00000;
+    // normal before and after: subtract 8 from the exponent field
+    if (ex >= 0x00900000 && ex != 0x7ff00000) return __hiloint2double(hi - 0x00800000, __double2loint(v));
+    return v * (1.0 / 256.0);
+}
+template <int KR, int SMALL>  // SMALL: spacing 1 (taps within three vectors), else any even spacing
+__global__ void __launch_bounds__(32) k_st_scale64(const double *__restrict__ c_prev, long prev_bs,
+                                                   double *__restrict__ c_next, long next_bs,
+                                                   double *__restrict__ w_out, long w_bs, int n, int s_arg, int boundary)
+{
+    pdl_wait();
+    const int s = SMALL ? 1 : s_arg;
+    const int x = (blockIdx.x * 32 + threadIdx.x) * 2;  // n is even: both columns are inside or outside
+    const int r0 = blockIdx.y % s, mb = (blockIdx.y / s) * KR;
+    const int rows = r0 + s * mb < n ? (n - 1 - r0) / s - mb + 1 : 0;  // of this residue, from mb on
+    if (x >= n || rows == 0) return;
+    const long b = blockIdx.z;
+    const double *cb = c_prev + b * prev_bs;
+    const bool inner = x >= 2 * s && x + 2 + 2 * s <= n;
+    // columns of the taps, folded once for all rows (edge lanes)
+    int xm2[2], xm1[2], xp1[2], xp2[2];
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+        xm2[u] = fold_index(x + u - 2 * s, n, boundary);
+        xm1[u] = fold_index(x + u - s, n, boundary);
+        xp1[u] = fold_index(x + u + s, n, boundary);
+        xp2[u] = fold_index(x + u + 2 * s, n, boundary);
+    }
+    const long px0 = (long)(r0 + s * mb) * n + x;
+    double *wp = w_out + b * w_bs + px0, *cp = c_next ? c_next + b * next_bs + px0 : nullptr;
+    const long step = (long)s * n;
+    auto v2 = [](const double *p) { return __ldg(reinterpret_cast<const double2 *>(p)); };
+    double win[5][2], ctr[3][2];
+#pragma unroll
+    for (int t = 0; t < KR + 4; ++t) {
+        if (t - 4 >= rows) break;  // the last row's window is complete
+        const double *row = cb + (long)fold_index(r0 + s * (mb + t - 2), n, boundary) * n;
+        const double2 c0 = v2(row + x);
+        double2 m2, m1, p1, p2;
+        if (inner) {
+            if constexpr (SMALL) {
+                const double2 l = v2(row + x - 2), r = v2(row + x + 2);
+                m2 = l;
+                m1 = make_double2(l.y, c0.x);
+                p1 = make_double2(c0.y, r.x);
+                p2 = r;
+            } else {
+                m2 = v2(row + x - 2 * s);
+                m1 = v2(row + x - s);
+                p1 = v2(row + x + s);
+                p2 = v2(row + x + 2 * s);
+            }
+        } else {
+            m2 = make_double2(__ldg(row + xm2[0]), __ldg(row + xm2[1]));
+            m1 = make_double2(__ldg(row + xm1[0]), __ldg(row + xm1[1]));
+            p1 = make_double2(__ldg(row + xp1[0]), __ldg(row + xp1[1]));
+            p2 = make_double2(__ldg(row + xp2[0]), __ldg(row + xp2[1]));
+        }
+        win[t % 5][0] = tap5(m2.x, m1.x, c0.x, p1.x, p2.x);
+        win[t % 5][1] = tap5(m2.y, m1.y, c0.y, p1.y, p2.y);
+        ctr[t % 3][0] = c0.x;
+        ctr[t % 3][1] = c0.y;
+        if (t >= 4) {
+            const int k = t - 4;
+            double cj[2], w[2];
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                cj[u] = over256(tap5(win[k % 5][u], win[(k + 1) % 5][u], win[(k + 2) % 5][u], win[(k + 3) % 5][u],
+                                     win[(k + 4) % 5][u]));
+                w[u] = ctr[(k + 2) % 3][u] - cj[u];
+            }
+            __stcs(reinterpret_cast<double2 *>(wp), make_double2(w[0], w[1]));
+            if (cp) *reinterpret_cast<double2 *>(cp) = make_double2(cj[0], cj[1]);
+            wp += step;
+            if (cp) cp += step;
+        }
+    }
+}
+
+// ---------------------------------------------------------------------------
 // Column pass of large scale j fused with the row pass of scale j + 1.  A CTA
 // owns KR whole rows y_k = r0 + s (m KR + k) of one map (rows at the stride s
 // of scale j, like k_st_col): each thread runs the column filter down CPT
@@ -1324,12 +1423,21 @@ static int starlet_impl(const T *kappa, T *pyr, long pyr_bs, int n, int J, int b
     constexpr int VW = 16 / sizeof(T);
     constexpr int KR = 8;
     const long nn = (long)n * n;
-    const int f = auto_fuse(n, J, cfg);
+    int f = auto_fuse(n, J, cfg);
     const int bnd = cfg.boundary;
     T *A = scratch;
     T *Bb = scratch ? scratch + (long)batch * nn : nullptr;
     T *last = pyr + (long)(J - 1) * nn;  // slot of the smooth array
     const bool vec_ok = n % VW == 0 && aligned16(kappa) && aligned16(pyr) && (!scratch || aligned16(scratch));
+    // fp64: one pass a scale (k_st_scale64) for all scales, or for those after
+    // an explicit depth, unless another large path or the plain form
+    // (fuse_depth -1) is asked for
+    TunedPlan plan64;
+    const bool one_pass64 =
+        sizeof(T) == 8 && vec_ok && Bb && batch <= 65535 &&
+        (cfg.large_path == 4 || (cfg.large_path == 0 && cfg.fuse_depth >= 0 &&
+                                 (!tune_lookup(n, J, cfg.precision, &plan64) || plan64.large_path == 4)));
+    if (one_pass64 && cfg.fuse_depth == 0) f = 0;
     if (f >= 1) {
         T *c_out = f == J - 1 ? (bands_only ? nullptr : last) : A;
         const long c_bs = f == J - 1 ? pyr_bs : nn;
@@ -1391,6 +1499,26 @@ static int starlet_impl(const T *kappa, T *pyr, long pyr_bs, int n, int J, int b
         }
         if (j0 > J - 1) return FM_OK;
         if (c_in == Bb) std::swap(A, Bb);  // the passes below keep c in A
+    } else {
+        if (one_pass64) {  // c_j alternates as above
+            for (; j0 <= J - 1; ++j0) {
+                const int sp = 1 << (j0 - 1);
+                T *dst = j0 == J - 1 ? (bands_only ? nullptr : last) : (c_in == A ? Bb : A);
+                // 16 output rows a warp where that still leaves six warps an SM, else 8
+                // or 4 (more row filters a pixel, shorter chains): 1 x 256^2 J = 6
+                // starlet with 16 / 8 rows 100 / 58 us, 8 x 1024^2 J = 7 1120 / 1170
+                const long w16 = (long)batch * ((n + 63) / 64) * ((n + 15) / 16);
+                const int kr = w16 >= 6 * 152 ? 16 : w16 >= 6 * 38 ? 8 : 4;
+                const dim3 grid((n + 63) / 64, sp * ((((n + sp - 1) / sp) + kr - 1) / kr), batch);
+                auto k = kr == 16  ? (sp == 1 ? k_st_scale64<16, 1> : k_st_scale64<16, 0>)
+                         : kr == 8 ? (sp == 1 ? k_st_scale64<8, 1> : k_st_scale64<8, 0>)
+                                   : (sp == 1 ? k_st_scale64<4, 1> : k_st_scale64<4, 0>);
+                FM_LAUNCH(FM_K_STARLET_COL, k, grid, 32, 0, s, (const double *)c_in, nn, (double *)dst,
+                          j0 == J - 1 ? pyr_bs : nn, (double *)(pyr + (long)(j0 - 1) * nn), pyr_bs, n, sp, bnd);
+                c_in = dst;
+            }
+            return FM_OK;
+        }
     }
     const unsigned gx = (unsigned)((n + 128 * VW - 1) / (128 * VW));
     // row pass: up to 256 threads (1024 fp32 pixels) of one row per CTA, so
