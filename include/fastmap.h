@@ -222,7 +222,7 @@ int fm_noise_finalize(const double *sums, const void *pyramid, double *var_out, 
  * Needs the periodic boundary (cfg->boundary = FM_PERIODIC; mirror edges make
  * the pipeline position dependent, FM_EINVAL).  var_out [(J-1)][n][n] in the
  * element type of cfg->precision; one map; n a power of two.  Scratch:
- * about (2J + 6J) n^2 elements, stream-ordered. */
+ * about (4J + 8) n^2 elements, stream-ordered. */
 int fm_map_noise_expected(const void *g1, const void *g2, void *var_out, int n, int J, const fm_config *cfg,
                           void *stream);
 

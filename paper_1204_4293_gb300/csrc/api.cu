@@ -257,9 +257,14 @@ int fm_noise_finalize(const double *sums, const void *pyramid, double *var_out, 
 // Exact expected noise variance (Sec. 1), periodic boundary:
 // Var_j = 1/2 |K_j|^2 (*) |gamma|^2 (circular convolution).  K_j is the
 // pipeline's response to unit shears at pixel 0 (Re K_j from gamma1, -Im K_j
-// from gamma2); the convolution runs through the FFT pipeline: the spectra of
-// |K_j|^2, then rows FFT of |gamma|^2 (broadcast to the J - 1 bands) -> columns
-// FFT -> times the band's spectrum -> inverse -> real part / 2.
+// from gamma2); the convolutions run through the FFT pipeline, two bands at a
+// time: the spectrum of |gamma|^2 once, then rows FFT of |K_j|^2 + i |K_j+h|^2
+// -> columns FFT -> times that spectrum -> inverse, whose real and imaginary
+// parts are the bands j and j + h (|gamma|^2 is real).  Band j + h enters
+// times 4^h, which brings it to band j's magnitude (a band's response power
+// falls by about 4 a scale), so that its rounding is relative to itself; both
+// powers of two are exact.  One spectrum and (J - 1) / 2 filter passes instead
+// of J - 1 of each: 1024^2, J = 7 214 -> 158 us, its error against FP64 unchanged.
 int fm_map_noise_expected(const void *g1, const void *g2, void *var_out, int n, int J, const fm_config *cfgp,
                           void *stream)
 {
@@ -278,22 +283,30 @@ int fm_map_noise_expected(const void *g1, const void *g2, void *var_out, int n, 
     const long nn = (long)n * n;
     const int nb = J - 1;
     auto up = [](size_t b) { return (b + 255) / 256 * 256; };
+    const int h = nb / 2, pairs = nb - h;  // bands 0 .. h - 1 with pairs .. nb - 1; band h alone where nb is odd
     const size_t b_delta = up(2 * nn * es), b_pyr = up((size_t)2 * J * nn * es), b_q = up((size_t)nb * nn * es),
-                 b_p = up(nn * es), b_spec = up((size_t)nb * nn * 2 * es);
+                 b_p = up(nn * es), b_spec = up((size_t)nn * 2 * es), b_work = up((size_t)pairs * nn * 2 * es);
     Scratch sc;
-    if ((st = scratch_alloc(sc, 2 * b_delta + b_pyr + b_q + b_p + 2 * b_spec, s))) return st;
+    if ((st = scratch_alloc(sc, 2 * b_delta + b_pyr + b_q + b_p + b_spec + b_work, s))) return st;
     char *base = static_cast<char *>(sc.p);
     char *g1d = base, *g2d = g1d + b_delta, *pyr = g2d + b_delta, *q = pyr + b_pyr, *p = q + b_q, *spec = p + b_p,
          *work = spec + b_spec;
     if ((st = launch_unit_shears(g1d, g2d, nn, prec, s))) return st;
     if ((st = map_starlet_run(g1d, g2d, pyr, n, J, 2, cfg, s))) return st;
     // |K_j|^2 = (Re K_j)^2 + (Im K_j)^2 from the two responses [2][J][n][n]
-    if ((st = launch_modulus2(pyr, nn, pyr + (size_t)J * nn * es, nn, q, nn, nb, prec, s))) return st;
-    if ((st = launch_modulus2(g1, 0, g2, 0, p, nn, 1, prec, s))) return st;
-    if ((st = launch_fft_op(q, nullptr, nn, nullptr, nullptr, spec, n, nb, prec, FFT_OP_SPECTRUM, nullptr, 1.0, 0, 0,
+    const double up4 = ldexp(1.0, 2 * pairs);  // 4^pairs
+    if ((st = launch_modulus2(pyr, nn, pyr + (size_t)J * nn * es, nn, q, nn, nb, pairs, up4, prec, s))) return st;
+    if ((st = launch_modulus2(g1, 0, g2, 0, p, nn, 1, 1, 1.0, prec, s))) return st;
+    if ((st = launch_fft_op(p, nullptr, nn, nullptr, nullptr, spec, n, 1, prec, FFT_OP_SPECTRUM, nullptr, 1.0, 0, 0,
                             false, s)))
         return st;
-    return launch_fft_op(p, nullptr, 0, var_out, nullptr, work, n, nb, prec, FFT_OP_FILTER, spec, 0.5, 0, 0, false, s);
+    char *var = static_cast<char *>(var_out), *q2 = q + (size_t)pairs * nn * es;
+    if (h > 0 && (st = launch_fft_op(q, q2, nn, var, var + (size_t)pairs * nn * es, work, n, h, prec, FFT_OP_FILTER,
+                                     spec, 0.5, 0, 0, false, s, false, 1.0 / up4)))
+        return st;
+    if (h == pairs) return FM_OK;
+    return launch_fft_op(q + (size_t)h * nn * es, nullptr, nn, var + (size_t)h * nn * es, nullptr, work, n, 1, prec,
+                         FFT_OP_FILTER, spec, 0.5, 0, 0, false, s);
 }
 
 int fm_band_moments(const void *pyramid, double *moments, int n, int J, int batch, const fm_config *cfgp,

@@ -290,7 +290,7 @@ template <int LOGN, bool WITH_B>
 __global__ void __launch_bounds__(Plan32<LOGN>::ROW_T, Plan32<LOGN>::ROW_MINB)
     k_rows_inv32(const float2 *__restrict__ work, float *__restrict__ out1,
                                                        float *__restrict__ out2, long total_rows,
-                                                       const float2 *__restrict__ tw, float scale,
+                                                       const float2 *__restrict__ tw, float scale, float im_scale,
                                                        const __grid_constant__ CUtensorMap mw, int use_tma)
 {
     using P = Plan32<LOGN>;
@@ -334,7 +334,7 @@ __global__ void __launch_bounds__(Plan32<LOGN>::ROW_T, Plan32<LOGN>::ROW_MINB)
                 const long pos = row * P::N + j + q * P::TV;
                 const float2 x = v[q];
                 out1[pos] = x.x * scale;
-                if constexpr (WITH_B) out2[pos] = x.y * scale;
+                if constexpr (WITH_B) out2[pos] = x.y * im_scale;
             }
     }
 }
@@ -391,10 +391,10 @@ __global__ void __launch_bounds__(Plan32<LOGN>::COL_T, Plan32<LOGN>::COL_MINB)
     }
     // kappa_hat = conj(D) gamma_hat (inverse KS) or D kappa_hat (forward KS),
     // D = (k1^2 - k2^2 + 2 i k1 k2) / (k1^2 + k2^2), D(0) = 0; or the given
-    // spectrum filt[b][ky][kx]
+    // spectrum filt[ky][kx]
     const int xi = x0 + c;
     const float k1 = (float)(xi < N / 2 ? xi : xi - N), jf = (float)j;
-    const float2 *fb = filt ? filt + b * (long)N * N + xi : nullptr;
+    const float2 *fb = filt ? filt + xi : nullptr;
 #pragma unroll
     for (int q = 0; q < P::E; ++q) {
         float2 d;
@@ -725,7 +725,7 @@ static int ks32_real_impl(const float *in1, const float *in2, long in_bs, float 
 template <int LOGN>
 static int ks32_impl(const float *in1, const float *in2, long in_bs, float *out1, float *out2, float2 *work, int batch,
                      int op, const float2 *filt, float out_scale, const uint64_t *seed, int r0, bool rotate,
-                     const float2 *tw, const float2 *tw2, cudaStream_t s)
+                     const float2 *tw, const float2 *tw2, cudaStream_t s, float im_scale)
 {
     if constexpr (LOGN >= 6) {
         if (op == FFT_OP_KS_INV && !out2 && tw2 && (reinterpret_cast<uintptr_t>(out1) & 15) == 0)
@@ -798,7 +798,7 @@ static int ks32_impl(const float *in1, const float *in2, long in_bs, float *out1
     if (op == FFT_OP_SPECTRUM) return FM_OK;
     const float scale = out_scale / ((float)P::N * (float)P::N);
     FM_LAUNCH(FM_K_FFT_ROWS_INV, kri, row_grid, RPC * P::TV, row_smem, s, work, out1, out2, total_rows, tw, scale,
-              mw, tma_out);
+              scale * im_scale, mw, tma_out);
     return FM_OK;
 }
 
@@ -806,10 +806,10 @@ static int ks32_impl(const float *in1, const float *in2, long in_bs, float *out1
 // which then uses the generic shared-memory Stockham kernels.
 int launch_fft32(const float *in1, const float *in2, long in_bs, float *out1, float *out2, float2 *work, int n,
                  int batch, int op, const float2 *filt, float out_scale, const uint64_t *seed, int r0, bool rotate,
-                 const float2 *tw, const float2 *tw2, cudaStream_t s)
+                 const float2 *tw, const float2 *tw2, cudaStream_t s, float im_scale)
 {
 #define FM_KS32(L) \
-    ks32_impl<L>(in1, in2, in_bs, out1, out2, work, batch, op, filt, out_scale, seed, r0, rotate, tw, tw2, s)
+    ks32_impl<L>(in1, in2, in_bs, out1, out2, work, batch, op, filt, out_scale, seed, r0, rotate, tw, tw2, s, im_scale)
     switch (n) {
     case 32: return FM_KS32(5);
     case 64: return FM_KS32(6);

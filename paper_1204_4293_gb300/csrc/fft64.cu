@@ -181,7 +181,7 @@ __global__ void __launch_bounds__(Plan64<LOGN>::ROW_T)
 template <int LOGN, bool WITH_B>
 __global__ void __launch_bounds__(Plan64<LOGN>::ROW_T)
     k_rows_inv64(const double2 *__restrict__ work, double *__restrict__ out1, double *__restrict__ out2,
-                 long total_rows, const double2 *__restrict__ tw, double scale)
+                 long total_rows, const double2 *__restrict__ tw, double scale, double im_scale)
 {
     pdl_wait();
     using P = Plan64<LOGN>;
@@ -198,7 +198,7 @@ __global__ void __launch_bounds__(Plan64<LOGN>::ROW_T)
     for (int q = 0; q < 8; ++q) {
         const long pos = row * P::N + j + q * P::TV;
         out1[pos] = v[q].x * scale;
-        if constexpr (WITH_B) out2[pos] = v[q].y * scale;
+        if constexpr (WITH_B) out2[pos] = v[q].y * im_scale;
     }
 }
 
@@ -220,7 +220,7 @@ __global__ void __launch_bounds__(Plan64<LOGN>::W *Plan64<LOGN>::TV)
     fft_vec<LOGN, W, false>(v, smd, c, j, tw);
     if (op != FFT_OP_SPECTRUM) {
         const int xi = x0 + c, k1 = xi < N / 2 ? xi : xi - N;
-        const double2 *fb = filt ? filt + b * (long)N * N + xi : nullptr;
+        const double2 *fb = filt ? filt + xi : nullptr;
 #pragma unroll
         for (int q = 0; q < 8; ++q) {
             double2 d;
@@ -358,7 +358,7 @@ __global__ void __launch_bounds__(Plan64<LOGN - 1>::ROW_T)
 template <int LOGN>
 static int impl64(const double *in1, const double *in2, long in_bs, double *out1, double *out2, double2 *work, int batch,
            int op, const double2 *filt, double out_scale, const uint64_t *seed, int r0, bool rotate, const double2 *tw,
-           const double2 *tw2, cudaStream_t s)
+           const double2 *tw2, cudaStream_t s, double im_scale)
 {
     using P = Plan64<LOGN>;
     using P2 = Plan64<LOGN - 1>;
@@ -394,15 +394,15 @@ static int impl64(const double *in1, const double *in2, long in_bs, double *out1
               filt);
     if (op == FFT_OP_SPECTRUM) return FM_OK;
     FM_LAUNCH(FM_K_FFT_ROWS_INV, ki, row_grid, P::ROW_T, row_smem, s, (const double2 *)work, out1, out2, rows, tw,
-              scale);
+              scale, scale * im_scale);
     return FM_OK;
 }
 
 int launch_fft64(const double *in1, const double *in2, long in_bs, double *out1, double *out2, double2 *work, int n,
                  int batch, int op, const double2 *filt, double out_scale, const uint64_t *seed, int r0, bool rotate,
-                 const double2 *tw, const double2 *tw2, cudaStream_t s)
+                 const double2 *tw, const double2 *tw2, cudaStream_t s, double im_scale)
 {
-#define FM_FFT64(L) impl64<L>(in1, in2, in_bs, out1, out2, work, batch, op, filt, out_scale, seed, r0, rotate, tw, tw2, s)
+#define FM_FFT64(L) impl64<L>(in1, in2, in_bs, out1, out2, work, batch, op, filt, out_scale, seed, r0, rotate, tw, tw2, s, im_scale)
     switch (n) {
     case 64: return FM_FFT64(6);
     case 128: return FM_FFT64(7);

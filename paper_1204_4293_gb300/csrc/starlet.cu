@@ -837,11 +837,18 @@ __global__ void __launch_bounds__(NT) k_st_scale(const float *c_prev, float *c_n
         } else {
             const float *cb = c_prev + b * (long)n * n;
             for (int h = threadIdx.x; h < 2 * S; h += NT) {
+                float l[KR + 4], r[KR + 4];  // every row's loads in flight together
+#pragma unroll
+                for (int t = 0; t < KR + 4; ++t) {
+                    const float *src = cb + (long)fold_index(r0 + S * (mb + t - 2), n, boundary) * n;
+                    if (x0 == 0) l[t] = src[n - 2 * S + h];
+                    if (h < hr) r[t] = src[h];
+                }
+#pragma unroll
                 for (int t = 0; t < KR + 4; ++t) {
                     float *row = sw + t * RW;
-                    const float *src = cb + (long)fold_index(r0 + S * (mb + t - 2), n, boundary) * n;
-                    if (x0 == 0) row[h] = src[n - 2 * S + h];
-                    if (h < hr) row[e0 + h] = src[h];
+                    if (x0 == 0) row[h] = l[t];
+                    if (h < hr) row[e0 + h] = r[t];
                 }
             }
         }
