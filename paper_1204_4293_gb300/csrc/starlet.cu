@@ -827,11 +827,16 @@ __global__ void __launch_bounds__(NT) k_st_scale(const float *c_prev, float *c_n
         const int e0 = n - x0 + 2 * S;                              // staged index of map column n
         if (boundary != FM_PERIODIC) {
             for (int h = threadIdx.x; h < 2 * S; h += NT) {
+                float l[KR + 4], r[KR + 4];  // every row's loads in flight together
 #pragma unroll
                 for (int t = 0; t < KR + 4; ++t) {
-                    float *row = sw + t * RW;
-                    if (x0 == 0) row[h] = row[4 * S - h];
-                    if (h < hr) row[e0 + h] = row[e0 - 2 - h];
+                    if (x0 == 0) l[t] = sw[t * RW + 4 * S - h];
+                    if (h < hr) r[t] = sw[t * RW + e0 - 2 - h];
+                }
+#pragma unroll
+                for (int t = 0; t < KR + 4; ++t) {
+                    if (x0 == 0) sw[t * RW + h] = l[t];
+                    if (h < hr) sw[t * RW + e0 + h] = r[t];
                 }
             }
         } else {
