@@ -71,6 +71,8 @@ int fm_ks_invert(const void *g1, const void *g2, void *kappa_E, void *kappa_B, i
     if (batch < 1) return einval("batch must be >= 1");
     if (!g1 || !g2 || !kappa_E) return einval("null pointer");
     cudaStream_t s = (cudaStream_t)stream;
+    if (small_map_ok(n, 0, batch, cfg, true))
+        return launch_small_ks((const float *)g1, (const float *)g2, (float *)kappa_E, (float *)kappa_B, n, batch, s);
     Scratch work;
     const size_t bytes = (size_t)batch * n * n * 2 * esize(cfg);
     if ((st = scratch_alloc(work, bytes, s))) return st;
@@ -101,6 +103,8 @@ int fm_starlet_forward(const void *kappa, void *pyramid, int n, int J, int batch
     if (batch < 1) return einval("batch must be >= 1");
     if (!kappa || !pyramid) return einval("null pointer");
     cudaStream_t s = (cudaStream_t)stream;
+    if (small_map_ok(n, J, batch, cfg, (reinterpret_cast<uintptr_t>(pyramid) & 15) == 0))
+        return launch_small_starlet((const float *)kappa, (float *)pyramid, n, J, batch, cfg.boundary, s);
     Scratch sc;
     if ((st = scratch_alloc(sc, starlet_scratch_elems(n, J, batch, cfg) * esize(cfg), s))) return st;
     return launch_starlet(kappa, pyramid, (long)J * n * n, n, J, batch, cfg, sc.p, s);

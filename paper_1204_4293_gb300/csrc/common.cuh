@@ -235,6 +235,12 @@ int launch_fft64(const double *in1, const double *in2, long in_bs, double *out1,
 extern std::atomic<int> g_ks_real;
 bool ks_real_for(int n, bool batched);
 size_t starlet_scratch_elems(int n, int J, int batch, const fm_config &cfg);
+// small maps in one kernel (small.cu); J = 0 for Kaiser-Squires alone
+bool small_map_ok(int n, int J, int batch, const fm_config &cfg, bool aligned);
+int launch_small_map(const float *g1, const float *g2, float *pyr, int n, int J, int batch, int boundary,
+                     cudaStream_t s);
+int launch_small_ks(const float *g1, const float *g2, float *kE, float *kB, int n, int batch, cudaStream_t s);
+int launch_small_starlet(const float *kappa, float *pyr, int n, int J, int batch, int boundary, cudaStream_t s);
 // ---- autotuned plans (tune.cu) ----------------------------------------------------
 // A plan for maps of n^2, J scales, one precision: fused depth, large-scale
 // path (1 or 3), fp32 tile kernel form (1 = register window, 0 = shared

@@ -205,6 +205,8 @@ void drop_graph(GraphEntry &e)
 static int map_starlet_dev(const void *g1, const void *g2, void *pyramid, int n, int J, int batch,
                            const fm_config &cfg, cudaStream_t s, bool allow_graph = true)
 {
+    if (small_map_ok(n, J, batch, cfg, (reinterpret_cast<uintptr_t>(pyramid) & 15) == 0))
+        return launch_small_map((const float *)g1, (const float *)g2, (float *)pyramid, n, J, batch, cfg.boundary, s);
     const ChunkPlan p = plan_chunks(n, J, batch, cfg);
     if (p.C >= batch) {  // one chunk: straight onto the caller's stream
         Scratch sc;
