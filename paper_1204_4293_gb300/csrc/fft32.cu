@@ -335,7 +335,7 @@ __global__ void __launch_bounds__(Plan32<LOGN>::COL_T, Plan32<LOGN>::COL_MINB)
         if (threadIdx.x == 0) {
             for (int k = 0; k < N / BR; ++k) tma_store_3d(&mw, 2 * x0, k * BR, (int)b, sm32 + k * BR * W);
             bulk_commit();
-            bulk_wait_all();
+            bulk_wait_read();
         }
         return;
     }
@@ -375,7 +375,7 @@ template <int LOGN> struct PlanE {
 template <int LOGN>
 __global__ void __launch_bounds__(PlanE<LOGN>::NT, PlanE<LOGN>::MINB)
     k_cols_ks32_e(const float2 *__restrict__ work, float2 *__restrict__ half, const float2 *__restrict__ tw,
-                  const __grid_constant__ CUtensorMap mw, int use_tma)
+                  const __grid_constant__ CUtensorMap mw, const __grid_constant__ CUtensorMap mh, int use_tma)
 {
     using P = Plan32<LOGN>;
     using E = PlanE<LOGN>;
@@ -397,7 +397,7 @@ __global__ void __launch_bounds__(PlanE<LOGN>::NT, PlanE<LOGN>::MINB)
     const int tid = threadIdx.x, hf = tid / NH, t = tid % NH, c = t % WS, j = t / WS;
     float2 *R = hf ? R2 : R1;  // this half's strip and exchange region
     float2 v[P::E];
-    if (use_tma) {
+    if (use_tma & 1) {
         constexpr int BR = N < 256 ? N : 256;  // rows per copy
         if (tid == 0) {
             // the strip, [n][WS] (Gamma1, Gamma2) pairs, over both regions
@@ -475,6 +475,25 @@ __global__ void __launch_bounds__(PlanE<LOGN>::NT, PlanE<LOGN>::MINB)
         }
     }
     fft_vec<LOGN, WS, true, NH>(v, R1, c, j, tw);
+    if constexpr (WS >= 2) {
+        if (use_tma & 2) {
+            // the strip's columns back through shared memory, dense [n][WS], and out
+            // by bulk tensor stores (mh: the half spectrum as floats {n, n, batch},
+            // box {2 WS, min(n, 256), 1})
+            constexpr int BR = N < 256 ? N : 256;
+            part_sync<NH>();  // the last pass may still read the exchange buffer
+#pragma unroll
+            for (int q = 0; q < P::E; ++q) R1[(j + q * P::TV) * WS + c] = v[q];
+            fence_async_smem();
+            part_sync<NH>();
+            if (tid == 0) {
+                for (int k = 0; k < N / BR; ++k) tma_store_3d(&mh, 2 * s0, k * BR, (int)b, R1 + k * BR * WS);
+                bulk_commit();
+                bulk_wait_read();
+            }
+            return;
+        }
+    }
     float2 *dst = half + b * (long)N * (N / 2) + s0 + c;
 #pragma unroll
     for (int q = 0; q < P::E; ++q) dst[(long)(j + q * P::TV) * (N / 2)] = v[q];
@@ -591,7 +610,8 @@ static int ks32_real_impl(const float *in1, const float *in2, long in_bs, float 
     FM_CUDA_TRY(fm::smem_attr((const void *)krf, row_smem));
     FM_CUDA_TRY(fm::smem_attr((const void *)k_cols_ks32_e<LOGN>, col_smem));
     FM_CUDA_TRY(fm::smem_attr((const void *)k_rows_inv32_c2r<LOGN>, row2_smem));
-    CUtensorMap m1, m2, mc, mk;
+    CUtensorMap m1, m2, mc, mk, mh;
+    memset(&mh, 0, sizeof(mh));
     memset(&m1, 0, sizeof(m1));
     memset(&m2, 0, sizeof(m2));
     memset(&mc, 0, sizeof(mc));
@@ -605,7 +625,10 @@ static int ks32_real_impl(const float *in1, const float *in2, long in_bs, float 
         const uint64_t dims[3] = {d0, (uint64_t)(P::N / d0), rows};
         const uint64_t strides[2] = {(uint64_t)d0 * 4, (uint64_t)P::N * 4};
         const uint32_t box[3] = {d0, (uint32_t)(P::N / d0), (uint32_t)RPC};
-        tma_in = (tma_mode & 2) && (in_bs == nn || (in_bs == 0 && RPC <= P::N)) &&
+        // per-thread loads for many rows of up to 1024: the copies only add a pass
+        // through shared memory there (TMA / loads: 32 x 1024^2 538 / 534 us, 64 x
+        // 512^2 268 / 264; 4 x 4096^2 1655 / 1682, one 1024^2 map 42.2 / 43.2)
+        tma_in = (tma_mode & 2) && (P::N > 1024 || row_grid < 512) && (in_bs == nn || (in_bs == 0 && RPC <= P::N)) &&
                  encode_map3d_f32(&m1, in1, dims, strides, box) && (!in2 || encode_map3d_f32(&m2, in2, dims, strides, box));
         // kappa's buffer as rows of n floats (= n/2 float2 of half spectrum)
         if (P2::N >= 64 && (tma_mode & 4)) {
@@ -618,12 +641,21 @@ static int ks32_real_impl(const float *in1, const float *in2, long in_bs, float 
         const uint64_t cdims[3] = {(uint64_t)2 * P::N, (uint64_t)P::N, (uint64_t)batch};
         const uint64_t cstrides[2] = {(uint64_t)P::N * 8, (uint64_t)P::N * P::N * 8};
         const uint32_t cbox[3] = {(uint32_t)(4 * E::WS), (uint32_t)(P::N < 256 ? P::N : 256), 1};
+        // out the same way where a strip has at least 16 bytes a row (per-thread
+        // stores / bulk: 8 x 2048^2 J = 8 646 / 627 us, KS alone 4 x 4096^2 719 / 693,
+        // 32 x 1024^2 J = 7 539 / 536)
         tma_col = encode_map3d_f32(&mc, work, cdims, cstrides, cbox) ? 1 : 0;
+        if (tma_col && (tma_mode & 64) && E::WS >= 2) {
+            const uint64_t hdims[3] = {(uint64_t)P::N, (uint64_t)P::N, (uint64_t)batch};
+            const uint64_t hstrides[2] = {(uint64_t)P::N * 4, (uint64_t)P::N * P::N * 4};
+            const uint32_t hbox[3] = {(uint32_t)(2 * E::WS), (uint32_t)(P::N < 256 ? P::N : 256), 1};
+            if (encode_map3d_f32(&mh, out1, hdims, hstrides, hbox)) tma_col |= 2;
+        }
     }
     FM_LAUNCH(FM_K_FFT_ROWS_FWD, krf, row_grid, RPC * P::TV, row_smem, s, in1, in2, in_bs, work, total_rows, tw, seed,
               r0, m1, m2, tma_in);
     FM_LAUNCH(FM_K_FFT_COLS_KS, k_cols_ks32_e<LOGN>, col_grid, col_threads, col_smem, s, (const float2 *)work,
-              reinterpret_cast<float2 *>(out1), tw, mc, tma_col);
+              reinterpret_cast<float2 *>(out1), tw, mc, mh, tma_col);
     const float scale = out_scale / ((float)P::N * (float)P::N);
     FM_LAUNCH(FM_K_FFT_ROWS_INV, k_rows_inv32_c2r<LOGN>, row2_grid, RPC2 * P2::TV, row2_smem, s, out1, total_rows, tw,
               tw2, scale, mk, tma_out);
@@ -694,10 +726,11 @@ static int ks32_impl(const float *in1, const float *in2, long in_bs, float *out1
         const uint64_t cdims[3] = {(uint64_t)2 * P::N, (uint64_t)P::N, (uint64_t)batch};
         const uint64_t cstrides[2] = {(uint64_t)P::N * 8, (uint64_t)P::N * P::N * 8};
         const uint32_t cbox[3] = {(uint32_t)(2 * P::W), (uint32_t)(P::N < 256 ? P::N : 256), 1};
-        // stores the same way only at n = 8192 (KS + starlet: 1 x 8192^2 3.18 ->
-        // 3.15 ms; 32 x 1024^2 0.813 -> 0.828, 16 x 4096^2 10.95 -> 11.00)
+        // stores the same way at n = 2048 (8 maps with kappa_B 349 -> 335 us) and
+        // 8192; not at 1024 (one map slower) and 4096 (804 -> 813 for 4: one CTA an
+        // SM, whose store nothing overlaps)
         tma_col = encode_map3d_f32(&mc, work, cdims, cstrides, cbox)
-                      ? (1 | ((tma_mode & 64) && P::N >= 8192 ? 2 : 0))
+                      ? (1 | ((tma_mode & 64) && (P::N == 2048 || P::N >= 8192) ? 2 : 0))
                       : 0;
     }
     FM_LAUNCH(FM_K_FFT_ROWS_FWD, krf, row_grid, RPC * P::TV, row_smem, s, in1, in2, in_bs, work, total_rows, tw, seed,

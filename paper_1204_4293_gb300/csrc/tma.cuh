@@ -83,10 +83,10 @@ __device__ __forceinline__ void tma_store_3d(const CUtensorMap *map, int x, int 
 }
 __device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 __device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
-// the issuing thread waits until its committed bulk stores are complete
-// (their shared-memory sources read and their writes performed); the CTA
-// must not exit before the sources have been read
-__device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
+// the issuing thread waits until its committed bulk stores have read their
+// shared-memory sources, which must outlive them; the writes are performed by
+// the end of the grid
+__device__ __forceinline__ void bulk_wait_read() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
 
 __device__ __forceinline__ bool mbar_test_wait(uint64_t *bar, uint32_t parity)
 {
