@@ -29,8 +29,8 @@
 // What bounds it: the FP32 pipe and the shared-memory loads together (1024^2,
 // R = 32: 52.7 M warp FMAs of two lanes, 84 us at two a cycle and SM; ncu: FMA
 // pipe 56 %, shared-memory and L1 data path 69 %, 20 warps an SM).  One 1024^2
-// map, starlet Q theta = 16 (R = 32): 372 -> 209 us; S98 theta = 64 1246 ->
-// 658, masked 3050 -> 866; masked 2 x 1000^2 S98 theta = 16 445 -> 236; fp64
+// map, starlet Q theta = 16 (R = 32): 372 -> 199 us; S98 theta = 64 1246 ->
+// 618, masked 3050 -> 825; masked 2 x 1000^2 S98 theta = 16 445 -> 236; fp64
 // 512^2 S98 theta = 16 3079 -> 472 (the plain sum over all rows, with a CTA's
 // warps sharing each staged row behind a barrier).  16 columns a lane halve
 // the window loads but need 116 to 142 registers: 225 us; groups of four taps
@@ -454,13 +454,16 @@ __global__ void __launch_bounds__(256) k_direct_sum(const T *__restrict__ parts,
 std::atomic<int> g_direct_form{-1};
 
 // Parts of the dy: a function of n and the radius only, so that a map's
-// result does not depend on the maps beside it.  Enough warps for two full
-// loads of the GPU (152 SMs x 20 warps), at least four dy a part, at most 16.
-static int direct_parts(int n, int Ri, int TX)
+// result does not depend on the maps beside it.  Eight full loads of the GPU
+// (152 SMs x 20 warps), so that the last warps to finish are short ones (one
+// 1024^2 map, S98 theta = 64, two / four / eight loads 658 / 644 / 618 us), with
+// at least four dy a part, eight with weights (2 x 1000^2 theta = 16 with four
+// 235 -> 249 us), at most 16.
+static int direct_parts(int n, int Ri, int TX, bool mask)
 {
     const long warps = (long)n * ((n + TX - 1) / TX);
-    long P = (2 * 152 * 20 + warps - 1) / warps;
-    P = std::min<long>({P, 16, (Ri + 1) / 4});
+    long P = (8 * 152 * 20 + warps - 1) / warps;
+    P = std::min<long>({P, 16, (Ri + 1) / (mask ? 8 : 4)});
     return P < 1 ? 1 : (int)P;
 }
 // maps per launch pair when the parts go through scratch: at most 256 MiB of
@@ -488,7 +491,7 @@ static int map_direct_impl(const T *g1, const T *g2, const T *wgt, long w_bs, T 
         for (int dy = 0; dy <= Ri; ++dy) n_r += (dy ? 2 : 1) * (2L * disc_half_width(dy, R2) + 1);
         n_r -= 1;
     }
-    const int P = direct_parts(n, Ri, D::TX), slice = direct_slice(P, n, batch, sizeof(T));
+    const int P = direct_parts(n, Ri, D::TX, MASK), slice = direct_slice(P, n, batch, sizeof(T));
     auto up = [](size_t b) { return ((b + 255) / 256) * 256; };
     const size_t tap_b = up((size_t)(Ri + 1) * tw * sizeof(V)), dx_b = up((size_t)(Ri + 1) * sizeof(int));
     const long nn = (long)n * n;
