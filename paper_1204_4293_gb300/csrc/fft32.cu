@@ -133,7 +133,6 @@ __global__ void __launch_bounds__(Plan32<LOGN>::ROW_T, Plan32<LOGN>::ROW_MINB)
                 const int x = j + r * P::TV;
                 float a = st1[vr * P::N + x];
                 float cc = in2 ? st2[vr * P::N + x] : 0.f;
-                if constexpr (ROT) rotate_shear(a, cc, sd, r0 + b, y, x, P::N);
                 v[r] = make_float2(a, cc);
             }
             staged = true;  // fft_vec's first barrier orders these reads before the exchange writes
@@ -149,12 +148,17 @@ __global__ void __launch_bounds__(Plan32<LOGN>::ROW_T, Plan32<LOGN>::ROW_MINB)
             const int x = j + r * P::TV;
             float a = __ldcs(p1 + x);  // the shear is read once
             float cc = p2 ? __ldcs(p2 + x) : 0.f;
-            if constexpr (ROT) rotate_shear(a, cc, sd, r0 + b, y, x, P::N);
             v[r] = make_float2(a, cc);
         }
     } else if (!staged) {
 #pragma unroll
         for (int r = 0; r < P::E; ++r) v[r] = make_float2(0.f, 0.f);
+    }
+    if constexpr (ROT) {
+        const uint64_t z = rot_state(sd, r0 + (row >> LOGN), (int)(row & (P::N - 1)), P::N) + (uint64_t)j * kGolden;
+#pragma unroll
+        for (int r = 0; r < P::E; r += 2)
+            rotate_shear2(v[r], v[r + 1], z + (uint64_t)(r * P::TV) * kGolden, z + (uint64_t)((r + 1) * P::TV) * kGolden);
     }
     fft_vec<LOGN, 1, false>(v, sm, 0, j, tw);
     if constexpr (SPLIT) {
