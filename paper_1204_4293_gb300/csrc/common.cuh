@@ -287,7 +287,7 @@ int launch_band_moments(const void *pyr, double *moments, int n, int J, int batc
                         cudaStream_t s);
 // acc: FP64 S1, S2 (accum 0) or fp32 Kahan pairs s1, c1, s2, c2 (accum 1), bands * nn elements each
 int launch_noise_accum(const void *pyr, int nb, long pyr_bs, long nn, int bands, void *acc, int precision, int accum,
-                       cudaStream_t s);
+                       bool first, bool beside, cudaStream_t s);
 // the seed into *dseed and, unless d1 is null, the two input maps (bytes each)
 // into the library's copies d1, d2
 int launch_noise_stage(const void *g1, const void *g2, void *d1, void *d2, size_t bytes, uint64_t seed,

@@ -39,16 +39,54 @@ int launch_noise_stage(const void *g1, const void *g2, void *d1, void *d2, size_
     return FM_OK;
 }
 
+// f(the vector at p of every realisation), in order, kAccLoads of them
+// loaded ahead (4 / 8 / 16 at two CTAs an SM, R = 256 of 1024^2: 5701 / 5599 /
+// 5784 us)
+constexpr int kAccLoads = 8;
+template <typename V, typename T, typename F>
+__device__ __forceinline__ void for_realisations(const T *__restrict__ p, int nb, long bs, F &&f)
+{
+    int b = 0;
+    for (; b + kAccLoads <= nb; b += kAccLoads) {
+        V v[kAccLoads];
+#pragma unroll
+        for (int k = 0; k < kAccLoads; ++k) v[k] = __ldcs(reinterpret_cast<const V *>(p + (b + k) * bs));
+#pragma unroll
+        for (int k = 0; k < kAccLoads; ++k) f(v[k]);
+    }
+    for (; b < nb; ++b) f(__ldcs(reinterpret_cast<const V *>(p + b * bs)));
+}
+
+// two neighbouring FP64 sums, as one 16-byte word where they are aligned
+// (`wide`; the caller's own sums need not be); streaming, as they are next
+// used a batch later
+__device__ __forceinline__ void add_sums(double *p, double a, double b, bool first, bool wide)
+{
+    if (wide) {
+        double2 v = make_double2(0.0, 0.0);
+        if (!first) v = __ldcs(reinterpret_cast<const double2 *>(p));
+        __stcs(reinterpret_cast<double2 *>(p), make_double2(v.x + a, v.y + b));
+    } else {
+        p[0] = first ? a : p[0] + a;
+        p[1] = first ? b : p[1] + b;
+    }
+}
+
 // S1 += sum_b w, S2 += sum_b w^2 over a batch of `nb` (<= 32) realisations'
 // pyramids ([nb][J][n][n], bands 0..J-2 used).  The batch's partial sums are
 // formed in the element type (at most 32 terms) and added once to the FP64
 // running sums: GB300's FP64 rate is a small fraction of its FP32 rate, so
 // the FP64 work is two additions per band pixel per batch.  The pyramids are
 // read once with streaming (evict-first) loads, so they do not push the chunk
-// pipeline's intermediates out of L2.
+// pipeline's intermediates out of L2.  The first batch writes the sums
+// (`first`) instead of adding to zeroed ones.  Bound by HBM: 32 realisations
+// of 6 bands of 1024^2 and their sums, 1 GB, in 171 us; R = 100 with the sums'
+// zeroing, their scalar accesses and the S/N's map after the last batch 2427,
+// now 2299 us.
 template <typename T, typename V>
 __global__ void __launch_bounds__(256) k_noise_accum(const T *__restrict__ pyr, int nb, long pyr_bs, long nn,
-                                                     int bands, double *__restrict__ s1, double *__restrict__ s2)
+                                                     int bands, double *__restrict__ s1, double *__restrict__ s2,
+                                                     int first, int wide)
 {
     pdl_entry();
     constexpr int VW = sizeof(V) / sizeof(T);
@@ -58,19 +96,18 @@ __global__ void __launch_bounds__(256) k_noise_accum(const T *__restrict__ pyr, 
         T a[VW], q[VW];
 #pragma unroll
         for (int u = 0; u < VW; ++u) a[u] = q[u] = (T)0;
-        for (int b = 0; b < nb; ++b) {
-            const V v = __ldcs(reinterpret_cast<const V *>(pyr + b * pyr_bs + e));
+        for_realisations<V>(pyr + e, nb, pyr_bs, [&](const V &v) {
             const T *w = reinterpret_cast<const T *>(&v);
 #pragma unroll
             for (int u = 0; u < VW; ++u) {
                 a[u] += w[u];
                 q[u] = fma(w[u], w[u], q[u]);
             }
-        }
+        });
 #pragma unroll
-        for (int u = 0; u < VW; ++u) {
-            s1[e + u] += (double)a[u];
-            s2[e + u] += (double)q[u];
+        for (int u = 0; u < VW; u += 2) {
+            add_sums(s1 + e + u, (double)a[u], (double)a[u + 1], first, wide);
+            add_sums(s2 + e + u, (double)q[u], (double)q[u + 1], first, wide);
         }
     }
 }
@@ -80,7 +117,7 @@ __global__ void __launch_bounds__(256) k_noise_accum(const T *__restrict__ pyr, 
 // s - c; a batch's partial sum a enters as y = a - c, t = s + y,
 // c = (t - s) - y, s = t.  The arrays are s1, c1, s2, c2, each nb floats.
 __global__ void __launch_bounds__(256) k_noise_accum_kahan(const float *__restrict__ pyr, int nb, long pyr_bs,
-                                                           long nn, int bands, float *__restrict__ acc)
+                                                           long nn, int bands, float *__restrict__ acc, int first)
 {
     pdl_entry();
     const long ne = bands * nn;
@@ -88,16 +125,21 @@ __global__ void __launch_bounds__(256) k_noise_accum_kahan(const float *__restri
     float4 *s1 = reinterpret_cast<float4 *>(acc), *c1 = s1 + nq, *s2 = c1 + nq, *c2 = s2 + nq;
     for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < nq; i += (long)gridDim.x * blockDim.x) {
         float a[4] = {0.f, 0.f, 0.f, 0.f}, q[4] = {0.f, 0.f, 0.f, 0.f};
-        for (int b = 0; b < nb; ++b) {
-            const float4 v = __ldcs(reinterpret_cast<const float4 *>(pyr + b * pyr_bs) + i);
+        for_realisations<float4>(pyr + i * 4, nb, pyr_bs, [&](const float4 &v) {
             const float w[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
                 a[u] += w[u];
                 q[u] = fmaf(w[u], w[u], q[u]);
             }
+        });
+        float4 S1 = make_float4(0.f, 0.f, 0.f, 0.f), C1 = S1, S2 = S1, C2 = S1;
+        if (!first) {
+            S1 = s1[i];
+            C1 = c1[i];
+            S2 = s2[i];
+            C2 = c2[i];
         }
-        float4 S1 = s1[i], C1 = c1[i], S2 = s2[i], C2 = c2[i];
         float *ps1 = &S1.x, *pc1 = &C1.x, *ps2 = &S2.x, *pc2 = &C2.x;
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
@@ -117,22 +159,30 @@ __global__ void __launch_bounds__(256) k_noise_accum_kahan(const float *__restri
     }
 }
 
-// acc: FP64 s1, s2 (accum 0) or fp32 s1, c1, s2, c2 (accum 1), bands * nn each
+// acc: FP64 s1, s2 (accum 0) or fp32 s1, c1, s2, c2 (accum 1), bands * nn each;
+// first: they are written, not added to; beside: a full batch of maps runs
+// beside it, so it takes three CTAs an SM instead of sixteen and leaves the
+// maps' kernels room.  A short batch ends before a narrow accumulation does:
+// there it is wide.  1024^2, wide / four / three / two / one CTA an SM: R = 256
+// 5763 / 5754 / 5651 / 5599 / 6402 us, R = 100 2326 / 2314 / 2299 / 2298 / 2526;
+// 512^2, R = 100 545 / 542 / 536 / 558 / 603.
 int launch_noise_accum(const void *pyr, int nb, long pyr_bs, long nn, int bands, void *acc, int precision, int accum,
-                       cudaStream_t s)
+                       bool first, bool beside, cudaStream_t s)
 {
     long g = (bands * nn / 4 + 255) / 256;
-    if (g > 152L * 16) g = 152L * 16;
+    const long gmax = 152L * (beside ? 3 : 16);
+    if (g > gmax) g = gmax;
     double *s1 = static_cast<double *>(acc), *s2 = s1 + (long)bands * nn;
+    const int wide = (reinterpret_cast<uintptr_t>(acc) & 15) == 0;
     if (accum == 1)
         FM_LAUNCH(FM_K_NOISE_ACCUM, k_noise_accum_kahan, (unsigned)g, 256, 0, s, (const float *)pyr, nb, pyr_bs, nn,
-                  bands, static_cast<float *>(acc));
+                  bands, static_cast<float *>(acc), (int)first);
     else if (precision == FM_F64)
         FM_LAUNCH(FM_K_NOISE_ACCUM, (k_noise_accum<double, double2>), (unsigned)g, 256, 0, s, (const double *)pyr,
-                  nb, pyr_bs, nn, bands, s1, s2);
+                  nb, pyr_bs, nn, bands, s1, s2, (int)first, wide);
     else
         FM_LAUNCH(FM_K_NOISE_ACCUM, (k_noise_accum<float, float4>), (unsigned)g, 256, 0, s, (const float *)pyr, nb,
-                  pyr_bs, nn, bands, s1, s2);
+                  pyr_bs, nn, bands, s1, s2, (int)first, wide);
     return FM_OK;
 }
 

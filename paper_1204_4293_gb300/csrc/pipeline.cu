@@ -319,11 +319,11 @@ NoiseLayout noise_layout(int n, int J, int R, const fm_config &cfg, bool multi_s
     return L;
 }
 
-// The bands of one fm_map_noise call: zero the FP64 sums; every batch of
-// rotated realisations through KS + starlet, chunk by chunk (over the
-// internal streams when `ds` is given, else on `s`), then S1 += w, S2 += w^2
-// over the batch's pyramids on `s`; with_data: the unrotated pass for S/N into
-// the first pyramid.  With internal streams and more than one batch, two
+// The bands of one fm_map_noise call: every batch of rotated realisations
+// through KS + starlet, chunk by chunk (over the internal streams when `ds` is
+// given, else on `s`), then S1 += w, S2 += w^2 over the batch's pyramids on
+// `s` (the first batch writes them); with_data: the unrotated pass for S/N
+// (noise_data_off).  With internal streams and more than one batch, two
 // pyramid buffers alternate so that the chunk streams run on into the next
 // batch while `s` accumulates (R = 1000 at 1024^2: 32.2 -> 31.6 ms; the
 // accumulation's pyramid loads are streaming, evict-first: 31.5 ms).
@@ -336,7 +336,6 @@ int noise_submit(const void *g1, const void *g2, bool with_data, int n, int J, i
 {
     const size_t es = cfg.precision == FM_F64 ? 8 : 4;
     const long nn = (long)n * n;
-    const long nb = (long)(J - 1) * nn;
     void *acc = ext_sums ? static_cast<void *>(ext_sums) : static_cast<void *>(scr);  // FP64 S1, S2 or the fp32
                                                                                        // Kahan pairs: 16 B / band px
     char *pyr = scr + L.acc_b, *slots = pyr + (size_t)L.pyr_bufs * L.pyr_b;
@@ -345,13 +344,12 @@ int noise_submit(const void *g1, const void *g2, bool with_data, int n, int J, i
     const uint64_t *seed = reinterpret_cast<const uint64_t *>(scr + L.seed_off());
     const char *c1 = static_cast<const char *>(g1), *c2 = static_cast<const char *>(g2);
     int r;
-    if (!ext_sums) FM_CUDA_TRY(cudaMemsetAsync(acc, 0, (size_t)2 * nb * sizeof(double), s));
     for (int r0 = 0, ib = 0; r0 < R; r0 += L.batch, ++ib) {
         const int b = R - r0 < L.batch ? R - r0 : L.batch;
         const int buf = ib % L.pyr_bufs;
         char *pb = pyr + (size_t)buf * L.pyr_b;
         if (multi && (L.pyr_bufs == 1 || ib == 0)) {
-            // start after `s` (the zeroed sums; with one buffer, the last accumulation)
+            // start after `s` (with one buffer, after the last accumulation)
             FM_CUDA_TRY(cudaEventRecord(ds->fork, s));
             for (int k = 0; k < L.slots; ++k) FM_CUDA_TRY(cudaStreamWaitEvent(ds->s[k], ds->fork, 0));
         } else if (multi && ib >= L.pyr_bufs) {
@@ -366,25 +364,43 @@ int noise_submit(const void *g1, const void *g2, bool with_data, int n, int J, i
                                multi ? ds->s[k] : s, true, seed, rbase + r0 + c0)))
                 return r;
         }
+        const bool last = r0 + b >= R;
+        if (last && with_data && b < L.batch) {  // the S/N's bands (noise_data_off), beside the batch's last chunks
+            const int k = multi ? i % L.slots : 0;
+            if ((r = run_chunk(c1, c2, pb + (size_t)b * J * nn * es, n, J, 0, 1, cfg, p, slots + k * p.slot_b,
+                               multi ? ds->s[k] : s)))
+                return r;
+        }
         if (multi)
             for (int k = 0; k < L.slots; ++k) {
                 FM_CUDA_TRY(cudaEventRecord(ds->join[k], ds->s[k]));
                 FM_CUDA_TRY(cudaStreamWaitEvent(s, ds->join[k], 0));
             }
-        if ((r = launch_noise_accum(pb, b, (long)J * nn, nn, J - 1, acc, cfg.precision, cfg.accum, s))) return r;
+        if ((r = launch_noise_accum(pb, b, (long)J * nn, nn, J - 1, acc, cfg.precision, cfg.accum, !ext_sums && ib == 0,
+                                    multi && L.pyr_bufs > 1 && R - r0 - b >= L.batch, s)))
+            return r;
         if (multi && L.pyr_bufs > 1) FM_CUDA_TRY(cudaEventRecord(ds->acc[buf], s));
     }
-    // S/N needs the unrotated bands; finalize reads them from the first pyramid
-    // (every chunk stream has joined `s` after the last batch)
-    if (with_data) return run_chunk(c1, c2, pyr, n, J, 0, 1, cfg, p, slots, s);
+    // S/N needs the unrotated bands: where the last batch is full, on `s` (every
+    // chunk stream has joined it) into the first pyramid, which that batch has left
+    if (with_data && R % L.batch == 0) return run_chunk(c1, c2, pyr, n, J, 0, 1, cfg, p, slots, s);
     return FM_OK;
+}
+
+// Where the unrotated bands lie: behind the last batch's pyramids, or in the
+// first pyramid where that batch fills its buffer.
+size_t noise_data_off(const NoiseLayout &L, int n, int J, int R, const fm_config &cfg)
+{
+    const int b = R % L.batch, ib = R / L.batch;
+    const size_t pyramid = (size_t)J * n * n * (cfg.precision == FM_F64 ? 8 : 4);
+    return L.acc_b + (b ? (size_t)(ib % L.pyr_bufs) * L.pyr_b + b * pyramid : 0);
 }
 
 int noise_finish(const NoiseLayout &L, char *scr, double *var_out, void *snr_out, int n, int J, int R,
                  const fm_config &cfg, cudaStream_t s)
 {
-    return launch_noise_finalize(scr, snr_out ? scr + L.acc_b : nullptr, var_out, snr_out, (long)(J - 1) * n * n, R,
-                                 cfg.precision, cfg.accum, s);
+    const char *data = snr_out ? scr + noise_data_off(L, n, J, R, cfg) : nullptr;
+    return launch_noise_finalize(scr, data, var_out, snr_out, (long)(J - 1) * n * n, R, cfg.precision, cfg.accum, s);
 }
 
 // A recorded noise call: its graph reads the shear and the seed from the
