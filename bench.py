@@ -411,6 +411,8 @@ def side_legs(fm, torch, n, J, g1, g2, pyr):
         t_s98 = cuda_time(torch, lambda: fm.fm_map_direct(s1, s2, fm.FM_FILTER_S98, theta), reps)
         t_stq = cuda_time(torch, lambda: fm.fm_map_direct(s1, s2, fm.FM_FILTER_STARLET, theta), reps)
         # the direct sum is FP32-FMA bound: 4 flops per tap (A gamma1 + B gamma2)
+        # of the plain sum; the kernel adds rows y + dy and y - dy first, so one
+        # FMA serves two taps and the fraction of the peak may pass 1
         tf_s98 = 4.0 * disc_taps(theta) * n * n / (t_s98 * 1e-3) / 1e12
         tf_stq = 4.0 * disc_taps(2 * theta) * n * n / (t_stq * 1e-3) / 1e12
         # the Gaussian filter (JBJ04, b = 1/2) needs a cut well beyond theta

@@ -7,7 +7,7 @@
 // TV], q = 0 .. E - 1, before and X[j + q TV] after the transform, so a
 // forward transform's output is in the inverse's input order without a
 // further exchange.  The passes exchange through shared memory (one slot of
-// padding per 16 elements keeps the stride-E stores conflict free; padded
+// padding per E elements keeps the stride-E stores conflict free; padded
 // addresses are one base a thread plus compile-time offsets).  Small DFTs run
 // in registers with constant twiddles; inter-pass twiddles come from
 // FP64-computed tables laid out in the order in which a warp reads them

@@ -13,6 +13,10 @@
 //             writes w_1..w_F and c_F.
 //   st_tile32 / st_tile : the same scales with a row-filtered shared buffer
 //             (fp32 alternative behind a tuning knob / fp64 and generic).
+//   st_scale : (fp32, n a multiple of 4, spacing 4..128 px) one large scale in
+//             one pass, its window rows staged by bulk copies or 16-byte loads.
+//   st_scale64 : (fp64, n a multiple of 2) one scale in one pass.
+//   st_colrow : columns of scale j and rows of scale j + 1 in one kernel.
 //   st_row  : r = rows-filtered c_{j-1} for one (large) scale.
 //   st_col  : c_j = columns-filtered r, w_j = c_{j-1} - c_j; c_j may overwrite
 //             c_{j-1} in place (each thread reads and writes only its own
