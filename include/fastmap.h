@@ -389,7 +389,9 @@ int fm_tune(int knob, int64_t value);
  * over: fused depth 1..4 (fp64 1..3, at most J - 1), large-scale path 1 or 3,
  * fp32 tile kernel form (1 = register window, 0 = shared buffer) and chunk
  * budget 40 / 60 / 80 / 120 MiB; a candidate replaces the best so far only
- * when 1 % faster.  The winner goes into a process-wide table keyed by
+ * when 1 % faster.  A batch that runs in one kernel (few fp32 maps of 64^2,
+ * 128^2 or 256^2) has no candidates beside the built-in plan and keeps that
+ * form whatever the table says.  The winner goes into a process-wide table keyed by
  * (n, J, precision), which the automatic fields (fuse_depth = 0,
  * large_path = 0) and the default tile form and chunk budget then follow
  * (knobs set by fm_tune keep precedence).  fm_autotune allocates its own

@@ -246,8 +246,9 @@ static bool cluster16_ok()
 // Whether a call takes the one-kernel form: fp32 maps of 64^2, 128^2 or 256^2
 // in batches up to where the separate kernels, which spread a batch over the
 // GPU with no barriers, catch up; with nothing asked for that names another
-// form (depth, large path, tuned plan, knobs, per-kernel timing).  J = 0:
-// Kaiser-Squires alone.  Measured, one kernel / separate kernels (us a call,
+// form (depth, large path, knobs, per-kernel timing).  An autotuned plan names
+// none: it describes the separate kernels, and so governs the batches above
+// these limits.  J = 0: Kaiser-Squires alone.  Measured, one kernel / separate kernels (us a call,
 // host included): KS + starlet 64^2 J = 5 x 256 27 / 41, x 512 51 / 58; 128^2 J
 // = 6 x 48 26 / 33, x 64 41 / 36; 256^2 J = 6 x 6 23 / 33, x 8 33 / 32; KS alone
 // 64^2 x 512 24 / 25, 128^2 x 96 18 / 23, x 128 25 / 23, 256^2 x 16 18 / 23, x 24
@@ -257,12 +258,10 @@ bool small_map_ok(int n, int J, int batch, const fm_config &cfg, bool aligned)
     if (cfg.precision != FM_F32 || !aligned || cfg.fuse_depth != 0 || cfg.large_path != 0) return false;
     const int most = J == 0 ? (n == 64 ? 512 : n == 128 ? 96 : n == 256 ? 16 : 0)
                             : (n == 64 ? 256 : n == 128 ? 48 : n == 256 ? 6 : 0);
-    TunedPlan tp;
     return batch <= most && g_prof_kid.load(std::memory_order_relaxed) == 0 &&
            g_ks_real.load(std::memory_order_relaxed) != 1 && g_tile_variant.load(std::memory_order_relaxed) < 0 &&
            g_wait_test.load(std::memory_order_relaxed) == 0 &&
-           g_use_tma.load(std::memory_order_relaxed) == kDefaultTma && !tune_lookup(n, J, FM_F32, &tp) &&
-           (n < 256 || cluster16_ok());
+           g_use_tma.load(std::memory_order_relaxed) == kDefaultTma && (n < 256 || cluster16_ok());
 }
 
 int launch_small_map(const float *g1, const float *g2, float *pyr, int n, int J, int batch, int boundary,

@@ -200,7 +200,9 @@ int fm_autotune(int n, int J, int batch, const fm_config *cfgp, fm_plan *best)
     double cur_ms = base_ms;
     const int fmax = std::min(cfg.precision == FM_F64 ? 3 : 4, J - 1);
     const int chunks[] = {24, 36, 48, 64, 96};
-    for (int sweep = 0; sweep < 2; ++sweep) {
+    // a batch that runs in one kernel leaves nothing to choose: no plan reaches it
+    const int sweeps = small_map_ok(n, J, batch, cfg, true) ? 0 : 2;
+    for (int sweep = 0; sweep < sweeps; ++sweep) {
         for (int dim = 0; dim < 4; ++dim) {
             std::vector<TunedPlan> cand;
             if (dim == 0)
