@@ -94,7 +94,7 @@ typedef struct {
                        memory (fp32, n a multiple of 4, scales with spacing
                        4..128 px; the form 1 for the others); in fp64,
                        automatic or 4: one pass for every scale that an
-                       explicit fuse_depth leaves (n even) */
+                       explicit or tuned depth leaves (n even) */
 } fm_config;
 
 /* ---- Kaiser-Squires (Sec. 4.5) ---------------------------------------------
@@ -119,8 +119,11 @@ int fm_starlet_forward(const void *kappa, void *pyramid, int n, int J, int batch
 
 /* Number of scales the fused tile kernel computes for fm_starlet_forward /
  * fm_map_starlet with these n, J and cfg (0 = none); the remaining
- * J - 1 - depth scales take one row and one column pass each.  Host only;
- * FM_EINVAL on a bad n, J or cfg. */
+ * J - 1 - depth scales take the large-scale path.  It is the depth of the tile
+ * form: two automatic calls take another one and launch no tile, few fp32 maps
+ * of 64^2, 128^2 or 256^2 (one kernel a call) and fp64 maps of an even side
+ * without a tuned plan of another depth or path (one pass a scale from the
+ * first on).  Host only; FM_EINVAL on a bad n, J or cfg. */
 int fm_starlet_fuse_depth(int n, int J, const fm_config *cfg);
 
 /* KS inversion then the starlet of kappa_E: the aperture-mass maps of every
@@ -394,7 +397,9 @@ int fm_tune(int knob, int64_t value);
  * form whatever the table says.  The winner goes into a process-wide table keyed by
  * (n, J, precision), which the automatic fields (fuse_depth = 0,
  * large_path = 0) and the default tile form and chunk budget then follow
- * (knobs set by fm_tune keep precedence).  fm_autotune allocates its own
+ * (knobs set by fm_tune keep precedence).  In fp64 an entry of the built-in
+ * depth and path (which fm_autotune times as its baseline) stands for the
+ * built-in form, one pass a scale and no tile; any other is run as it is named.  fm_autotune allocates its own
  * buffers, synchronises with the device and drops the cached graphs; do not
  * run it concurrently with other calls.  `best` (may be NULL) receives the
  * plan, its time and the built-in plan's time.

@@ -250,6 +250,8 @@ struct TunedPlan {
     double ms = 0, default_ms = 0;
 };
 bool tune_lookup(int n, int J, int precision, TunedPlan *out);  // false if no entry
+// whether a plan names the built-in depth and path (an entry like that stands for the built-in form)
+bool tune_is_builtin(int n, int J, const TunedPlan &p, const fm_config &cfg);
 int starlet_builtin_fuse(int n, int J, const fm_config &cfg);  // automatic depth without a table entry
 int starlet_builtin_large_path(int n, int J, int fuse);
 int64_t chunk_budget_default();

@@ -1417,14 +1417,15 @@ static int starlet_impl(const T *kappa, T *pyr, long pyr_bs, int n, int J, int b
     T *last = pyr + (long)(J - 1) * nn;  // slot of the smooth array
     const bool vec_ok = n % VW == 0 && aligned16(kappa) && aligned16(pyr) && (!scratch || aligned16(scratch));
     // fp64: one pass a scale (k_st_scale64) for all scales, or for those after
-    // an explicit depth, unless another large path or the plain form
-    // (fuse_depth -1) is asked for
+    // the depth that the call or a tuned plan names, unless another large path
+    // or the plain form (fuse_depth -1) is asked for.  The built-in depth and
+    // path in the table stand for the built-in form: no tile.
     TunedPlan plan64;
-    const bool one_pass64 =
-        sizeof(T) == 8 && vec_ok && Bb && batch <= 65535 &&
-        (cfg.large_path == 4 || (cfg.large_path == 0 && cfg.fuse_depth >= 0 &&
-                                 (!tune_lookup(n, J, cfg.precision, &plan64) || plan64.large_path == 4)));
-    if (one_pass64 && cfg.fuse_depth == 0) f = 0;
+    const bool tuned64 = sizeof(T) == 8 && tune_lookup(n, J, cfg.precision, &plan64) && !tune_is_builtin(n, J, plan64, cfg);
+    const bool one_pass64 = sizeof(T) == 8 && vec_ok && Bb && batch <= 65535 &&
+                            (cfg.large_path == 4 || (cfg.large_path == 0 && cfg.fuse_depth >= 0 &&
+                                                     (!tuned64 || plan64.large_path == 4)));
+    if (one_pass64 && cfg.fuse_depth == 0 && !tuned64) f = 0;
     if (f >= 1) {
         T *c_out = f == J - 1 ? (bands_only ? nullptr : last) : A;
         const long c_bs = f == J - 1 ? pyr_bs : nn;

@@ -108,6 +108,12 @@ bool tune_lookup(int n, int J, int precision, TunedPlan *out)
     return true;
 }
 
+bool tune_is_builtin(int n, int J, const TunedPlan &p, const fm_config &cfg)
+{
+    const TunedPlan b = builtin_plan(n, J, cfg);
+    return p.fuse == b.fuse && p.large_path == b.large_path;
+}
+
 }  // namespace fm
 
 using namespace fm;
