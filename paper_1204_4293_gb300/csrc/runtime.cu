@@ -125,15 +125,14 @@ static const void *twiddles_one(int n, int precision, cudaStream_t s, int *statu
         if (n >= 32)
             fft32_fill_table(n, t);
         else
-            for (int i = 0; i < n; ++i)
-                t[i] = make_float2((float)cos(-2.0 * M_PI * i / n), (float)sin(-2.0 * M_PI * i / n));
+            for (int i = 0; i < n; ++i) t[i] = unit_root<float2>(i, n);
     } else {
         host.resize((size_t)(n >= 32 ? fft_table_elems(n, kFft64LogE) : n) * sizeof(double2));
         double2 *t = reinterpret_cast<double2 *>(host.data());
         if (n >= 32)
             fft_fill_table(n, kFft64LogE, t);
         else
-            for (int i = 0; i < n; ++i) t[i] = make_double2(cos(-2.0 * M_PI * i / n), sin(-2.0 * M_PI * i / n));
+            for (int i = 0; i < n; ++i) t[i] = unit_root<double2>(i, n);
     }
     void *d = nullptr;
     e = dev_malloc(&d, host.size());
