@@ -660,7 +660,7 @@ static int ks32_real_impl(const float *in1, const float *in2, long in_bs, float 
               r0, m1, m2, tma_in);
     FM_LAUNCH(FM_K_FFT_COLS_KS, k_cols_ks32_e<LOGN>, col_grid, col_threads, col_smem, s, (const float2 *)work,
               reinterpret_cast<float2 *>(out1), tw, mc, mh, tma_col);
-    const float scale = out_scale / ((float)P::N * (float)P::N);
+    const float scale = out_scale * kFft32Gain / ((float)P::N * (float)P::N);
     FM_LAUNCH(FM_K_FFT_ROWS_INV, k_rows_inv32_c2r<LOGN>, row2_grid, RPC2 * P2::TV, row2_smem, s, out1, total_rows, tw,
               tw2, scale, mk, tma_out);
     return FM_OK;
@@ -741,7 +741,7 @@ static int ks32_impl(const float *in1, const float *in2, long in_bs, float *out1
               r0, m1, m2, tma_in);
     FM_LAUNCH(FM_K_FFT_COLS_KS, kcl, col_grid, col_threads, col_smem, s, work, tw, op, filt, mc, tma_col);
     if (op == FFT_OP_SPECTRUM) return FM_OK;
-    const float scale = out_scale / ((float)P::N * (float)P::N);
+    const float scale = out_scale * kFft32Gain / ((float)P::N * (float)P::N);
     FM_LAUNCH(FM_K_FFT_ROWS_INV, kri, row_grid, RPC * P::TV, row_smem, s, work, out1, out2, total_rows, tw, scale,
               scale * im_scale, mw, tma_out);
     return FM_OK;

@@ -190,7 +190,7 @@ static int small_launch_t(const float *in1, const float *in2, float *out1, float
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = g_pdl.load(std::memory_order_relaxed) ? 2 : 1;
-    const float scale = 1.f / ((float)M::N * (float)M::N);
+    const float scale = kFft32Gain / ((float)M::N * (float)M::N);
     cudaError_t e = cudaLaunchKernelEx(&cfg, k, in1, in2, out1, out2, tw, J, boundary, scale);
     g_launches.fetch_add(1, std::memory_order_relaxed);
     if (e != cudaSuccess) return cuda_fail(e, "k_small_map");
