@@ -5,54 +5,66 @@
 // Two passes over the pyramid: the first sums x per (map, array), the second
 // sums (x - mean)^2, ^3, ^4.  A strand is the run of at most 16 pixels S
 // apart (S = 256 ceil(nn / 4096)) whose sums are formed in fp32; strands are
-// added in pairs of floats (hi + lo by error-free two-sums) over a thread and
-// a block, and by one FP64 atomic per block and quantity; a last tiny kernel
-// forms the moments.
+// added in three floats (hi + mid + lo by error-free two-sums) over a thread
+// and a block, and by one FP64 atomic per block and quantity; a last tiny
+// kernel forms the moments.
 //
 // The work is two reads of the pyramid.  FP64 adds are the scarce resource
 // otherwise (one warp instruction in 16 to 32 cycles an SM on GB300): an FP64
 // shuffle tree over every thread's sums kept the second pass at 219 us for 8
-// pyramids of 7 x 1024^2 (235 MB, 35 us a read).  The float pairs carry 48
+// pyramids of 7 x 1024^2 (235 MB, 35 us a read).  The three floats carry 72
 // bits and leave FP64 a few instructions a block; 16-byte loads, eight in
-// flight a thread.  Those 8 pyramids: 293 -> 88 us for the whole call.
-// Running both passes over 20 .. 80 MB groups of arrays, so that the second
-// read comes from L2, was no faster (154 .. 90 us: shorter launches).
+// flight a thread.  Those 8 pyramids: 293 -> 84 us for the whole call; in fp64
+// 234 (two floats, 48 bits, instead of three 230).  Running both passes over 20
+// .. 80 MB groups of arrays, so that the second read comes from L2, was no
+// faster (154 .. 90 us against 90: shorter launches).
 #include <algorithm>
 
 #include "common.cuh"
 
 namespace fm {
 
-// hi + lo = the exact sum of the floats added so far, up to the rounding of
-// lo.  Sums of 2^100 and more (and infinities and NaN) move to FP64.
-struct FloatPair {  // (no initialisers: it is kept in shared memory too)
-    float hi, lo;
-    __device__ __forceinline__ void add(float p)
+// A sum of floats as hi + mid + lo: two chained two-sums (Knuth, TAOCP 4.2.2)
+// carry every rounding error down, so the sum holds up to 72 bits, more than
+// an FP64 sum's 53.
+struct FloatSum {  // (no initialisers: it is kept in shared memory too)
+    float hi, mid, lo;
+    // a += b, returning the rounding error
+    __device__ __forceinline__ static float two_sum(float &a, float b)
     {
-        const float s = __fadd_rn(hi, p), b = __fsub_rn(s, hi);
-        lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, b)), __fsub_rn(p, b)));
-        hi = s;
+        const float s = __fadd_rn(a, b), t = __fsub_rn(s, a);
+        const float e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, t)), __fsub_rn(b, t));
+        a = s;
+        return e;
     }
-    __device__ __forceinline__ double value() const { return isfinite(hi) ? (double)hi + (double)lo : (double)hi; }
-    __device__ __forceinline__ bool large() const { return !(fabsf(hi) < 1.2676506e30f); }  // 2^100
+    __device__ __forceinline__ void add(float p) { lo = __fadd_rn(lo, two_sum(mid, two_sum(hi, p))); }
+    __device__ __forceinline__ void add(const FloatSum &v)
+    {
+        add(v.hi);
+        lo = __fadd_rn(lo, __fadd_rn(two_sum(mid, v.mid), v.lo));
+    }
+    __device__ __forceinline__ double value() const { return (double)hi + ((double)mid + (double)lo); }
 };
+// Strands of 2^100 and more (and infinities and NaN) go to the FP64 sums
+// directly: a block's sums of the others stay finite (2^100 x 256 threads x
+// their strands, 2^14 at 8192^2).
+constexpr float kStrandMax = 1.2676506e30f;
 
-// the sum over the first N lanes' pairs, in lane 0
-template <int N> __device__ __forceinline__ FloatPair lane_sum(FloatPair v)
+// the sum over the first N lanes, in lane 0
+template <int N> __device__ __forceinline__ FloatSum lane_sum(FloatSum v)
 {
 #pragma unroll
-    for (int o = N / 2; o > 0; o >>= 1) {
-        const float h = __shfl_down_sync(0xffffffffu, v.hi, o), l = __shfl_down_sync(0xffffffffu, v.lo, o);
-        v.add(h);
-        v.lo = __fadd_rn(v.lo, l);
-    }
+    for (int o = N / 2; o > 0; o >>= 1)
+        v.add(FloatSum{__shfl_down_sync(0xffffffffu, v.hi, o), __shfl_down_sync(0xffffffffu, v.mid, o),
+                       __shfl_down_sync(0xffffffffu, v.lo, o)});
     return v;
 }
 
 // grid = (blocks per array, J, batch); sums[(b * J + j) * 4 + q].  A thread takes VW neighbouring
-// strands at a time (VW > 1: nn a multiple of VW and 16-byte aligned arrays).
+// strands at a time (VW > 1: nn a multiple of VW and 16-byte aligned arrays).  The bound of one block an SM
+// lets the compiler keep all eight loads in flight (8 x 7 x 1024^2 89 -> 84 us, 1023^2 150 -> 111).
 template <typename T, int PASS, int VW>
-__global__ void __launch_bounds__(256) k_moments(const T *__restrict__ pyr, long nn, long S, double inv_nn,
+__global__ void __launch_bounds__(256, 1) k_moments(const T *__restrict__ pyr, long nn, long S, double inv_nn,
                                                  double *__restrict__ sums)
 {
     pdl_entry();
@@ -64,16 +76,16 @@ __global__ void __launch_bounds__(256) k_moments(const T *__restrict__ pyr, long
     const T *x = pyr + array * nn;
     double *acc = sums + array * 4;
     __shared__ float s_mean;
-    __shared__ FloatPair red[NQ][8];
+    __shared__ FloatSum red[NQ][8];
     float mean = 0.f;
     if constexpr (PASS == 1) {
         if (threadIdx.x == 0) s_mean = (float)(acc[0] * inv_nn);
         __syncthreads();
         mean = s_mean;
     }
-    FloatPair tot[NQ];
+    FloatSum tot[NQ];
 #pragma unroll
-    for (int q = 0; q < NQ; ++q) tot[q] = FloatPair{0.f, 0.f};
+    for (int q = 0; q < NQ; ++q) tot[q] = FloatSum{0.f, 0.f, 0.f};
     for (long v0 = ((long)blockIdx.x * 256 + threadIdx.x) * VW; v0 < S; v0 += (long)gridDim.x * 256 * VW) {
         float s[VW][NQ] = {};
         auto add = [&](const Vec &v) {
@@ -98,27 +110,33 @@ __global__ void __launch_bounds__(256) k_moments(const T *__restrict__ pyr, long
             for (int k = 0; k < 8; ++k) add(v[k]);
         }
         for (; i < nn; i += S) add(*reinterpret_cast<const Vec *>(x + i));
+        float big = 0.f;
 #pragma unroll
-        for (int q = 0; q < NQ; ++q) {
+        for (int u = 0; u < VW; ++u)
 #pragma unroll
-            for (int u = 0; u < VW; ++u) {
-                tot[q].add(s[u][q]);
-                if (tot[q].large()) {
-                    atomicAdd(acc + PASS + q, tot[q].value());
-                    tot[q] = FloatPair{0.f, 0.f};
-                }
-            }
+            for (int q = 0; q < NQ; ++q) big += fabsf(s[u][q]);
+        // one test for all, so that the quantities' chains of adds run beside each other
+        if (big < kStrandMax) {
+#pragma unroll
+            for (int u = 0; u < VW; ++u)
+#pragma unroll
+                for (int q = 0; q < NQ; ++q) tot[q].add(s[u][q]);
+        } else {
+#pragma unroll
+            for (int u = 0; u < VW; ++u)
+#pragma unroll
+                for (int q = 0; q < NQ; ++q) atomicAdd(acc + PASS + q, (double)s[u][q]);
         }
     }
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
     for (int q = 0; q < NQ; ++q) {
-        const FloatPair r = lane_sum<32>(tot[q]);
+        const FloatSum r = lane_sum<32>(tot[q]);
         if (lane == 0) red[q][warp] = r;
     }
     __syncthreads();
     if (warp < NQ) {  // one quantity a warp
-        const FloatPair r = lane_sum<8>(lane < 8 ? red[warp][lane] : FloatPair{0.f, 0.f});
+        const FloatSum r = lane_sum<8>(lane < 8 ? red[warp][lane] : FloatSum{0.f, 0.f, 0.f});
         if (lane == 0) atomicAdd(acc + PASS + warp, r.value());
     }
 }
