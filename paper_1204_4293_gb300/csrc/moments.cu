@@ -47,7 +47,7 @@ struct FloatSum {  // (no initialisers: it is kept in shared memory too)
 };
 // Strands of 2^100 and more (and infinities and NaN) go to the FP64 sums
 // directly: a block's sums of the others stay finite (2^100 x 256 threads x
-// their strands, 2^14 at 8192^2).
+// their strands, 2^14 at 8192^2 and with eight blocks an SM at 65536^2).
 constexpr float kStrandMax = 1.2676506e30f;
 
 // the sum over the first N lanes, in lane 0
@@ -159,9 +159,7 @@ __global__ void k_moments_final(const double *__restrict__ sums, double *__restr
 template <typename T, int VW>
 static int moments_impl(const T *pyr, double *sums, int J, int batch, long nn, cudaStream_t s)
 {
-    long per = (nn + 256 * 16 - 1) / (256 * 16);  // strands of ~16 pixels (fp32 partial sums)
-    if (per > 4096) per = 4096;
-    const long S = per * 256;
+    const long S = (nn + 256 * 16 - 1) / (256 * 16) * 256;  // strands of at most 16 pixels (fp32 partial sums)
     // about eight blocks an SM over all arrays (4 / 8: 93 / 88 us for 8
     // pyramids of 7 x 1024^2), at least one an array
     const long count = (long)J * batch;

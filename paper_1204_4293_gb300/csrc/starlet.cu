@@ -31,6 +31,10 @@
 
 namespace fm {
 
+// Scaled taps: finite wherever the map stays below half the type's largest
+// value.  The unscaled taps (tap5, one exact scaling at the end) round the same
+// way but overflow from 1/256 of it on; they are kept to the fp32 tile, the
+// fp32 passes that follow one, and k_st_scale64, which falls back to these.
 template <typename T> struct B3 {
     // h = [1, 4, 6, 4, 1] / 16
     static constexpr T h0 = (T)0.0625, h1 = (T)0.25, h2 = (T)0.375;
@@ -39,13 +43,6 @@ template <typename T> struct B3 {
         return h0 * (m2 + p2) + h1 * (m1 + p1) + h2 * c;
     }
 };
-
-// fp32: integer taps and one exact scaling, the rounding of the packed filters
-// (tap5) below whatever the kernel
-template <> __device__ __forceinline__ float B3<float>::apply(float m2, float m1, float c, float p1, float p2)
-{
-    return fmaf(6.f, c, fmaf(4.f, m1 + p1, m2 + p2)) * 0.0625f;
-}
 
 // 16-byte vectors: 4 floats or 2 doubles
 template <typename T> struct Vec16;
@@ -890,6 +887,20 @@ __device__ __forceinline__ double over256(double v)
     if (ex >= 0x00900000 && ex != 0x7ff00000) return __hiloint2double(hi - 0x00800000, __double2loint(v));
     return v * (1.0 / 256.0);
 }
+// c_j of one pixel by the scaled taps
+__device__ __noinline__ double filter25(const double *cb, int n, int x, int y, int s, int boundary)
+{
+    int xf[5];
+    double r[5];
+#pragma unroll
+    for (int i = 0; i < 5; ++i) xf[i] = fold_index(x + (i - 2) * s, n, boundary);
+#pragma unroll
+    for (int i = 0; i < 5; ++i) {
+        const double *p = cb + (long)fold_index(y + (i - 2) * s, n, boundary) * n;
+        r[i] = B3<double>::apply(p[xf[0]], p[xf[1]], p[xf[2]], p[xf[3]], p[xf[4]]);
+    }
+    return B3<double>::apply(r[0], r[1], r[2], r[3], r[4]);
+}
 template <int KR, int SMALL>  // SMALL: spacing 1 (taps within three vectors), else any even spacing
 __global__ void __launch_bounds__(32) k_st_scale64(const double *__restrict__ c_prev, long prev_bs,
                                                    double *__restrict__ c_next, long next_bs,
@@ -918,6 +929,7 @@ __global__ void __launch_bounds__(32) k_st_scale64(const double *__restrict__ c_
     const long step = (long)s * n;
     auto v2 = [](const double *p) { return __ldg(reinterpret_cast<const double2 *>(p)); };
     double win[5][2], ctr[3][2];
+    bool bad = false;  // an output outside the finite range
 #pragma unroll
     for (int t = 0; t < KR + 4; ++t) {
         if (t - 4 >= rows) break;  // the last row's window is complete
@@ -954,12 +966,29 @@ __global__ void __launch_bounds__(32) k_st_scale64(const double *__restrict__ c_
             for (int u = 0; u < 2; ++u) {
                 cj[u] = over256(tap5(win[k % 5][u], win[(k + 1) % 5][u], win[(k + 2) % 5][u], win[(k + 3) % 5][u],
                                      win[(k + 4) % 5][u]));
+                bad |= (__double2hiint(cj[u]) & 0x7ff00000) == 0x7ff00000;
                 w[u] = ctr[(k + 2) % 3][u] - cj[u];
             }
             __stcs(reinterpret_cast<double2 *>(wp), make_double2(w[0], w[1]));
             if (cp) *reinterpret_cast<double2 *>(cp) = make_double2(cj[0], cj[1]);
             wp += step;
             if (cp) cp += step;
+        }
+    }
+    if (bad) {
+        // the unscaled sums left the range (values from 1/256 of the largest one
+        // on, infinities, NaN): the thread's outputs once more, scaled
+        const int last = rows < KR ? rows : KR;
+#pragma unroll 1
+        for (int k = 0; k < last; ++k) {
+            const int y = r0 + s * (mb + k);
+#pragma unroll 1
+            for (int u = 0; u < 2; ++u) {
+                const long px = (long)y * n + x + u;
+                const double v = filter25(cb, n, x + u, y, s, boundary);
+                w_out[b * w_bs + px] = cb[px] - v;
+                if (c_next) c_next[b * next_bs + px] = v;
+            }
         }
     }
 }
