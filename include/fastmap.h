@@ -190,7 +190,8 @@ int fm_map_direct_masked(const void *g1, const void *g2, const void *weight, lon
  * CUDA graph (keyed by sizes, R, config and chunk plan; it reads copies of
  * the shear and the seed, so it serves every buffer and seed of a shape) and
  * replayed as one launch; calls of one shape on several streams follow each
- * other.  Scratch: 16 (J-1) bytes per pixel of sums, the shear's copies, the
+ * other, but maps up to 256^2 that keep overlapping on two streams get a graph
+ * and scratch each.  Scratch: 16 (J-1) bytes per pixel of sums, the shear's copies, the
  * batches' pyramids and the chunks' intermediates, kept with the graph until
  * fm_trim or eviction. */
 int fm_map_noise(const void *g1, const void *g2, double *var_out, void *snr_out, int n, int J, int R, uint64_t seed,

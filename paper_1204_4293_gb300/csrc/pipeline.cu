@@ -426,11 +426,31 @@ struct NoiseGraph {
     cudaGraphExec_t exec = nullptr;
     void *scratch = nullptr;
     cudaEvent_t done = nullptr;
+    cudaStream_t stream = nullptr;  // of its last call: a preference only, `done` orders whatever the stream
+    int waits = 0;                  // calls that found it busy on another stream
     uint64_t used = 0;
     int64_t kernels = 0;
 };
 std::vector<NoiseGraph> g_noise_graphs;  // guarded by g_ds_mu
 constexpr size_t kMaxNoiseGraphs = 2;
+// Calls of one shape on two streams run beside each other on a graph and scratch
+// each where a map leaves much of the GPU idle, up to 256^2: two calls, R = 100,
+// one after the other / beside each other, 64^2 243 / 136 us, 128^2 298 / 175,
+// 256^2 523 / 353; from 512^2 on they only get in each other's way (recorded per
+// buffer, with slower kernels, 512^2 1558 / 1604, 1024^2 5738 / 6320).
+constexpr int kNoiseTwinMaxN = 256;
+
+// whether the graph's last call has finished (asked in relaxed capture mode: a
+// capture on another thread stays valid)
+bool noise_idle(const NoiseGraph &e)
+{
+    cudaStreamCaptureMode m = cudaStreamCaptureModeRelaxed;
+    if (cudaThreadExchangeStreamCaptureMode(&m) != cudaSuccess) return false;
+    const cudaError_t q = cudaEventQuery(e.done);
+    if (q == cudaErrorNotReady) cudaGetLastError();
+    cudaThreadExchangeStreamCaptureMode(&m);
+    return q == cudaSuccess;
+}
 
 void drop_noise_graph(NoiseGraph &e)
 {
@@ -443,10 +463,50 @@ void drop_noise_graph(NoiseGraph &e)
     e.done = nullptr;
 }
 
+// Records the realisations of a shape into a graph with scratch of its own.
+int record_noise(const NoiseKey &key, const NoiseLayout &L, size_t in_b, DevStreams *ds, NoiseGraph *out)
+{
+    NoiseGraph e;
+    e.key = key;
+    cudaError_t ce = dev_malloc(&e.scratch, L.total + 2 * in_b);
+    if (ce != cudaSuccess) return cuda_fail(ce, "cudaMalloc (noise graph scratch)");
+    cudaGraph_t graph = nullptr;
+    ce = cudaStreamBeginCapture(ds->cap, cudaStreamCaptureModeRelaxed);
+    if (ce != cudaSuccess) {
+        cudaFree(e.scratch);
+        return cuda_fail(ce, "cudaStreamBeginCapture");
+    }
+    const int64_t before = g_launches.load();
+    char *scr = (char *)e.scratch;
+    int st = noise_submit(scr + L.total, scr + L.total + in_b, key.with_data, key.n, key.J, key.R, key.cfg, L, scr,
+                          ds->cap, ds);
+    e.kernels = g_launches.load() - before;
+    g_launches.fetch_sub(e.kernels);
+    ce = cudaStreamEndCapture(ds->cap, &graph);
+    if (st == FM_OK && ce != cudaSuccess) st = cuda_fail(ce, "cudaStreamEndCapture");
+    if (st == FM_OK) {
+        ce = cudaGraphInstantiate(&e.exec, graph, 0);
+        if (ce != cudaSuccess) st = cuda_fail(ce, "cudaGraphInstantiate");
+    }
+    if (graph) cudaGraphDestroy(graph);
+    if (st == FM_OK) {
+        ce = cudaEventCreateWithFlags(&e.done, cudaEventDisableTiming);
+        if (ce != cudaSuccess) st = cuda_fail(ce, "cudaEventCreate (noise graph)");
+    }
+    if (st != FM_OK) {
+        if (e.exec) cudaGraphExecDestroy(e.exec);
+        cudaFree(e.scratch);
+        return st;
+    }
+    *out = e;
+    return FM_OK;
+}
+
 }  // namespace
 
 // allow_graph: record the realisations of a shape once into a CUDA graph
-// (kept with its scratch, LRU of two) and replay it; otherwise launch eagerly
+// (kept with its scratch, LRU of two; a small shape may have both) and replay
+// it; otherwise launch eagerly
 // with stream-ordered scratch (the serving path, which bounds its memory).
 int map_noise_run(const void *g1, const void *g2, double *var_out, void *snr_out, int n, int J, int R, uint64_t seed,
                   const fm_config &cfg, cudaStream_t s, bool allow_graph, bool multi_eager)
@@ -486,9 +546,25 @@ int map_noise_run(const void *g1, const void *g2, double *var_out, void *snr_out
     NoiseKey key{n, J, R, 0, snr_out != nullptr, cfg, L.p.C, L.slots,
                  g_pdl.load() | ((g_tile_variant.load() + 1) << 1) | (g_use_tma.load() << 3) | (g_wait_test.load() << 10) | ((g_ks_real.load() + 1) << 11)};
     FM_CUDA_TRY(cudaGetDevice(&key.dev));
-    NoiseGraph *hit = nullptr;
+    NoiseGraph *hit = nullptr, *busy = nullptr;
     for (auto &e : g_noise_graphs)
-        if (e.key == key) hit = &e;
+        if (e.key == key && e.stream == s) hit = &e;
+    for (auto &e : g_noise_graphs) {
+        if (hit || !(e.key == key)) continue;
+        if (noise_idle(e))
+            hit = &e;
+        else
+            busy = &e;
+    }
+    // a second stream that keeps finding it busy gets its own, if there is room
+    if (!hit && busy && n <= kNoiseTwinMaxN && ++busy->waits > 1 && g_noise_graphs.size() < kMaxNoiseGraphs) {
+        NoiseGraph e;
+        if (record_noise(key, L, in_b, ds, &e) == FM_OK) {
+            g_noise_graphs.push_back(e);
+            hit = &g_noise_graphs.back();
+        }
+    }
+    if (!hit) hit = busy;  // follows the call that uses it
     if (!hit) {
         if (g_noise_graphs.size() >= kMaxNoiseGraphs) {
             auto lru = std::min_element(g_noise_graphs.begin(), g_noise_graphs.end(),
@@ -497,49 +573,25 @@ int map_noise_run(const void *g1, const void *g2, double *var_out, void *snr_out
             g_noise_graphs.erase(lru);
         }
         NoiseGraph e;
-        e.key = key;
-        cudaError_t ce = dev_malloc(&e.scratch, L.total + 2 * in_b);
-        if (ce != cudaSuccess) return cuda_fail(ce, "cudaMalloc (noise graph scratch)");
-        cudaGraph_t graph = nullptr;
-        ce = cudaStreamBeginCapture(ds->cap, cudaStreamCaptureModeRelaxed);
-        if (ce != cudaSuccess) {
-            cudaFree(e.scratch);
-            return cuda_fail(ce, "cudaStreamBeginCapture");
-        }
-        const int64_t before = g_launches.load();
-        char *scr = (char *)e.scratch;
-        st = noise_submit(scr + L.total, scr + L.total + in_b, key.with_data, n, J, R, cfg, L, scr, ds->cap, ds);
-        e.kernels = g_launches.load() - before;
-        g_launches.fetch_sub(e.kernels);
-        ce = cudaStreamEndCapture(ds->cap, &graph);
-        if (st == FM_OK && ce != cudaSuccess) st = cuda_fail(ce, "cudaStreamEndCapture");
-        if (st == FM_OK) {
-            ce = cudaGraphInstantiate(&e.exec, graph, 0);
-            if (ce != cudaSuccess) st = cuda_fail(ce, "cudaGraphInstantiate");
-        }
-        if (graph) cudaGraphDestroy(graph);
-        if (st == FM_OK) {
-            ce = cudaEventCreateWithFlags(&e.done, cudaEventDisableTiming);
-            if (ce != cudaSuccess) st = cuda_fail(ce, "cudaEventCreate (noise graph)");
-        }
-        if (st != FM_OK) {
-            if (e.exec) cudaGraphExecDestroy(e.exec);
-            cudaFree(e.scratch);
-            return st;
-        }
+        if ((st = record_noise(key, L, in_b, ds, &e))) return st;
         g_noise_graphs.push_back(e);
         hit = &g_noise_graphs.back();
     }
     hit->used = ++g_graph_clock;
+    hit->stream = s;
     char *scr = (char *)hit->scratch;
     FM_CUDA_TRY(cudaStreamWaitEvent(s, hit->done, 0));  // the scratch's previous use, on any stream
-    if ((st = launch_noise_stage(g1, g2, scr + L.total, scr + L.total + in_b, (size_t)n * n * (cfg.precision == FM_F64 ? 8 : 4),
-                                 seed, (uint64_t *)(scr + L.seed_off()), s)))
-        return st;
-    FM_CUDA_TRY(cudaGraphLaunch(hit->exec, s));
-    g_launches.fetch_add(hit->kernels);
-    st = noise_finish(L, scr, var_out, snr_out, n, J, R, cfg, s);
-    FM_CUDA_TRY(cudaEventRecord(hit->done, s));
+    st = launch_noise_stage(g1, g2, scr + L.total, scr + L.total + in_b, (size_t)n * n * (cfg.precision == FM_F64 ? 8 : 4),
+                            seed, (uint64_t *)(scr + L.seed_off()), s);
+    if (st == FM_OK) {
+        const cudaError_t ce = cudaGraphLaunch(hit->exec, s);
+        if (ce != cudaSuccess)
+            st = cuda_fail(ce, "cudaGraphLaunch (noise)");
+        else
+            g_launches.fetch_add(hit->kernels);
+    }
+    if (st == FM_OK) st = noise_finish(L, scr, var_out, snr_out, n, J, R, cfg, s);
+    FM_CUDA_TRY(cudaEventRecord(hit->done, s));  // whatever of it was launched
     return st;
 }
 
