@@ -71,7 +71,11 @@ int fm_ks_invert(const void *g1, const void *g2, void *kappa_E, void *kappa_B, i
     if (batch < 1) return einval("batch must be >= 1");
     if (!g1 || !g2 || !kappa_E) return einval("null pointer");
     cudaStream_t s = (cudaStream_t)stream;
-    if (small_map_ok(n, 0, batch, cfg, true))
+    // kappa laid over the shear of other maps (not in place): the separate kernels read all of it first
+    const size_t map_b = (size_t)batch * n * n * esize(cfg);
+    auto apart = [&](const void *out, const void *in) { return out == in || !overlap(out, map_b, in, map_b); };
+    const bool one = batch == 1 || (apart(kappa_E, g1) && apart(kappa_E, g2) && apart(kappa_B, g1) && apart(kappa_B, g2));
+    if (one && small_map_ok(n, 0, batch, cfg, true))
         return launch_small_ks((const float *)g1, (const float *)g2, (float *)kappa_E, (float *)kappa_B, n, batch, s);
     Scratch work;
     const size_t bytes = (size_t)batch * n * n * 2 * esize(cfg);

@@ -235,7 +235,15 @@ int launch_fft64(const double *in1, const double *in2, long in_bs, double *out1,
 extern std::atomic<int> g_ks_real;
 bool ks_real_for(int n, bool batched);
 size_t starlet_scratch_elems(int n, int J, int batch, const fm_config &cfg);
-// small maps in one kernel (small.cu); J = 0 for Kaiser-Squires alone
+// whether two buffers share bytes
+inline bool overlap(const void *a, size_t an, const void *b, size_t bn)
+{
+    const uintptr_t x = reinterpret_cast<uintptr_t>(a), y = reinterpret_cast<uintptr_t>(b);
+    return a && b && x < y + bn && y < x + an;
+}
+// small maps in one kernel (small.cu); J = 0 for Kaiser-Squires alone.  A map's
+// outputs are written as soon as its own inputs are read: the caller makes
+// sure that no other map's inputs lie there
 bool small_map_ok(int n, int J, int batch, const fm_config &cfg, bool aligned);
 int launch_small_map(const float *g1, const float *g2, float *pyr, int n, int J, int batch, int boundary,
                      cudaStream_t s);

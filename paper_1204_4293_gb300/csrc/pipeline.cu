@@ -205,7 +205,10 @@ void drop_graph(GraphEntry &e)
 static int map_starlet_dev(const void *g1, const void *g2, void *pyramid, int n, int J, int batch,
                            const fm_config &cfg, cudaStream_t s, bool allow_graph = true)
 {
-    if (small_map_ok(n, J, batch, cfg, (reinterpret_cast<uintptr_t>(pyramid) & 15) == 0))
+    // a pyramid laid over several maps' shear: the separate kernels read all of it first
+    const size_t in_b = (size_t)batch * n * n * (cfg.precision == FM_F64 ? 8 : 4), out_b = in_b * J;
+    const bool apart = batch == 1 || !(overlap(pyramid, out_b, g1, in_b) || overlap(pyramid, out_b, g2, in_b));
+    if (apart && small_map_ok(n, J, batch, cfg, (reinterpret_cast<uintptr_t>(pyramid) & 15) == 0))
         return launch_small_map((const float *)g1, (const float *)g2, (float *)pyramid, n, J, batch, cfg.boundary, s);
     const ChunkPlan p = plan_chunks(n, J, batch, cfg);
     if (p.C >= batch) {  // one chunk: straight onto the caller's stream
