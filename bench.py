@@ -19,6 +19,7 @@ import argparse
 import hashlib
 import json
 import os
+import re
 import statistics
 import subprocess
 import sys
@@ -76,12 +77,30 @@ def load_peaks():
         return 6800.0, "fallback"
 
 
+def source_digest(path):
+    """Digest of a kernel source and of the project headers beside it that it
+    includes, theirs too, without comments and white space."""
+    seen, text = set(), []
+
+    def add(p):
+        if p in seen or not os.path.exists(p):
+            return
+        seen.add(p)
+        src = open(p, encoding="utf-8").read()
+        for name in re.findall(r'^\s*#include "([^"/]+)"', src, re.M):
+            add(os.path.join(os.path.dirname(p), name))
+        text.append(re.sub(r"\s+", "", re.sub(r"//[^\n]*|/\*.*?\*/", "", src, flags=re.S)))
+
+    add(path)
+    return hashlib.sha256("\n".join(text).encode()).hexdigest()[:16]
+
+
 def ncu_traffic(kernel, field="dram_bytes_per_px", shape=None):
     """Bytes per map pixel of one launch of `kernel` from the committed ncu
     summary (a warm capture on a small case): DRAM read + write
     (dram_bytes_per_px) or SM <-> L2 read + write (l2_bytes_per_px), valid
-    only while the kernel source is unchanged (sha at capture); None
-    otherwise."""
+    only while the kernel's source and headers are unchanged (their digest at
+    the capture); None otherwise."""
     path = os.path.join(ROOT, "profiles", "ncu_traffic.txt")
     if not os.path.exists(path):
         return None
@@ -98,8 +117,7 @@ def ncu_traffic(kernel, field="dram_bytes_per_px", shape=None):
     if shape is not None and (rec.get("n"), rec.get("J"), rec.get("fuse")) != tuple(str(v) for v in shape):
         return None  # captured on another workload
     src = os.path.join(ROOT, "paper_1204_4293_gb300", "csrc", rec["source"])
-    sha = hashlib.sha256(open(src, "rb").read()).hexdigest()[:16]
-    if sha != rec.get("sha"):
+    if source_digest(src) != rec.get("sha"):
         return None
     return float(rec[field])
 
