@@ -126,8 +126,6 @@ __global__ void __launch_bounds__(Plan32<LOGN>::ROW_T, Plan32<LOGN>::ROW_MINB)
                 if (in2) tma_load_3d(st2, &m2, 0, 0, z, &bar);
             }
             if (!tma_wait_all(&bar, 0)) return;  // the copies never completed (flagged)
-            const long b = row >> LOGN;
-            const int y = (int)(row & (P::N - 1));
 #pragma unroll
             for (int r = 0; r < P::E; ++r) {
                 const int x = j + r * P::TV;

@@ -47,7 +47,6 @@
 #include <math.h>
 
 #include <algorithm>
-#include <atomic>
 #include <type_traits>
 
 #include "common.cuh"
@@ -449,9 +448,6 @@ __global__ void __launch_bounds__(256) k_direct_sum(const T *__restrict__ parts,
         }
     }
 }
-
-// FM_TUNE_DIRECT: kept for its callers; every value runs the one kernel form
-std::atomic<int> g_direct_form{-1};
 
 // Parts of the dy: a function of n and the radius only, so that a map's
 // result does not depend on the maps beside it.  Eight full loads of the GPU
