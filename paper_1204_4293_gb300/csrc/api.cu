@@ -308,13 +308,18 @@ int fm_map_noise_expected(const void *g1, const void *g2, void *var_out, int n, 
     if ((st = launch_fft_op(p, nullptr, nn, nullptr, nullptr, spec, n, 1, prec, FFT_OP_SPECTRUM, nullptr, 1.0, 0, 0,
                             false, s)))
         return st;
+    // The responses are scaled for two transforms there and back, but a unit
+    // shear's transform there is exact: half of that gain is too much in K_j, the
+    // whole of it once in |K_j|^2 (bias of the bands' |K_j|^2, n = 32 .. 2048: as
+    // scaled 0.5 .. 1.8e-7, unscaled -0.5 .. -1.6e-7, so -0.7 .. 0.6e-7).
+    const double half = prec == FM_F32 && n >= 32 ? 0.5 / kFft32Gain : 0.5;
     char *var = static_cast<char *>(var_out), *q2 = q + (size_t)pairs * nn * es;
     if (h > 0 && (st = launch_fft_op(q, q2, nn, var, var + (size_t)pairs * nn * es, work, n, h, prec, FFT_OP_FILTER,
-                                     spec, 0.5, 0, 0, false, s, false, 1.0 / up4)))
+                                     spec, half, 0, 0, false, s, false, 1.0 / up4)))
         return st;
     if (h == pairs) return FM_OK;
     return launch_fft_op(q + (size_t)h * nn * es, nullptr, nn, var + (size_t)h * nn * es, nullptr, work, n, 1, prec,
-                         FFT_OP_FILTER, spec, 0.5, 0, 0, false, s);
+                         FFT_OP_FILTER, spec, half, 0, 0, false, s);
 }
 
 int fm_band_moments(const void *pyramid, double *moments, int n, int J, int batch, const fm_config *cfgp,

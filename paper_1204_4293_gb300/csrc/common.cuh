@@ -217,6 +217,18 @@ int launch_ks32(const float *in1, const float *in2, long in_bs, float *out1, flo
 //                   imaginary times out_scale * im_scale)
 //   FFT_OP_SPECTRUM stop after the columns FFT: `work` holds the spectrum
 enum { FFT_OP_KS_INV = 0, FFT_OP_KS_FWD = 1, FFT_OP_FILTER = 2, FFT_OP_SPECTRUM = 3 };
+// Gain of the two transforms there and back, taken up by the last scaling.  The
+// constants W_32^m rounded to fp32 have moduli a little below 1, and so do the
+// pass twiddles on average: over the four one-dimensional transforms the
+// amplitude comes out 0.8e-7 (n = 32, 64) to 1.7e-7 (8192) too small, the same
+// for every pixel.  That bias, and not the pixels' independent roundings, was
+// nearly all of the error of a noise variance (fp32, rms of the mean variance,
+// 64^2 / 256^2 / 512^2 / 1024^2 1.7 / 2.2 / 2.5 / 2.8e-7, now 1.3 / 1.0 / 1.1 /
+// 0.9e-7).  1 + 2^-23 leaves at most 5.3e-8 of the gain at any n.  It belongs to the
+// Kaiser-Squires transforms, whose inputs have no constant part: the constant
+// part of a field passes the transforms without a rounded constant, and a
+// filter's fields (the expected variance) are mostly that.
+constexpr float kFft32Gain = 1.00000012f;
 int launch_fft_op(const void *in1, const void *in2, long in_bstride, void *out1, void *out2, void *work, int n,
                   int batch, int precision, int op, const void *filt, double out_scale, const uint64_t *rot_seed, int rot_r0,
                   bool rotate, cudaStream_t s, bool real_ok = false, double im_scale = 1.0);

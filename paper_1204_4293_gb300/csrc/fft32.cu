@@ -739,7 +739,8 @@ static int ks32_impl(const float *in1, const float *in2, long in_bs, float *out1
               r0, m1, m2, tma_in);
     FM_LAUNCH(FM_K_FFT_COLS_KS, kcl, col_grid, col_threads, col_smem, s, work, tw, op, filt, mc, tma_col);
     if (op == FFT_OP_SPECTRUM) return FM_OK;
-    const float scale = out_scale * kFft32Gain / ((float)P::N * (float)P::N);
+    const float gain = op == FFT_OP_FILTER ? 1.f : kFft32Gain;
+    const float scale = out_scale * gain / ((float)P::N * (float)P::N);
     FM_LAUNCH(FM_K_FFT_ROWS_INV, kri, row_grid, RPC * P::TV, row_smem, s, work, out1, out2, total_rows, tw, scale,
               scale * im_scale, mw, tma_out);
     return FM_OK;

@@ -9,16 +9,6 @@
 
 namespace fm {
 
-// Gain of the two transforms there and back, taken up by the last scaling.  The
-// constants W_32^m rounded to fp32 have moduli a little below 1, and so do the
-// pass twiddles on average: over the four one-dimensional transforms the
-// amplitude comes out 0.8e-7 (n = 32, 64) to 1.7e-7 (8192) too small, the same
-// for every pixel.  That bias, and not the pixels' independent roundings, was
-// nearly all of the error of a noise variance (fp32, rms of the mean variance,
-// 64^2 / 256^2 / 512^2 / 1024^2 1.7 / 2.2 / 2.5 / 2.8e-7, now 1.3 / 1.0 / 1.1 /
-// 0.9e-7).  1 + 2^-23 leaves at most 5.3e-8 of the gain at any n.
-constexpr float kFft32Gain = 1.00000012f;
-
 // shared-memory slot of element a of a transform of length 2^LOGN: one slot of
 // padding per E, so that E-strided stores of W interleaved vectors hit every
 // bank (the stride E W + W is W modulo 16 eight-byte slots)
