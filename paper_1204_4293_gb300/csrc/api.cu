@@ -269,10 +269,13 @@ int fm_noise_finalize(const double *sums, const void *pyramid, double *var_out, 
 // time: the spectrum of |gamma|^2 once, then rows FFT of |K_j|^2 + i |K_j+h|^2
 // -> columns FFT -> times that spectrum -> inverse, whose real and imaginary
 // parts are the bands j and j + h (|gamma|^2 is real).  Band j + h enters
-// times 4^h, which brings it to band j's magnitude (a band's response power
-// falls by about 4 a scale), so that its rounding is relative to itself; both
-// powers of two are exact.  One spectrum and (J - 1) / 2 filter passes instead
-// of J - 1 of each: 1024^2, J = 7 214 -> 158 us, its error against FP64 unchanged.
+// times a power of two that brings it to band j's magnitude, so that its
+// rounding is relative to itself: 4^pairs, as a band's response power falls by
+// 4.0 to 5.5 a scale, and for band 0's partner, as band 0 has 20 times the power
+// of band 1, that times 8 (4 for one pair).  With 4^pairs alone the partner's
+// error was 2.5 times the other bands' (rms of its mean, 256^2 .. 2048^2 3.3 ..
+// 4.0e-7, now 1.3 .. 1.8e-7).  One spectrum and (J - 1) / 2 filter passes instead of J - 1
+// of each: 1024^2, J = 7 214 -> 158 us.
 int fm_map_noise_expected(const void *g1, const void *g2, void *var_out, int n, int J, const fm_config *cfgp,
                           void *stream)
 {
@@ -302,9 +305,9 @@ int fm_map_noise_expected(const void *g1, const void *g2, void *var_out, int n, 
     if ((st = launch_unit_shears(g1d, g2d, nn, prec, s))) return st;
     if ((st = map_starlet_run(g1d, g2d, pyr, n, J, 2, cfg, s))) return st;
     // |K_j|^2 = (Re K_j)^2 + (Im K_j)^2 from the two responses [2][J][n][n]
-    const double up4 = ldexp(1.0, 2 * pairs);  // 4^pairs
-    if ((st = launch_modulus2(pyr, nn, pyr + (size_t)J * nn * es, nn, q, nn, nb, pairs, up4, prec, s))) return st;
-    if ((st = launch_modulus2(g1, 0, g2, 0, p, nn, 1, 1, 1.0, prec, s))) return st;
+    const double up4 = ldexp(1.0, 2 * pairs), lead = up4 * (pairs > 1 ? 8 : 4);  // 4^pairs; band 0's partner
+    if ((st = launch_modulus2(pyr, nn, pyr + (size_t)J * nn * es, nn, q, nn, nb, pairs, lead, up4, prec, s))) return st;
+    if ((st = launch_modulus2(g1, 0, g2, 0, p, nn, 1, 1, 1.0, 1.0, prec, s))) return st;
     if ((st = launch_fft_op(p, nullptr, nn, nullptr, nullptr, spec, n, 1, prec, FFT_OP_SPECTRUM, nullptr, 1.0, 0, 0,
                             false, s)))
         return st;
@@ -315,7 +318,7 @@ int fm_map_noise_expected(const void *g1, const void *g2, void *var_out, int n, 
     const double half = prec == FM_F32 && n >= 32 ? 0.5 / kFft32Gain : 0.5;
     char *var = static_cast<char *>(var_out), *q2 = q + (size_t)pairs * nn * es;
     if (h > 0 && (st = launch_fft_op(q, q2, nn, var, var + (size_t)pairs * nn * es, work, n, h, prec, FFT_OP_FILTER,
-                                     spec, half, 0, 0, false, s, false, 1.0 / up4)))
+                                     spec, half, 0, 0, false, s, false, 1.0 / up4, 1.0 / lead)))
         return st;
     if (h == pairs) return FM_OK;
     return launch_fft_op(q + (size_t)h * nn * es, nullptr, nn, var + (size_t)h * nn * es, nullptr, work, n, 1, prec,

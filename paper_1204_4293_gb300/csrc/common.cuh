@@ -214,7 +214,7 @@ int launch_ks32(const float *in1, const float *in2, long in_bs, float *out1, flo
 //   FFT_OP_KS_FWD   multiply by D        (shear of a convergence map)
 //   FFT_OP_FILTER   multiply by the spectrum filt[ky][kx], one for the batch (a
 //                   periodic convolution; real output times out_scale,
-//                   imaginary times out_scale * im_scale)
+//                   imaginary times out_scale * im_scale, im_scale0 in map 0)
 //   FFT_OP_SPECTRUM stop after the columns FFT: `work` holds the spectrum
 enum { FFT_OP_KS_INV = 0, FFT_OP_KS_FWD = 1, FFT_OP_FILTER = 2, FFT_OP_SPECTRUM = 3 };
 // Gain of the two transforms there and back, taken up by the last scaling.  The
@@ -231,14 +231,14 @@ enum { FFT_OP_KS_INV = 0, FFT_OP_KS_FWD = 1, FFT_OP_FILTER = 2, FFT_OP_SPECTRUM 
 constexpr float kFft32Gain = 1.00000012f;
 int launch_fft_op(const void *in1, const void *in2, long in_bstride, void *out1, void *out2, void *work, int n,
                   int batch, int precision, int op, const void *filt, double out_scale, const uint64_t *rot_seed, int rot_r0,
-                  bool rotate, cudaStream_t s, bool real_ok = false, double im_scale = 1.0);
+                  bool rotate, cudaStream_t s, bool real_ok = false, double im_scale = 1.0, double im_scale0 = 1.0);
 int launch_fft32(const float *in1, const float *in2, long in_bs, float *out1, float *out2, float2 *work, int n,
                  int batch, int op, const float2 *filt, float out_scale, const uint64_t *seed, int r0, bool rotate,
-                 const float2 *tw, const float2 *tw2, cudaStream_t s, float im_scale = 1.f);
+                 const float2 *tw, const float2 *tw2, cudaStream_t s, float im_scale = 1.f, float im_scale0 = 1.f);
 // the fp64 form, n = 64 .. 2048 (fft64.cu)
 int launch_fft64(const double *in1, const double *in2, long in_bs, double *out1, double *out2, double2 *work, int n,
                  int batch, int op, const double2 *filt, double out_scale, const uint64_t *seed, int r0, bool rotate,
-                 const double2 *tw, const double2 *tw2, cudaStream_t s, double im_scale);
+                 const double2 *tw, const double2 *tw2, cudaStream_t s, double im_scale, double im_scale0);
 // inverse KS with a real output (kappa_E only) through the half spectrum
 // (FM_TUNE_KS_REAL): -1 = by size (default), 0 = never, 1 = whenever
 // possible (fp32, n >= 64)
@@ -299,9 +299,9 @@ int map_noise_run(const void *g1, const void *g2, double *var_out, void *snr_out
                   const fm_config &cfg, cudaStream_t s, bool allow_graph, bool multi_eager = false);
 int map_noise_accumulate_run(const void *g1, const void *g2, double *sums, int n, int J, int r0, int R, uint64_t seed,
                              const fm_config &cfg, cudaStream_t s);
-// out[c] = (a[c]^2 + b[c]^2) f0 4^c', c' = c - h for c >= h, else f0 = 1 alone (see noise.cu)
+// out[c] = (a[c]^2 + b[c]^2) times 1 for c < h, fh for c = h, f0 above (see noise.cu)
 int launch_modulus2(const void *a, long a_bs, const void *b, long b_bs, void *out, long nn, int count, int h,
-                    double f0, int precision, cudaStream_t s);
+                    double fh, double f0, int precision, cudaStream_t s);
 int launch_unit_shears(void *g1d, void *g2d, long nn, int precision, cudaStream_t s);
 int launch_band_moments(const void *pyr, double *moments, int n, int J, int batch, int precision, void *scratch,
                         cudaStream_t s);

@@ -205,7 +205,8 @@ __global__ void __launch_bounds__(1024) k_cols_ks(cplx_t<T> *__restrict__ work, 
 template <typename T, int E>
 __global__ void __launch_bounds__(1024) k_rows_inv(const cplx_t<T> *__restrict__ work, T *__restrict__ out1,
                                                    T *__restrict__ out2, int n, int logn, int lognvec,
-                                                   long total_rows, const cplx_t<T> *__restrict__ tw, T scale, T im_scale)
+                                                   long total_rows, const cplx_t<T> *__restrict__ tw, T scale, T im_scale,
+                                                   T im_scale0)
 {
     pdl_entry();
     using V = cplx_t<T>;
@@ -229,7 +230,7 @@ __global__ void __launch_bounds__(1024) k_rows_inv(const cplx_t<T> *__restrict__
         if (grow < total_rows) {
             const V v = buf[rr * vstride + x + (x >> 3)];
             out1[grow * n + x] = v.x * scale;
-            if (out2) out2[grow * n + x] = v.y * im_scale;
+            if (out2) out2[grow * n + x] = v.y * (grow < n ? im_scale0 : im_scale);
         }
     }
 }
@@ -237,7 +238,8 @@ __global__ void __launch_bounds__(1024) k_rows_inv(const cplx_t<T> *__restrict__
 // ---------------------------------------------------------------------------
 template <typename T>
 static int ks_impl(const T *in1, const T *in2, long in_bstride, T *out1, T *out2, cplx_t<T> *work, int n, int batch,
-                   int op, const cplx_t<T> *filt, T out_scale, const uint64_t *seed, int r0, bool rotate, cudaStream_t s, T im_scale)
+                   int op, const cplx_t<T> *filt, T out_scale, const uint64_t *seed, int r0, bool rotate, cudaStream_t s, T im_scale,
+                   T im_scale0)
 {
     using V = cplx_t<T>;
     int st = FM_OK;
@@ -276,13 +278,13 @@ static int ks_impl(const T *in1, const T *in2, long in_bstride, T *out1, T *out2
     if (op == FFT_OP_SPECTRUM) return FM_OK;
     const T scale = out_scale / ((T)n * (T)n);
     FM_LAUNCH(FM_K_FFT_ROWS_INV, kri, row_grid, row_threads, row_smem, s, work, out1, out2, n, logn, lognvec,
-              total_rows, tw, scale, scale * im_scale);
+              total_rows, tw, scale, scale * im_scale, scale * im_scale0);
     return FM_OK;
 }
 
 int launch_fft_op(const void *in1, const void *in2, long in_bstride, void *out1, void *out2, void *work, int n,
                   int batch, int precision, int op, const void *filt, double out_scale, const uint64_t *rot_seed, int rot_r0,
-                  bool rotate, cudaStream_t s, bool real_ok, double im_scale)
+                  bool rotate, cudaStream_t s, bool real_ok, double im_scale, double im_scale0)
 {
     if (precision == FM_F64 && n >= 64 && n <= 2048) {  // register-resident radix-8 path (fft64.cu)
         int st = FM_OK;
@@ -294,12 +296,12 @@ int launch_fft_op(const void *in1, const void *in2, long in_bstride, void *out1,
             return st;
         return launch_fft64((const double *)in1, (const double *)in2, in_bstride, (double *)out1, (double *)out2,
                             (double2 *)work, n, batch, op, (const double2 *)filt, out_scale, rot_seed, rot_r0, rotate,
-                            tw, tw2, s, im_scale);
+                            tw, tw2, s, im_scale, im_scale0);
     }
     if (precision == FM_F64)
         return ks_impl<double>((const double *)in1, (const double *)in2, in_bstride, (double *)out1, (double *)out2,
                                (double2 *)work, n, batch, op, (const double2 *)filt, out_scale, rot_seed, rot_r0,
-                               rotate, s, im_scale);
+                               rotate, s, im_scale, im_scale0);
     if (n >= 32) {  // register-resident radix-32 path (fft32.cu)
         int st = FM_OK;
         const float2 *tw = static_cast<const float2 *>(twiddles(n, FM_F32, s, &st));
@@ -310,11 +312,11 @@ int launch_fft_op(const void *in1, const void *in2, long in_bstride, void *out1,
             return st;
         return launch_fft32((const float *)in1, (const float *)in2, in_bstride, (float *)out1, (float *)out2,
                             (float2 *)work, n, batch, op, (const float2 *)filt, (float)out_scale, rot_seed, rot_r0,
-                            rotate, tw, tw2, s, (float)im_scale);
+                            rotate, tw, tw2, s, (float)im_scale, (float)im_scale0);
     }
     return ks_impl<float>((const float *)in1, (const float *)in2, in_bstride, (float *)out1, (float *)out2,
                           (float2 *)work, n, batch, op, (const float2 *)filt, (float)out_scale, rot_seed, rot_r0,
-                          rotate, s, (float)im_scale);
+                          rotate, s, (float)im_scale, (float)im_scale0);
 }
 
 int launch_ks(const void *in1, const void *in2, long in_bstride, void *out1, void *out2, void *work, int n, int batch,

@@ -200,7 +200,7 @@ template <int LOGN, bool WITH_B>
 __global__ void __launch_bounds__(Plan32<LOGN>::ROW_T, Plan32<LOGN>::ROW_MINB)
     k_rows_inv32(const float2 *__restrict__ work, float *__restrict__ out1,
                                                        float *__restrict__ out2, long total_rows,
-                                                       const float2 *__restrict__ tw, float scale, float im_scale,
+                                                       const float2 *__restrict__ tw, float scale, float im_scale, float im_scale0,
                                                        const __grid_constant__ CUtensorMap mw, int use_tma)
 {
     using P = Plan32<LOGN>;
@@ -239,12 +239,13 @@ __global__ void __launch_bounds__(Plan32<LOGN>::ROW_T, Plan32<LOGN>::ROW_MINB)
     }
     fft_vec<LOGN, 1, true>(v, sm, 0, j, tw);
     if (live) {
+        [[maybe_unused]] const float ims = row < P::N ? im_scale0 : im_scale;
 #pragma unroll
         for (int q = 0; q < P::E; ++q) {
                 const long pos = row * P::N + j + q * P::TV;
                 const float2 x = v[q];
                 out1[pos] = x.x * scale;
-                if constexpr (WITH_B) out2[pos] = x.y * im_scale;
+                if constexpr (WITH_B) out2[pos] = x.y * ims;
             }
     }
 }
@@ -667,7 +668,7 @@ static int ks32_real_impl(const float *in1, const float *in2, long in_bs, float 
 template <int LOGN>
 static int ks32_impl(const float *in1, const float *in2, long in_bs, float *out1, float *out2, float2 *work, int batch,
                      int op, const float2 *filt, float out_scale, const uint64_t *seed, int r0, bool rotate,
-                     const float2 *tw, const float2 *tw2, cudaStream_t s, float im_scale)
+                     const float2 *tw, const float2 *tw2, cudaStream_t s, float im_scale, float im_scale0)
 {
     if constexpr (LOGN >= 6) {
         if (op == FFT_OP_KS_INV && !out2 && tw2 && (reinterpret_cast<uintptr_t>(out1) & 15) == 0)
@@ -742,7 +743,7 @@ static int ks32_impl(const float *in1, const float *in2, long in_bs, float *out1
     const float gain = op == FFT_OP_FILTER ? 1.f : kFft32Gain;
     const float scale = out_scale * gain / ((float)P::N * (float)P::N);
     FM_LAUNCH(FM_K_FFT_ROWS_INV, kri, row_grid, RPC * P::TV, row_smem, s, work, out1, out2, total_rows, tw, scale,
-              scale * im_scale, mw, tma_out);
+              scale * im_scale, scale * im_scale0, mw, tma_out);
     return FM_OK;
 }
 
@@ -750,10 +751,10 @@ static int ks32_impl(const float *in1, const float *in2, long in_bs, float *out1
 // which then uses the generic shared-memory Stockham kernels.
 int launch_fft32(const float *in1, const float *in2, long in_bs, float *out1, float *out2, float2 *work, int n,
                  int batch, int op, const float2 *filt, float out_scale, const uint64_t *seed, int r0, bool rotate,
-                 const float2 *tw, const float2 *tw2, cudaStream_t s, float im_scale)
+                 const float2 *tw, const float2 *tw2, cudaStream_t s, float im_scale, float im_scale0)
 {
 #define FM_KS32(L) \
-    ks32_impl<L>(in1, in2, in_bs, out1, out2, work, batch, op, filt, out_scale, seed, r0, rotate, tw, tw2, s, im_scale)
+    ks32_impl<L>(in1, in2, in_bs, out1, out2, work, batch, op, filt, out_scale, seed, r0, rotate, tw, tw2, s, im_scale, im_scale0)
     switch (n) {
     case 32: return FM_KS32(5);
     case 64: return FM_KS32(6);

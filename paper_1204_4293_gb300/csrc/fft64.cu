@@ -181,7 +181,8 @@ __global__ void __launch_bounds__(Plan64<LOGN>::ROW_T)
 template <int LOGN, bool WITH_B>
 __global__ void __launch_bounds__(Plan64<LOGN>::ROW_T)
     k_rows_inv64(const double2 *__restrict__ work, double *__restrict__ out1, double *__restrict__ out2,
-                 long total_rows, const double2 *__restrict__ tw, double scale, double im_scale)
+                 long total_rows, const double2 *__restrict__ tw, double scale, double im_scale,
+                 double im_scale0)
 {
     pdl_wait();
     using P = Plan64<LOGN>;
@@ -194,11 +195,12 @@ __global__ void __launch_bounds__(Plan64<LOGN>::ROW_T)
     for (int r = 0; r < 8; ++r) v[r] = live ? work[row * P::N + j + r * P::TV] : make_double2(0.0, 0.0);
     fft_vec<LOGN, 1, true>(v, smd + vr * P::VS, 0, j, tw);
     if (!live) return;
+    [[maybe_unused]] const double ims = row < P::N ? im_scale0 : im_scale;
 #pragma unroll
     for (int q = 0; q < 8; ++q) {
         const long pos = row * P::N + j + q * P::TV;
         out1[pos] = v[q].x * scale;
-        if constexpr (WITH_B) out2[pos] = v[q].y * im_scale;
+        if constexpr (WITH_B) out2[pos] = v[q].y * ims;
     }
 }
 
@@ -358,7 +360,7 @@ __global__ void __launch_bounds__(Plan64<LOGN - 1>::ROW_T)
 template <int LOGN>
 static int impl64(const double *in1, const double *in2, long in_bs, double *out1, double *out2, double2 *work, int batch,
            int op, const double2 *filt, double out_scale, const uint64_t *seed, int r0, bool rotate, const double2 *tw,
-           const double2 *tw2, cudaStream_t s, double im_scale)
+           const double2 *tw2, cudaStream_t s, double im_scale, double im_scale0)
 {
     using P = Plan64<LOGN>;
     using P2 = Plan64<LOGN - 1>;
@@ -394,15 +396,15 @@ static int impl64(const double *in1, const double *in2, long in_bs, double *out1
               filt);
     if (op == FFT_OP_SPECTRUM) return FM_OK;
     FM_LAUNCH(FM_K_FFT_ROWS_INV, ki, row_grid, P::ROW_T, row_smem, s, (const double2 *)work, out1, out2, rows, tw,
-              scale, scale * im_scale);
+              scale, scale * im_scale, scale * im_scale0);
     return FM_OK;
 }
 
 int launch_fft64(const double *in1, const double *in2, long in_bs, double *out1, double *out2, double2 *work, int n,
                  int batch, int op, const double2 *filt, double out_scale, const uint64_t *seed, int r0, bool rotate,
-                 const double2 *tw, const double2 *tw2, cudaStream_t s, double im_scale)
+                 const double2 *tw, const double2 *tw2, cudaStream_t s, double im_scale, double im_scale0)
 {
-#define FM_FFT64(L) impl64<L>(in1, in2, in_bs, out1, out2, work, batch, op, filt, out_scale, seed, r0, rotate, tw, tw2, s, im_scale)
+#define FM_FFT64(L) impl64<L>(in1, in2, in_bs, out1, out2, work, batch, op, filt, out_scale, seed, r0, rotate, tw, tw2, s, im_scale, im_scale0)
     switch (n) {
     case 64: return FM_FFT64(6);
     case 128: return FM_FFT64(7);

@@ -312,20 +312,20 @@ int launch_noise_finalize(const void *acc, const void *wdata, double *var, void 
 }
 
 // ---- exact expected variance (periodic boundary) ----------------------------
-// out[c][p] = (a[c][p]^2 + b[c][p]^2) f, f = 1 for c < h and f0 (a power of
-// two) from h on: |K_j|^2 from the two delta responses (the second half of the
-// bands scaled up to the first's magnitude), |gamma|^2 from the shear.
+// out[c][p] = (a[c][p]^2 + b[c][p]^2) f, f = 1 for c < h, fh for c = h and f0
+// above (powers of two): |K_j|^2 from the two delta responses (the second half
+// of the bands scaled up to the first's magnitude), |gamma|^2 from the shear.
 // VW elements a thread; grid = (blocks, count).
 template <typename T, int VW>
 __global__ void __launch_bounds__(256) k_modulus2(const T *__restrict__ a, long a_bs, const T *__restrict__ b,
-                                                  long b_bs, T *__restrict__ out, long nn, int h, T f0)
+                                                  long b_bs, T *__restrict__ out, long nn, int h, T fh, T f0)
 {
     pdl_entry();
     struct alignas(VW * sizeof(T)) Vec {
         T e[VW];
     };
     const int c = blockIdx.y;
-    const T f = c < h ? (T)1 : f0;
+    const T f = c < h ? (T)1 : c == h ? fh : f0;
     a += c * a_bs;
     b += c * b_bs;
     out += c * nn;
@@ -349,30 +349,30 @@ template <typename T> __global__ void k_unit_shears(T *g1d, T *g2d, long nn)
 }
 
 template <typename T, int VW>
-static int modulus2_impl(const T *a, long a_bs, const T *b, long b_bs, T *out, long nn, int count, int h, T f0,
+static int modulus2_impl(const T *a, long a_bs, const T *b, long b_bs, T *out, long nn, int count, int h, T fh, T f0,
                          cudaStream_t s)
 {
     long g = (nn / VW + 255) / 256;
     if (g > 152L * 8) g = 152L * 8;
-    FM_LAUNCH(0, (k_modulus2<T, VW>), dim3((unsigned)g, count), 256, 0, s, a, a_bs, b, b_bs, out, nn, h, f0);
+    FM_LAUNCH(0, (k_modulus2<T, VW>), dim3((unsigned)g, count), 256, 0, s, a, a_bs, b, b_bs, out, nn, h, fh, f0);
     return FM_OK;
 }
 
 int launch_modulus2(const void *a, long a_bs, const void *b, long b_bs, void *out, long nn, int count, int h,
-                    double f0, int precision, cudaStream_t s)
+                    double fh, double f0, int precision, cudaStream_t s)
 {
     // 16-byte accesses (nn is a multiple of 16); the caller's shear may be aligned to its element only
     const bool al = ((reinterpret_cast<uintptr_t>(a) | reinterpret_cast<uintptr_t>(b)) & 15) == 0;
     if (precision == FM_F64) {
         const double *p = static_cast<const double *>(a), *q = static_cast<const double *>(b);
         double *o = static_cast<double *>(out);
-        return al ? modulus2_impl<double, 2>(p, a_bs, q, b_bs, o, nn, count, h, f0, s)
-                  : modulus2_impl<double, 1>(p, a_bs, q, b_bs, o, nn, count, h, f0, s);
+        return al ? modulus2_impl<double, 2>(p, a_bs, q, b_bs, o, nn, count, h, fh, f0, s)
+                  : modulus2_impl<double, 1>(p, a_bs, q, b_bs, o, nn, count, h, fh, f0, s);
     }
     const float *p = static_cast<const float *>(a), *q = static_cast<const float *>(b);
     float *o = static_cast<float *>(out);
-    return al ? modulus2_impl<float, 4>(p, a_bs, q, b_bs, o, nn, count, h, (float)f0, s)
-              : modulus2_impl<float, 1>(p, a_bs, q, b_bs, o, nn, count, h, (float)f0, s);
+    return al ? modulus2_impl<float, 4>(p, a_bs, q, b_bs, o, nn, count, h, (float)fh, (float)f0, s)
+              : modulus2_impl<float, 1>(p, a_bs, q, b_bs, o, nn, count, h, (float)fh, (float)f0, s);
 }
 
 int launch_unit_shears(void *g1d, void *g2d, long nn, int precision, cudaStream_t s)

@@ -22,3 +22,10 @@ def _errors(n, J):
 def test_error_over_all_bands(n, J):
     d, ref = _errors(n, J)
     assert (d.pow(2).mean() / ref.pow(2).mean()).sqrt().item() <= BOUND
+
+
+@pytest.mark.parametrize("n,J", [(64, 4), (256, 6), (512, 7), (1024, 7), (1024, 4), (256, 3)])
+def test_error_of_each_band(n, J):
+    d, ref = _errors(n, J)
+    rel = d.pow(2).mean(dim=(-1, -2)).sqrt() / ref.mean(dim=(-1, -2))
+    assert rel.max().item() <= BOUND, rel.tolist()
