@@ -113,7 +113,9 @@ int fm_ks_forward(const void *kappa, void *g1, void *g2, int n, int batch, const
  * Scale j filters rows then columns with h = [1,4,6,4,1]/16 at spacing
  * 2^(j-1) (the B3 two-scale filter) and stores w_j = c_{j-1} - c_j.
  * n need not be a power of two here (n >= 2^J).  kappa and pyramid must not
- * overlap.  Scratch: up to 2*batch*n*n elements. */
+ * overlap.  Finite for values up to half the type's largest one in fp64 and in
+ * the plain fp32 form (fuse_depth -1), up to 1/256 of it in the other fp32 forms.
+ * Scratch: up to 2*batch*n*n elements. */
 int fm_starlet_forward(const void *kappa, void *pyramid, int n, int J, int batch, const fm_config *cfg,
                        void *stream);
 
@@ -258,7 +260,7 @@ int fm_ks_invert_noalloc(const void *g1, const void *g2, void *kappa_E, void *ka
  * For every map b and pyramid array j of pyramid [batch][J][n][n] (any n),
  * moments[(b*J + j)*4 + 0..3] = mean, variance <M_ap^2> (over the n^2
  * pixels, divided by n^2), skewness and excess kurtosis.  Two passes; fp32
- * partial sums of at most ~16 pixels per thread, FP64 across threads. */
+ * sums of at most 16 pixels, added with more than the bits of an FP64 sum. */
 int fm_band_moments(const void *pyramid, double *moments, int n, int J, int batch, const fm_config *cfg,
                     void *stream);
 
@@ -363,7 +365,9 @@ int fm_device_error(void);
  *                        16-byte aligned), 0 = the complex inverse and its
  *                        real part; default: the real output from
  *                        n = 512 up, in fm_ks_invert and in the batched
- *                        pipeline's chunks (where it measured faster)
+ *                        pipeline's chunks (where it measured faster); fp64
+ *                        maps of 64^2 to 2048^2 with kappa_E 16-byte aligned
+ *                        take the real output unless the value is 0
  *   FM_TUNE_SERVE_MERGE  servers: most maps that one merged run of queued
  *                        pyramid-only requests (R = 0, n <= 1024) of one
  *                        shape may hold (default 16; 1 = every request runs
@@ -390,9 +394,9 @@ int fm_tune(int knob, int64_t value);
  * fm_autotune times fm_map_starlet on `batch` synthetic n x n maps (J scales,
  * cfg->precision and cfg->boundary; cfg's fuse_depth and large_path are
  * ignored) for candidate plans, by coordinate descent from the built-in rules
- * over: fused depth 1..4 (fp64 1..3, at most J - 1), large-scale path 1 or 3,
- * fp32 tile kernel form (1 = register window, 0 = shared buffer) and chunk
- * budget 40 / 60 / 80 / 120 MiB; a candidate replaces the best so far only
+ * over: fused depth 1..4 (fp64 1..3, at most J - 1), large-scale path 1, 3 or
+ * 4, fp32 tile kernel form (1 = register window, 0 = shared buffer) and chunk
+ * budget 24 / 36 / 48 / 64 / 96 MiB; a candidate replaces the best so far only
  * when 1 % faster.  A batch that runs in one kernel (few fp32 maps of 64^2,
  * 128^2 or 256^2) has no candidates beside the built-in plan and keeps that
  * form whatever the table says.  The winner goes into a process-wide table keyed by

@@ -266,16 +266,17 @@ int fm_noise_finalize(const double *sums, const void *pyramid, double *var_out, 
 // Var_j = 1/2 |K_j|^2 (*) |gamma|^2 (circular convolution).  K_j is the
 // pipeline's response to unit shears at pixel 0 (Re K_j from gamma1, -Im K_j
 // from gamma2); the convolutions run through the FFT pipeline, two bands at a
-// time: the spectrum of |gamma|^2 once, then rows FFT of |K_j|^2 + i |K_j+h|^2
-// -> columns FFT -> times that spectrum -> inverse, whose real and imaginary
-// parts are the bands j and j + h (|gamma|^2 is real).  Band j + h enters
-// times a power of two that brings it to band j's magnitude, so that its
-// rounding is relative to itself: 4^pairs, as a band's response power falls by
-// 4.0 to 5.5 a scale, and for band 0's partner, as band 0 has 20 times the power
-// of band 1, that times 8 (4 for one pair).  With 4^pairs alone the partner's
-// error was 2.5 times the other bands' (rms of its mean, 256^2 .. 2048^2 3.3 ..
-// 4.0e-7, now 1.3 .. 1.8e-7).  One spectrum and (J - 1) / 2 filter passes instead of J - 1
-// of each: 1024^2, J = 7 214 -> 158 us.
+// time: the spectrum of |gamma|^2 once, then rows FFT of |K_j|^2 + i |K_j+p|^2
+// (p = pairs, half the bands rounded up) -> columns FFT -> times that spectrum
+// -> inverse, whose real and imaginary parts are the bands j and j + p
+// (|gamma|^2 is real).  Band j + p enters times a power of two that brings it to
+// band j's magnitude, so that its rounding is relative to itself: 4^p, as a
+// band's response power falls by 4.0 to 5.5 a scale, and for band 0's partner,
+// as band 0 has 20 times the power of band 1, that times 8 (4 for p = 1).  With
+// 4^p alone the partner's error was 2.5 times the other bands' (rms of its
+// mean, 256^2 .. 2048^2 3.3 .. 4.0e-7, now 1.3 .. 1.8e-7).  One spectrum and
+// (J - 1) / 2 filter passes instead of J - 1 of each: 1024^2, J = 7 214 -> 158 us
+// (145 with the later steps).
 int fm_map_noise_expected(const void *g1, const void *g2, void *var_out, int n, int J, const fm_config *cfgp,
                           void *stream)
 {

@@ -68,10 +68,16 @@ __device__ __forceinline__ void pdl_wait()
 // CTAs an SM, as a chunk's kernels have, they fill its tail.  Behind a grid of
 // about one CTA an SM they crowd onto the SMs that happen to have room and stay
 // there, and the next kernel runs unevenly.  With the early trigger everywhere
-// / nowhere (us): one 256^2 map 27 / 30, one 1024^2 map 54.7 / 42.9, 32 maps of
-// 1024^2 (chunks of 4 on two streams) 538 / 541, one 8192^2 map (4096 CTAs and
-// more) 1896 / 1877.  The fp64 kernels, whose SMs are busy with few warps, never
-// trigger early (one 1024^2 map 614 / 420).
+// / by this rule / nowhere (us): one 256^2 map in separate kernels 27 / - / 30,
+// maps of 512^2 one 32.0 / 32.1 / 32.7, four 47.7 / 38.4 / 38.1, 64 in chunks
+// on two streams 265 / 266 / 268; 1024^2 one 49.0 / 40.4 / 40.2, four 91.9 /
+// 91.5 / 88.8, 32 530 / 531 / 542; 2048^2 one 112.2 / 112.3 / 111.6, eight 622 /
+// 625 / 634; 4096^2 one 458 / 460 / 460, four 1626 / 1630 / 1625; one 8192^2 map
+// 1898 / 1886 / 1885; noise R = 100 512^2 604 / 593 / 580, 1024^2 2296 / 2285 /
+// 2268; expected variance 1024^2 143 / 134 / 126.  What the upper window gives,
+// the two-stream batches, it takes from single streams of medium grids.  The
+// fp64 kernels, whose SMs are busy with few warps, never trigger early (one
+// 1024^2 map 614 / 420).
 __device__ __forceinline__ void pdl_entry()
 {
 #if defined(__CUDA_ARCH__) && __CUDA_ARCH__ >= 900

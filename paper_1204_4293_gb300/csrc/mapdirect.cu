@@ -12,7 +12,8 @@
 // y - dy enter together: with s = gamma1(y + dy) + gamma1(y - dy) and
 // d = gamma2(y + dy) - gamma2(y - dy),
 //   M(x, y) = sum_{dy >= 0} sum_dx A(dx, dy) s(x + dx) + B(dx, dy) d(x + dx),
-// half the multiplications of the plain sum.
+// half the multiplications of the plain sum (a pair's sum has to stay in the
+// type's range: pixels below half its largest value).
 //
 // Kernel layout: one warp owns one output row of 32 CX columns (CX adjacent
 // ones a lane) and shares nothing with the others.  For each dy it forms the
@@ -28,7 +29,7 @@
 //
 // What bounds it: the FP32 pipe and the shared-memory loads together (1024^2,
 // R = 32: 52.7 M warp FMAs of two lanes, 84 us at two a cycle and SM; ncu: FMA
-// pipe 56 %, shared-memory and L1 data path 69 %, 20 warps an SM).  One 1024^2
+// pipe 58 %, shared-memory and L1 data path 77 %, 19 warps an SM).  One 1024^2
 // map, starlet Q theta = 16 (R = 32): 372 -> 199 us; S98 theta = 64 1246 ->
 // 618, masked 3050 -> 825; masked 2 x 1000^2 S98 theta = 16 445 -> 236; fp64
 // 512^2 S98 theta = 16 3079 -> 472 (the plain sum over all rows, with a CTA's

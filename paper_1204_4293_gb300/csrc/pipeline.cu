@@ -15,11 +15,12 @@ namespace fm {
 
 // ---- KS + starlet over a batch, in L2-sized chunks ---------------------------------
 // A chunk of C maps runs KS then the starlet before the next chunk starts, so
-// its intermediates (FFT work buffer, kappa, starlet scratch: ~20 B/px fp32)
+// its intermediates (FFT work buffer, kappa, starlet scratch: ~12 B/px fp32)
 // stay in L2 and only the shear and the pyramid cross HBM.  Chunks alternate
 // over the internal streams (two by default, one scratch slot each) so one
-// chunk's kernels overlap the next one's.  Batches of more than one chunk are
-// recorded once into a CUDA graph per (pointers, sizes, config) and replayed.
+// chunk's kernels overlap the next one's.  A batch of more than one chunk is
+// launched at its first call and recorded into a CUDA graph, one per (pointers,
+// sizes, config), when the same call comes back (seen_before).
 namespace {
 
 constexpr int kMaxChunkStreams = 4;

@@ -13,10 +13,11 @@
 //   rows gathered from the CTAs that own them; band out, c_j kept.
 // The arithmetic is that of fft32.cu's complex form and of starlet.cu, operation
 // by operation, so the results are bit-identical to theirs.  What bounds it is
-// the chain of J + 3 cluster barriers (about 1 us each) with little work
-// between: KS + starlet of one map, J = 5 / 6 / 6, 64^2 33 -> 19 us a call, 128^2 34
-// -> 18, 256^2 34 -> 23 (the kernel itself 14, 17 and 24; with 32 rows a CTA 15,
-// 20 and 33).
+// the chain of J + 2 cluster barriers (two in Kaiser-Squires, one a scale, one at
+// the end; about 1 us each) with little work between: KS + starlet of one map,
+// J = 5 / 6 / 6, in a queue of calls, 64^2 33 -> 13 us a call, 128^2 34 -> 16,
+// 256^2 34 -> 23 (replayed from a graph, the GPU alone, 12.0, 15.5 and 21.8; with
+// 32 rows a CTA the kernel took 1.1, 1.2 and 1.4 times as long).
 #include <cooperative_groups.h>
 
 #include <atomic>

@@ -14,7 +14,8 @@
 //   st_tile32 / st_tile : the same scales with a row-filtered shared buffer
 //             (fp32 alternative behind a tuning knob / fp64 and generic).
 //   st_scale : (fp32, n a multiple of 4, spacing 4..128 px) one large scale in
-//             one pass, its window rows staged by bulk copies or 16-byte loads.
+//             one pass, its window rows staged by bulk copies (where the driver
+//             refuses a tensor map the row and the column pass run instead).
 //   st_scale64 : (fp64, n a multiple of 2) one scale in one pass.
 //   st_colrow : columns of scale j and rows of scale j + 1 in one kernel.
 //   st_row  : r = rows-filtered c_{j-1} for one (large) scale.
@@ -871,10 +872,10 @@ __global__ void __launch_bounds__(NT) k_st_scale(const float *c_prev, float *c_n
 // SM): 4 operations a filter (taps 1, 4, 6, 4, 1), 1.25 row filters and one
 // column filter a pixel, one difference; the scaling by 1 / 256 works on the
 // exponent field.  A tile of three fused scales computes its halo again (2.39 M
-// FP64 warp instructions for 1024^2 against 1.0 M), and a row and a column pass
+// FP64 warp instructions for 1024^2 against 1.08 M), and a row and a column pass
 // read and write the row-filtered map.  No shared memory and one-warp CTAs, so
 // that the few hundred of a single map spread evenly.  One 1024^2 map, J = 7: the
-// starlet 257 -> 164 us (fused tile of three scales 158, a large scale 32, now
+// starlet 257 -> 165 us (fused tile of three scales 158, a large scale 32, now
 // 30 each).
 __device__ __forceinline__ double tap5(double a, double b, double c, double d, double e)
 {
@@ -1259,7 +1260,8 @@ static int auto_fuse(int n, int J, const fm_config &cfg)
 
 // Large-scale path when cfg.large_path = 0: the autotuned plan's, else one
 // pass per scale (k_st_scale) after two or more fused scales on sides that are
-// multiples of 4 (fp32 only, fp64 takes the form 1), else the column pass
+// multiples of 4 (fp32; in fp64 the built-in form is k_st_scale64 for every
+// scale, and this names the path beside a tile), else the column pass
 // fused with the next row pass on small maps, else one row and one column pass
 // per scale.  The three forms 1 / 3 / 4, starlet alone (us): 256 x 128^2 J = 5
 // 113 / 94 / 50, 1 x 256^2 J = 6 27 / 22 / 18, 128 x 256^2 184 / 163 / 81,

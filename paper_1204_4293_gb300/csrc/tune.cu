@@ -156,8 +156,8 @@ int fm_autotune(int n, int J, int batch, const fm_config *cfgp, fm_plan *best)
         fm_trim();
     };
     // time one plan: enter it in the table, drop graphs recorded with the old
-    // one, run twice (the first call records the batched graph), then time
-    // enough calls for ~20 ms of work
+    // one, run twice (the batched graph is recorded by the second call at the
+    // latest), then time enough calls for ~20 ms of work
     auto time_plan = [&](const TunedPlan &p, double *ms) -> int {
         table_put(n, J, cfg.precision, p);
         fm_trim();
