@@ -148,7 +148,9 @@ int fm_map_starlet_host(const void *g1_host, const void *g2_host, void *pyramid_
  * gamma_t = -(gamma1 cos 2phi + gamma2 sin 2phi), phi the angle of d; pixels
  * outside the field add nothing.  R = cut_over_theta * theta_px, or the
  * filter's default cut when cut_over_theta <= 0.  ell is the S98 order.
- * One n x n map (n >= 1, any size).  Cost O(n^2 R^2). */
+ * One n x n map (n >= 1, any size).  Cost O(n^2 R^2).  Scratch: the weights
+ * and, where the rows alone do not fill the GPU, up to 256 MiB of partial sums
+ * (or one map's, if that is more; twice as much with pixel weights). */
 int fm_map_direct(const void *g1, const void *g2, void *map, int n, int filter, double theta_px, int ell,
                   double cut_over_theta, const fm_config *cfg, void *stream);
 
